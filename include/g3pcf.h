@@ -299,7 +299,10 @@ int g3pcf_fp32_peak(double* tflops, void* stream);
  *                             planned on the device instead)
  *   G3PCF_OPT_LIST_BYTES      device bytes for the pair lists (0: up to 40% of free
  *                             memory, at most 32 GB); more pairs than fit are
- *                             processed in several passes
+ *                             processed in several passes.  A plain forward's lists
+ *                             take 16 bytes per pair, or 4 where the budget would
+ *                             otherwise leave too few primaries per pass; the other
+ *                             calls' take 4
  *   G3PCF_OPT_GRAD_PRECISION  arithmetic of the pair stage for multipoles that are
  *                             differentiated (forwards with G3PCF_F_KEEP_ALM, the
  *                             backward and its recomputation): 0 = double-float

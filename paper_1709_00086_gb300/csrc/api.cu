@@ -72,6 +72,15 @@ double lfact(int k) { return std::lgamma((double)k + 1.0); }
 
 }  // namespace
 
+namespace {
+// Pair lists of one chunk of primaries: chunks of all and of the largest primary,
+// and whether they hold direction records.
+struct ListWarm {
+    int64_t total, most;
+    bool dirs;
+};
+}  // namespace
+
 struct g3pcf_plan_s {
     int nbins, lmax, los_mode;
     double rmin, rmax, box;
@@ -109,7 +118,7 @@ struct g3pcf_plan_s {
     DevBuf key_a, key_b, val_a, val_b, hist, hist_off, scan_tmp, pts, pts64, orig, cstart, plist;
     DevBuf small;       // status, queue
     DevBuf counts, A, partials, d_tiles, d_segs, d_segfirst, d_colmap, d_colscale, d_catoff;
-    DevBuf d_colconv, d_colcoef, d_bintab_s, d_slotconv, d_slotcoef, d_monoexp, d_monoconv, d_monoidx, d_monocoef;
+    DevBuf d_colconv, d_colcoef, d_slotconv, d_slotcoef, d_monoexp, d_monoconv, d_monoidx, d_monocoef;
     DevBuf d_ranges, d_tiles_tc, d_cats, d_mreal, d_V, d_bintab, wrow, d_vblk, d_strips_tc, d_items;
     DevBuf d_bop, d_bblk, d_bcat;
     DevBuf d_slotcoefdf, d_mrealdf, d_Vdf, d_colcoefdf;
@@ -135,9 +144,9 @@ struct g3pcf_plan_s {
     int* h_need = nullptr;
     int* h_base = nullptr;
     size_t h_list_cap = 0;
-    // graph capture of the list path: per A-chunk {total chunks, largest need} of
-    // the uncaptured warm-up run, consumed in order by the capture run
-    std::vector<std::pair<int64_t, int64_t>> gl_warm;
+    // graph capture of the list path: per A-chunk the list sizes of the uncaptured
+    // warm-up run, consumed in order by the capture run
+    std::vector<ListWarm> gl_warm;
     size_t gl_idx = 0;
     bool warm_for_graph = false;
     bool exact_alm = false;  // this forward runs with G3PCF_F_KEEP_ALM
@@ -151,7 +160,6 @@ struct g3pcf_plan_s {
     int cev_used = 0;
     bool last_chunked = false;
     std::vector<unsigned char> bintab;  // r^2 -> bin lookup (see compute_bins)
-    std::vector<signed char> bintab_s;  // signed form (pair-list scan)
     float bin_tscale = 0.f;
     // index state of the last forward (for the adjoint pair pass)
     bool last_plist = false;
@@ -250,10 +258,9 @@ int upload_consts(g3pcf_plan_t P) {
         return fail(G3PCF_ERR_ALLOC, "workspace allocation failed (constants)");
     CK(cudaMemcpy(P->d_strips_tc.p, P->strips_tc.data(), P->strips_tc.size() * sizeof(TcStrip),
                   cudaMemcpyHostToDevice));
-    if (P->d_bintab.ensure(P->bintab.size()) || P->d_bintab_s.ensure(P->bintab_s.size()))
+    if (P->d_bintab.ensure(P->bintab.size()))
         return fail(G3PCF_ERR_ALLOC, "workspace allocation failed (bin table)");
     CK(cudaMemcpy(P->d_bintab.p, P->bintab.data(), P->bintab.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(P->d_bintab_s.p, P->bintab_s.data(), P->bintab_s.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(P->d_colmap.p, P->colmap.data(), P->RL * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(P->d_colscale.p, P->colscale.data(), P->RL * sizeof(float), cudaMemcpyHostToDevice));
     if (P->d_colconv.ensure(P->colconv.size() * sizeof(int4)) ||
@@ -381,17 +388,19 @@ void compute_bins(g3pcf_plan_t P) {
                 break;
             }
     }
-    // Signed form for the pair-list scan: bin, -1 surely outside (also every
-    // cell from e_B^2 + g_B up, so the last entry takes all larger r^2), -3 check.
-    P->bintab_s.assign(T + 2, -3);
-    for (int t = 0; t < T + 2; ++t) {
-        const double lo = (t - 0.01) * D, hi = (t + 1.01) * D;
-        const unsigned char v = P->bintab[t];
-        if (v == 254 || lo > b.e2[B] + b.guard[B])
-            P->bintab_s[t] = -1;
-        else if (v < 254)
-            P->bintab_s[t] = (signed char)v;
+    // The pair-list scan rounds t = r invw + bin_c to the nearest integer.  It is
+    // the exact bin unless t lies within eps of a bin edge: eps covers the guard
+    // band of every edge (as a distance in r) and the FP32 error of t (rsqrt, two
+    // products, the rounded constants: below 8 ulp of the largest term).
+    double eps = 0.0;
+    for (int k = 0; k <= B; ++k) {
+        const double e = std::sqrt(b.e2[k]);
+        eps = std::max(eps, std::min(e > 0 ? b.guard[k] / e : HUGE_VAL, std::sqrt((double)b.guard[k])));
     }
+    const double w = (P->rmax - P->rmin) / B;
+    eps = eps / w + 8.0 * u * (2.0 * P->rmax / w + 1.0);
+    b.bin_c = (float)(-P->rmin / w - 0.5);
+    b.bin_lim = (float)(0.5 - eps);
 }
 
 // Column map of an A row: block m (m = 0: K_0 reals; m >= 1: Re and Im halves)
@@ -649,8 +658,6 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     la.counts = pa.counts;
     la.queue = pa.queue;
     la.status = pa.status;
-    la.bintab = P->d_bintab_s.as<signed char>();
-    la.bin_tscale = pa.bin_tscale;
     la.g = pa.g;
     la.bins = pa.bins;
     // multipoles that will be differentiated take the exact image separations and,
@@ -677,6 +684,10 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     la.qa = qa;
     la.qb = qb;
     la.ncand = reinterpret_cast<unsigned long long*>(pa.status + 24);  // zeroed with the status word
+    // plain forwards: the scan writes each pair's direction and weight (16 bytes)
+    // instead of its list entry (4 bytes), unless that leaves passes too small to
+    // fill the chip (below)
+    bool dirs = mode == 0 && !la.exact_img && P->opt_basis == 0;
     la.bop = nullptr;
     if (mode == 0 && pa.bop && !la.precise && P->opt_basis == 0 && !P->capturing) {
         la.bop = pa.bop;
@@ -691,11 +702,12 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         // the pool the warm-up run sized (sizes of that run, same A-chunk order)
         if (P->gl_idx >= P->gl_warm.size())
             return fail(G3PCF_ERR_STATE, "graph capture without a matching warm-up forward");
-        const std::pair<int64_t, int64_t> wm = P->gl_warm[P->gl_idx++];
-        const int64_t C = (int64_t)(P->l_pool.bytes / 128);
+        const ListWarm wm = P->gl_warm[P->gl_idx++];
+        dirs = wm.dirs;
+        const int64_t C = (int64_t)(P->l_pool.bytes / (dirs ? 512 : 128));
         int64_t slack = 0, stride = 0;
         int npass = 0;
-        graph_plan_sizes(C, wm.first, wm.second, P->nbins, slack, stride, npass);
+        graph_plan_sizes(C, wm.total, wm.most, P->nbins, slack, stride, npass);
         if (stride < 1 || (int64_t)P->l_tag.bytes / 4 < C || (int64_t)P->l_ord.bytes / 4 < C ||
             P->l_gbase.bytes < 8 * (size_t)nq || P->l_passq.bytes < 4 * (size_t)(npass + 1) ||
             P->l_scantmp.bytes < plan_scan_tmp_bytes(nq) || (int)P->lev.size() < P->lev_used + 4 * npass) {
@@ -705,6 +717,7 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
             return G3PCF_OK;
         }
         la.chunks = P->l_pool.as<int>();
+        la.dirs = dirs ? P->l_pool.as<float4>() : nullptr;
         la.tag = P->l_tag.as<int>();
         la.ord = P->l_ord.as<int>();
         ++P->launches;
@@ -759,20 +772,33 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         budget = 0.4 * (double)(fr + P->l_pool.bytes + P->l_tag.bytes + P->l_ord.bytes);
         if (budget > 32e9) budget = 32e9;
     }
-    int64_t cap = (int64_t)(budget / 136.0);
+    // Direction records (520 bytes per chunk against 136) make more and smaller
+    // passes.  Below about 28 primaries per SM and pass, list entries are faster: on
+    // the 2M-point workload 563 ms (records) against 586 ms (entries) at 4,200
+    // primaries per pass of records, 672 against 623 ms at 2,100.
+    const double drecs = budget / 520.0;
+    dirs = dirs && drecs >= (double)most &&
+           (drecs >= (double)total || drecs * (double)nq >= 28.0 * P->nsm * (double)total);
+    const size_t chunk_bytes = dirs ? 512 : 128;
+    // a third of the records (4 GB at least) per pass: a first call pays about
+    // 0.14 ms per GB of pool, every call about 0.27 ms per further pass
+    if (dirs && P->opt_list_bytes <= 0 && !P->warm_for_graph)
+        budget = std::min(budget, std::max(4e9, 520.0 * ((double)total / 3.0 + (double)most)));
+    int64_t cap = (int64_t)(budget / (double)(chunk_bytes + 8));
     if (cap > ((int64_t)1 << 30)) cap = (int64_t)1 << 30;
-    P->gl_warm.emplace_back(total, most);
+    P->gl_warm.push_back(ListWarm{total, most, dirs});
     // a warm-up for a graph capture keeps headroom for the device-planned passes
     const int64_t want = P->warm_for_graph ? total + total / 4 + 2 * most + P->nbins + 64 : total;
     if (cap > want) cap = want;
     if (cap < most)
         return fail(G3PCF_ERR_ALLOC, "pair lists of one primary (%lld chunks) exceed the list budget (%lld)",
                     (long long)most, (long long)cap);
-    if (cap > 0 && (ensure(P, P->l_pool, 128 * (size_t)cap, "pair lists") ||
+    if (cap > 0 && (ensure(P, P->l_pool, chunk_bytes * (size_t)cap, "pair lists") ||
                     ensure(P, P->l_tag, 4 * (size_t)cap, "pair lists") ||
                     ensure(P, P->l_ord, 4 * (size_t)cap, "pair lists")))
         return G3PCF_ERR_ALLOC;
     la.chunks = P->l_pool.as<int>();
+    la.dirs = dirs ? P->l_pool.as<float4>() : nullptr;
     la.tag = P->l_tag.as<int>();
     la.ord = P->l_ord.as<int>();
     if (P->warm_for_graph && cap > 0) {  // what the capture run will need (no allocation while capturing)
@@ -1983,7 +2009,7 @@ int g3pcf_destroy(g3pcf_plan_t P) {
     DevBuf* bufs[] = {&P->key_a, &P->key_b, &P->val_a, &P->val_b, &P->hist, &P->hist_off,
                       &P->scan_tmp, &P->pts, &P->pts64, &P->orig, &P->cstart, &P->plist,
                       &P->small, &P->counts, &P->A, &P->partials, &P->d_tiles, &P->d_segs,
-                      &P->d_segfirst, &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_colcoef, &P->d_bintab_s, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
+                      &P->d_segfirst, &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_colcoef, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
                       &P->d_tiles_tc, &P->d_cats, &P->d_mreal, &P->d_V, &P->d_bintab, &P->d_vblk,
                       &P->d_strips_tc, &P->d_items,
                       &P->d_slotcoefdf, &P->d_mrealdf, &P->d_Vdf, &P->d_colcoefdf,

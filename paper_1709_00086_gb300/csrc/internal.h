@@ -56,6 +56,8 @@ struct Bins {
     float hi_rej;     // r2 above this: surely >= e_B
     float slack;      // conservative slack for cell pruning
     float rmaxf;
+    float bin_c;      // -rmin invw - 1/2: round(r invw + bin_c) is the bin of r (k_scan)
+    float bin_lim;    // ... surely, within this distance of the bin's centre (in widths)
     double e2[kMaxBins + 1];
     float e2f[kMaxBins + 1];
     float guard[kMaxBins + 1];
@@ -177,8 +179,6 @@ struct ListArgs {
     unsigned long long* counts;
     int* queue;
     int* status;
-    const signed char* bintab;  // G3_BIN_TABLE + 2: bin, -1 no pair, -3 decide per pair
-    float bin_tscale;
     int* need;               // [q] (global processing-order index)
     unsigned long long* ncand;  // candidates visited (k_count adds)
     const int* base;         // [q] first chunk of q, relative to the pool arrays
@@ -217,7 +217,8 @@ struct ListArgs {
     int nblk;
     const int4* bcat;
     int skip_a;
-    int* chunks;             // pool: 32 ints per chunk
+    int* chunks;             // pool: 32 ints per chunk (list entries)
+    float4* dirs;            // or, for k_accum_dir (then non-null): 32 direction records per chunk
     int* tag;                // pool: (rank among its bin's chunks) << 5 | bin, per chunk
     int* ord;                // pool: the primary's chunks listed by bin (stable), chunk | bin << 26
     Grid g;

@@ -137,9 +137,7 @@ __device__ __forceinline__ void accum_pair_cheb(float (&acc0)[L + 1], float2 (&a
                 accc[b + k] = __ffma2_rn(make_float2(T[k], T[k]), c, accc[b + k]);
             });
             if constexpr (m + 2 <= L) {
-                const float t = fmaf(c.x, u2x, -c.y * u2y);
-                c.y = fmaf(c.x, u2y, c.y * u2x);
-                c.x = t;
+                c = __ffma2_rn(make_float2(c.x, c.x), make_float2(u2x, u2y), __fmul2_rn(make_float2(c.y, c.y), make_float2(-u2y, u2x)));
             }
         });
     }
@@ -382,15 +380,8 @@ __device__ __forceinline__ int decide_bin(float r2, float hi_rej, float lo_rej, 
     return bin;
 }
 
-// decide_bin split for warp-wide use: bin_fast settles almost every
-// candidate with one lookup in the signed r^2 table (bin, -1 = no pair, -3 =
-// in a guard band or an ambiguous cell; indices past the table clamp to its
-// last entry, which is -1); bin_slow finishes the -3 cases.
-__device__ __forceinline__ int bin_fast(float r2, float tscale, const signed char* tab) {
-    int ti = (int)(r2 * tscale);
-    ti = ti > kBinTable + 1 ? kBinTable + 1 : ti;
-    return tab[ti];
-}
+// The bin of a candidate that k_scan's rounding leaves open (see Bins::bin_lim):
+// guard-widened FP32 edges, then the exact FP64 rule.
 __device__ __noinline__ int bin_slow(float r2, float lo_rej, float hi_rej, float guard0, const float2* dec,
                                      float rminf, float invw, int B, bool exact_inputs, int code,
                                      const float4* __restrict__ pts, const double* pts64, int j,

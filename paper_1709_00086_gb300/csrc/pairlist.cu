@@ -12,15 +12,20 @@
 //               fit the list pool.
 //   k_scan   -- per primary (one warp), streams the candidates of 32 cell rows
 //               at a time, slot range by slot range, decides each pair's bin
-//               exactly and compacts the accepted pairs into a staging ring in
-//               shared memory; every 32 staged pairs are placed into per-bin
-//               chunks of 32 entries (128 bytes, tagged with the bin) of this
-//               primary.  Few registers: many warps hide the candidate loads.
-//   k_accum  -- per primary (one warp), walks its chunks bin by bin: each
-//               lane takes one pair of a chunk, evaluates Y_lm (FP32
-//               recurrence, pair_common.cuh) into (lmax+1)^2 register
-//               partials, and one warp butterfly per (primary, bin) reduces
-//               them; the normalised row of multipoles goes to A.
+//               exactly and compacts the accepted pairs into a stage in shared
+//               memory; every 32 staged pairs are placed into per-bin chunks of
+//               32 (tagged with the bin) of this primary.  For a plain forward
+//               a chunk holds 32 direction records (unit vector and weight, 512
+//               bytes), for the calls that differentiate 32 list entries (slot
+//               and image, 128 bytes).
+//   k_accum_dir -- plain forwards: per primary (one warp), walks its chunks bin
+//               by bin: each lane takes one record of a chunk, adds its
+//               harmonics (Chebyshev form, pair_common.cuh) to (lmax+1)^2
+//               register partials, and one warp butterfly per (primary, bin)
+//               reduces them; the normalised row of multipoles goes to A.
+//   k_accum  -- the same from list entries (gather, separation, direction per
+//               pair): forwards to be differentiated in FP32, and plain ones
+//               whose list budget is too small for records.
 //
 // Compared with the fused kernel (pair.cu, G3PCF_OPT_PAIR_KERNELS = 1, kept as
 // a cross-check), the accumulation runs without the scan's state in registers
@@ -36,37 +41,49 @@ namespace {
 constexpr int kLWarps = 4;
 constexpr int kLThreads = kLWarps * 32;
 constexpr int kChunk = 32;      // pairs per list chunk
-constexpr int kStage = 256;     // compaction stage of k_scan (entries)
 constexpr int kTrip = 4;        // candidate sub-iterations per trip in k_scan
+constexpr int kStage = (kTrip + 1) * kChunk;  // compaction stage of k_scan (pairs)
+constexpr int kScanWarps = 8;  // warps per CTA of k_scan, kScanCtas CTAs per SM
+constexpr int kScanThreads = kScanWarps * 32;
+constexpr int kScanCtas = 4;
 constexpr unsigned kNoPair = 0xffffffffu;  // padding entry of a list chunk (image code 31 is unused)
 
-// Per-warp shared memory of k_scan: img[27] float4, pd[4] double,
-// pcs[kMaxPieces] int4 (the slot ranges of a row batch: first, end, image
-// code), stage[kStage + 32] int2 (accepted pairs: entry, bin; the last 32 are
-// scratch), per-bin fill / open chunk / chunk count.
+// Per-warp shared memory of k_scan: img[27] float4, pd[4] double, pcs[kMaxPieces]
+// int2 (the slot ranges of a row batch: first | image code << 27, end), the compaction
+// stage (kStage accepted pairs: separation and weight, or list entry, and bin),
+// per bin the last written list slot and the chunk count, R[9] float.
+template <bool DIR>
 struct ScanSmem {
-    float4* img;
-    double* pd;
-    int4* pcs;
-    int2* stage;
-    int* bfill;
-    int* bcur;
-    int* bnbc;
+    using Item = typename std::conditional<DIR, float4, int>::type;
+    float4 img[27];
+    int2 pcs[kMaxPieces];
+    Item stage[kStage];
+    int sbin[kStage];
+    int bst[32];
+    int bnbc[32];
+    double pd[4];
+    float R[12];
 };
-__host__ __device__ constexpr size_t scan_smem_per_warp(int) {
-    return 27 * 16 + 4 * 8 + kMaxPieces * 16 + (kStage + 32) * 8 + 3 * 32 * 4;
+
+// Direction record of one accepted pair in radial mode: the unit vector (z, x, y)
+// of the separation rotated to the primary's line of sight, and the weight.
+__device__ __forceinline__ float4 pair_record(const float4& d, const float* R) {
+    const float dx = fmaf(R[0], d.x, fmaf(R[1], d.y, R[2] * d.z));
+    const float dy = fmaf(R[3], d.x, fmaf(R[4], d.y, R[5] * d.z));
+    const float dz = fmaf(R[6], d.x, fmaf(R[7], d.y, R[8] * d.z));
+    const float rinv = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+    return make_float4(dz * rinv, dx * rinv, dy * rinv, d.w);
 }
-__device__ __forceinline__ ScanSmem scan_smem(unsigned char* raw, int wid, int B) {
-    unsigned char* b = raw + (size_t)wid * scan_smem_per_warp(B);
-    ScanSmem S;
-    S.img = reinterpret_cast<float4*>(b);
-    S.pd = reinterpret_cast<double*>(b + 27 * 16);
-    S.pcs = reinterpret_cast<int4*>(b + 27 * 16 + 32);
-    S.stage = reinterpret_cast<int2*>(b + 27 * 16 + 32 + kMaxPieces * 16);
-    S.bfill = reinterpret_cast<int*>(b + 27 * 16 + 32 + kMaxPieces * 16 + (kStage + 32) * 8);
-    S.bcur = S.bfill + 32;
-    S.bnbc = S.bcur + 32;
-    return S;
+// Head (nearest FP32 values) of image `code` of the primary; see set_image.
+__device__ __forceinline__ float4 image_head(int code, const float4& P0, const double* pts64, int p, double boxd) {
+    const int sx = code % 3 - 1, sy = (code / 3) % 3 - 1, sz = code / 9 - 1;
+    double x = P0.x, y = P0.y, z = P0.z;
+    if (pts64) {
+        x = pts64[3 * (int64_t)p];
+        y = pts64[3 * (int64_t)p + 1];
+        z = pts64[3 * (int64_t)p + 2];
+    }
+    return make_float4((float)(x - sx * boxd), (float)(y - sy * boxd), (float)(z - sz * boxd), 0.f);
 }
 
 __global__ void __launch_bounds__(kLThreads) k_count(ListArgs a) {
@@ -97,11 +114,50 @@ __global__ void __launch_bounds__(kLThreads) k_count(ListArgs a) {
     }
 }
 
-__global__ void __launch_bounds__(kLThreads, 7) k_scan(ListArgs a) {
+// k_scan: about 180 warp instructions per 32 accepted pairs, and every
+// instruction slot counts: a packed FMA takes two issue cycles, logic and selects
+// two on their pipe, so the kernel is bound by issue and by the shared-memory
+// pipe (70% busy), not by DRAM.  The unit vector is formed here because the
+// distance test has the separation and 1/r at hand: gathering the point again and
+// forming it in the accumulate kernel cost about 100 cycles per chunk there.  The
+// bin comes from r = r^2 rsqrt(r^2) by one rounding instead of a table look-up
+// (whose bank conflicts cost 3.5 wavefronts per 32 candidates); the 1e-4 of
+// the candidates near an edge take the exact rule.  32 warps per SM at 64
+// registers: 28 warps are 3% slower, 24 are 9%, two or three loads per trip
+// instead of four 10% and 3%.  200,000 clustered points (L = 696, 4.0e9 pairs):
+// 19.8 ms writing 16 bytes per pair, as long as the form that wrote 4 bytes and
+// left the direction to the accumulate kernel.
+//
+// What k_scan writes per pair: a list entry, or for k_accum_dir its direction (in
+// radial mode rotated to the primary's line of sight).
+constexpr int kEntries = 0, kDirs = 1, kDirsRadial = 2;
+constexpr float kRound = 12582912.f;  // 1.5 * 2^23: x + kRound rounds x to the nearest integer
+// Predicated shared-memory stores of one staged pair, without a branch.
+__device__ __forceinline__ void put_if(bool acc, unsigned at, unsigned bat, int bin, const float4& d) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.s32 p, %0, 0;\n @p st.shared.v4.f32 [%1], {%4, %5, %6, %7};\n"
+        " @p st.shared.s32 [%2], %3;\n}\n" ::"r"((int)acc), "r"(at), "r"(bat), "r"(bin), "f"(d.x), "f"(d.y),
+        "f"(d.z), "f"(d.w)
+        : "memory");
+}
+__device__ __forceinline__ void put_if(bool acc, unsigned at, unsigned bat, int bin, unsigned e) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.s32 p, %0, 0;\n @p st.shared.u32 [%1], %4;\n"
+        " @p st.shared.s32 [%2], %3;\n}\n" ::"r"((int)acc), "r"(at), "r"(bat), "r"(bin), "r"(e)
+        : "memory");
+}
+// MUFU.RSQ alone (subnormal arguments give infinity, which the caller tests).
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+template <int MODE>
+__global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
+    constexpr bool DIR = MODE != kEntries;
     extern __shared__ __align__(16) unsigned char ls_raw[];
     __shared__ double s_e2[kMaxBins + 1];
     __shared__ float2 s_dec[kMaxBins];
-    __shared__ signed char s_tab[kBinTable + 2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int B = a.bins.nbins;
     for (int k = threadIdx.x; k <= B; k += blockDim.x) {
@@ -109,17 +165,15 @@ __global__ void __launch_bounds__(kLThreads, 7) k_scan(ListArgs a) {
         if (k < B)
             s_dec[k] = make_float2(a.bins.e2f[k] + a.bins.guard[k], a.bins.e2f[k + 1] - a.bins.guard[k + 1]);
     }
-    for (int k = threadIdx.x; k < kBinTable + 2; k += blockDim.x) s_tab[k] = a.bintab[k];
     __syncthreads();
-    const ScanSmem S = scan_smem(ls_raw, wid, B);
-    const unsigned lt = lanemask_lt();
+    ScanSmem<DIR>& S = reinterpret_cast<ScanSmem<DIR>*>(ls_raw)[wid];
+    const unsigned lt = lanemask_lt(), gt = ~lt & ~(1u << lane);
     const Grid& g = a.g;
-    const float Lb = g.box;
     const bool exact_inputs = (a.pts64 == nullptr);
-    const float hi_rej = a.bins.hi_rej, lo_rej = a.bins.lo_rej, guard0 = a.bins.guard[0];
-    const float rminf = a.bins.rmin, invw = a.bins.invw, tscale = a.bin_tscale;
-    const float slack = a.bins.slack, rmax2 = a.bins.rmax2f;
+    const float invw = a.bins.invw, binc = a.bins.bin_c, lim = a.bins.bin_lim;
     const int K = g.reach, W = 2 * K + 1, nrows = W * W;
+    const unsigned stage0 = (unsigned)__cvta_generic_to_shared(S.stage);
+    const unsigned bin0 = (unsigned)__cvta_generic_to_shared(S.sbin);
     unsigned long long my_total = 0;
     long long cur_cat = -1;
 
@@ -142,83 +196,86 @@ __global__ void __launch_bounds__(kLThreads, 7) k_scan(ListArgs a) {
         }
         const long long kbase = cat * g.cells_per_cat;
         const float4 P0 = a.pts[p];
-        if (lane < 27) {
-            const int sx = lane % 3 - 1, sy = (lane / 3) % 3 - 1, sz = lane / 9 - 1;
-            S.img[lane] = make_float4(P0.x - sx * Lb, P0.y - sy * Lb, P0.z - sz * Lb, 0.f);
-        }
+        if (lane < 27) S.img[lane] = image_head(lane, P0, a.pts64, p, g.boxd);
         if (lane < 3) {
             const float pv = lane == 0 ? P0.x : (lane == 1 ? P0.y : P0.z);
             S.pd[lane] = a.pts64 ? a.pts64[3 * (int64_t)p + lane] : (double)pv;
         }
-        __syncwarp();
+        if constexpr (MODE == kDirsRadial) {
+            if (lane < 9) {
+                double x0 = P0.x, x1 = P0.y, x2 = P0.z;
+                if (a.pts64) {
+                    x0 = a.pts64[3 * (int64_t)p];
+                    x1 = a.pts64[3 * (int64_t)p + 1];
+                    x2 = a.pts64[3 * (int64_t)p + 2];
+                }
+                S.R[lane] = los_rotation_entry(lane, x0, x1, x2, g.boxd);
+            }
+        }
         const int cy = cell_of(P0.y, g), cz = cell_of(P0.z, g);
-        int* const pool = a.chunks + (int64_t)a.base[q] * kChunk;  // this primary's chunks
+        // this primary's chunks: list entries, or (DIR) one direction per pair
+        int* const pool = a.chunks + (int64_t)a.base[q] * kChunk;
+        float4* const dpool = a.dirs + (int64_t)a.base[q] * kChunk;
         int* const ptag = a.tag + a.base[q];
         int* const pord = a.ord + a.base[q];
         const int cap_ch = a.need[q];  // chunks reserved for it
         int nch = 0;                   // chunks opened so far (warp-uniform)
-        // per-bin state in shared memory: fill of the open chunk (kChunk: none
-        // open), its index, chunks opened so far
-        if (lane < B) {
-            S.bfill[lane] = kChunk;
-            S.bcur[lane] = 0;
-            S.bnbc[lane] = 0;
-        }
+        // per bin: the last written slot of the open chunk (chunk * 32 + position;
+        // -1, like any full chunk, has position 31) and the chunks opened so far
+        S.bst[lane] = -1;
+        S.bnbc[lane] = 0;
         __syncwarp();
 
-        // Place one accepted pair per lane (bin < 0: none) into the open chunk of
-        // its bin, opening a new chunk where a bin's chunk fills.  Lanes with the
-        // same bin form a group (match); its lowest lane updates the bin state.
-        auto place = [&](int entry, int bin) {
-            const bool v = bin >= 0;
-            const unsigned mine = __match_any_sync(kFull, v ? bin : 63);
+        // Place one accepted pair per lane (bin 63: none) into the open chunk of
+        // its bin, opening a new chunk where a bin's chunk fills (at most one per
+        // bin and call).  Lanes of one bin form a group (match.any: its 72 cycles run
+        // beside the other warps' instructions); the group's highest lane opens
+        // the chunk and leaves the bin's last slot.
+        auto place = [&](typename ScanSmem<DIR>::Item it, int bin, bool v) {
+            const unsigned mine = __match_any_sync(kFull, bin);
             const int rank = __popc(mine & lt);
-            const int cnt = __popc(mine);
-            const int bs = v ? bin : 0;
-            const int fill = S.bfill[bs], cur = S.bcur[bs];
-            const bool grow = v && fill + cnt > kChunk;  // at most one new chunk per call
-            const bool lead = v && rank == 0;
-            const unsigned gm = __ballot_sync(kFull, grow && rank == 0);
-            const unsigned below_leader = mine & (0u - mine);  // lowest lane of the group
-            const int nnew = nch + __popc(gm & (below_leader - 1u));
-            nch += __popc(gm);
-            const int pos = fill + rank;
-            const int c = pos < kChunk ? cur : nnew;
-            if (v && c < cap_ch) pool[(int64_t)c * kChunk + (pos & (kChunk - 1))] = entry;
-            __syncwarp();
-            if (lead) {
-                S.bfill[bin] = grow ? fill + cnt - kChunk : fill + cnt;
-                if (grow) {
+            const int st = S.bst[bin & 31];
+            const int f = (st & 31) + 1 + rank;
+            int sl = st + 1 + rank;
+            const bool last = v && (mine & gt) == 0u;
+            const bool opens = last && f >= kChunk;
+            const unsigned gm = __ballot_sync(kFull, opens);
+            if (gm) {
+                // the new chunk of this lane's group: numbered by the groups' highest lanes
+                const int hl = 31 - __clz((int)mine);
+                const int nnew = nch + __popc(gm & ((1u << hl) - 1u));
+                if (f >= kChunk) sl = nnew * kChunk + (f - kChunk);
+                nch += __popc(gm);
+                if (opens) {
                     const int nb = S.bnbc[bin];
                     if (nnew < cap_ch)
                         ptag[nnew] = (nb << 5) | bin;  // (rank among the bin's chunks, bin)
                     else
                         atomicOr(a.status, kStatusOverflow);
                     S.bnbc[bin] = nb + 1;
-                    S.bcur[bin] = nnew;
                 }
             }
+            if (v && sl < cap_ch * kChunk) {
+                if constexpr (MODE == kDirs)
+                    dpool[sl] = it;
+                else if constexpr (MODE == kDirsRadial)
+                    dpool[sl] = pair_record(it, S.R);
+                else
+                    pool[sl] = it;
+            }
+            // (every lane has read the bin state: the ballot waited for it)
+            if (last) S.bst[bin] = sl;
             __syncwarp();
         };
-        // accepted pairs are first compacted into stage (warp-uniform head/count)
-        int shead = 0, scnt = 0;
-        auto drain = [&]() {
-            while (scnt >= kChunk) {
-                __syncwarp();
-                const int2 v = S.stage[(shead + lane) & (kStage - 1)];
-                shead = (shead + kChunk) & (kStage - 1);
-                scnt -= kChunk;
-                __syncwarp();
-                place(v.x, v.y);
-            }
-        };
+        int scnt = 0;  // accepted pairs in the stage (warp-uniform)
 
         // candidates: batches of 32 cell rows -> slot ranges (pieces) -> up to
         // kTrip x 32 slots per trip, all loads of a trip in flight together
         for (int rb = 0; rb < nrows; rb += 32) {
             int4 pm = make_int4(0, 0, 0, 0), p0 = pm, pp = pm;
             const int r = rb + lane;
-            if (r < nrows) row_pieces(r, W, K, cy, cz, P0, g, slack, rmax2, kbase, a.cstart, pm, p0, pp);
+            if (r < nrows)
+                row_pieces(r, W, K, cy, cz, P0, g, a.bins.slack, a.bins.rmax2f, kbase, a.cstart, pm, p0, pp);
             const int npc = (pm.y > pm.x) + (p0.y > p0.x) + (pp.y > pp.x);
             int incl = npc;
 #pragma unroll
@@ -230,73 +287,96 @@ __global__ void __launch_bounds__(kLThreads, 7) k_scan(ListArgs a) {
             __syncwarp();
             {
                 int k = incl - npc;
-                if (pm.y > pm.x) S.pcs[k++] = pm;
-                if (p0.y > p0.x) S.pcs[k++] = p0;
-                if (pp.y > pp.x) S.pcs[k++] = pp;
+                if (pm.y > pm.x) S.pcs[k++] = make_int2((int)((unsigned)pm.x | ((unsigned)pm.z << kIdxBits)), pm.y);
+                if (p0.y > p0.x) S.pcs[k++] = make_int2((int)((unsigned)p0.x | ((unsigned)p0.z << kIdxBits)), p0.y);
+                if (pp.y > pp.x) S.pcs[k++] = make_int2((int)((unsigned)pp.x | ((unsigned)pp.z << kIdxBits)), pp.y);
             }
             __syncwarp();
             for (int pi = 0; pi < npcs; ++pi) {
-                const int4 pc = S.pcs[pi];
-                const float4 o = S.img[pc.z];
-                const unsigned codebits = (unsigned)pc.z << kIdxBits;
-                for (int j0 = pc.x; j0 < pc.y; j0 += kTrip * kChunk) {
-                    const int nu = (pc.y - j0 + kChunk - 1) / kChunk;  // sub-iterations with slots
-                    // slots past the piece read as a far point (r^2 ~ 1e36: no pair)
-                    float4 qv[kTrip];
+                const int2 pc = S.pcs[pi];
+                const unsigned code = (unsigned)pc.x >> kIdxBits;
+                const float4 o = S.img[code];
+                for (int j0 = (pc.x & (int)kIdxMask) + lane; j0 < pc.y + lane; j0 += kTrip * kChunk) {
+                    // slots past the piece keep a far x (r^2 ~ 1e36: no pair)
+                    const float4* src = a.pts + j0;
+                    float4 d[kTrip];
 #pragma unroll
                     for (int u = 0; u < kTrip; ++u) {
-                        const int j = j0 + u * kChunk + lane;
-                        qv[u] = make_float4(o.x + 1e18f, o.y, o.z, 0.f);
-                        if (j < pc.y) qv[u] = __ldg(a.pts + j);
+                        d[u] = make_float4(1e18f, 0.f, 0.f, 0.f);
+                        if (j0 + u * kChunk < pc.y) d[u] = __ldg(src + u * kChunk);
                     }
+                    // bin = round((r - rmin) / width - 1/2); within bin_lim of the bin's
+                    // centre (in widths) the FP32 bin is the exact one, else (and where
+                    // r is NaN: r^2 is 0 or subnormal) bin_slow decides
                     int bn[kTrip];
-                    bool chk = false;
+                    float rinv[kTrip];
+                    bool near[kTrip], any = false;
 #pragma unroll
                     for (int u = 0; u < kTrip; ++u) {
-                        const float dx = qv[u].x - o.x, dy = qv[u].y - o.y, dz = qv[u].z - o.z;
-                        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        bn[u] = bin_fast(r2, tscale, s_tab);
-                        chk |= bn[u] < -1;
+                        d[u].x -= o.x;
+                        d[u].y -= o.y;
+                        d[u].z -= o.z;
+                        const float r2 = fmaf(d[u].x, d[u].x, fmaf(d[u].y, d[u].y, d[u].z * d[u].z));
+                        rinv[u] = rsqrt_ftz(r2);
+                        const float t = fmaf(r2 * rinv[u], invw, binc);
+                        const float m = __fadd_rn(t, kRound);
+                        bn[u] = __float_as_int(m) - __float_as_int(kRound);
+                        near[u] = !(fabsf(__fsub_rn(t, __fsub_rn(m, kRound))) <= lim);
+                        any |= near[u];
                     }
-                    if (__any_sync(kFull, chk)) {
+                    if (__any_sync(kFull, any)) {
 #pragma unroll
-                        for (int u = 0; u < kTrip; ++u) {
-                            if (bn[u] == -3) {
-                                const int j = j0 + u * kChunk + lane;
-                                const float dx = qv[u].x - o.x, dy = qv[u].y - o.y, dz = qv[u].z - o.z;
-                                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                                bn[u] = bin_slow(r2, lo_rej, hi_rej, guard0, s_dec, rminf, invw, B, exact_inputs,
-                                                 pc.z, a.pts, a.pts64, j, S.pd, g.boxd, g.periodic, s_e2);
+                        for (int u = 0; u < kTrip; ++u)
+                            if (near[u]) {
+                                const float r2 = fmaf(d[u].x, d[u].x, fmaf(d[u].y, d[u].y, d[u].z * d[u].z));
+                                rinv[u] = rsqrtf(r2);
+                                bn[u] = bin_slow(r2, a.bins.lo_rej, a.bins.hi_rej, a.bins.guard[0], s_dec,
+                                                 a.bins.rmin, invw, B, exact_inputs, (int)code, a.pts, a.pts64,
+                                                 j0 + u * kChunk, S.pd, g.boxd, g.periodic, s_e2);
                             }
-                        }
                     }
 #pragma unroll
                     for (int u = 0; u < kTrip; ++u) {
-                        if (u < nu) {
-                            // accepted lanes append in lane order; the others write a scratch slot
-                            const bool acc = bn[u] >= 0;
-                            const unsigned vm = __ballot_sync(kFull, acc);
-                            const int at = acc ? ((shead + scnt + __popc(vm & lt)) & (kStage - 1)) : kStage + lane;
-                            S.stage[at] = make_int2((int)((unsigned)(j0 + u * kChunk + lane) | codebits), bn[u]);
-                            scnt += __popc(vm);
-                        }
+                        // accepted lanes append in lane order
+                        const bool acc = (unsigned)bn[u] < (unsigned)B;
+                        const unsigned vm = __ballot_sync(kFull, acc);
+                        const int at = scnt + __popc(vm & lt);
+                        if constexpr (MODE == kDirs)
+                            put_if(acc, stage0 + at * 16, bin0 + at * 4, bn[u],
+                                   make_float4(d[u].z * rinv[u], d[u].x * rinv[u], d[u].y * rinv[u], d[u].w));
+                        else if constexpr (MODE == kDirsRadial)
+                            put_if(acc, stage0 + at * 16, bin0 + at * 4, bn[u], d[u]);
+                        else
+                            put_if(acc, stage0 + at * 4, bin0 + at * 4, bn[u],
+                                   (unsigned)(j0 + u * kChunk) | (code << kIdxBits));
+                        scnt += __popc(vm);
                     }
-                    drain();
+                    if (scnt >= kChunk) {
+                        __syncwarp();
+                        int at = lane;
+                        for (; scnt >= kChunk; scnt -= kChunk, at += kChunk) place(S.stage[at], S.sbin[at], true);
+                        // the rest (fewer than 32) to the stage's front
+                        const auto it = S.stage[at];
+                        const int bin = S.sbin[at];
+                        __syncwarp();
+                        S.stage[lane] = it;
+                        S.sbin[lane] = bin;
+                        __syncwarp();
+                    }
                 }
             }
             __syncwarp();
         }
         if (scnt > 0) {  // the last accepted pairs (fewer than 32)
             __syncwarp();
-            const int2 v = lane < scnt ? S.stage[(shead + lane) & (kStage - 1)] : make_int2(0, -1);
-            __syncwarp();
-            place(v.x, v.y);
+            place(S.stage[lane], lane < scnt ? S.sbin[lane] : 63, lane < scnt);
         }
         // the bin state back in lane b
         int cfill = kChunk, ccur = 0, nbc = 0;
         if (lane < B) {
-            cfill = S.bfill[lane];
-            ccur = S.bcur[lane];
+            const int st = S.bst[lane];
+            cfill = (st & 31) + 1;
+            ccur = st >> 5;
             nbc = S.bnbc[lane];
         }
         const unsigned padd = nbc > 0 ? (unsigned)((nbc - 1) * kChunk + cfill) : 0u;  // pairs of bin lane
@@ -307,7 +387,12 @@ __global__ void __launch_bounds__(kLThreads, 7) k_scan(ListArgs a) {
             pmask &= pmask - 1;
             const int c = __shfl_sync(kFull, ccur, b);
             const int f = __shfl_sync(kFull, cfill, b);
-            if (lane >= f && c < cap_ch) pool[(int64_t)c * kChunk + lane] = (int)kNoPair;
+            if (lane >= f && c < cap_ch) {
+                if constexpr (DIR)
+                    dpool[c * kChunk + lane] = make_float4(0.f, 1.f, 0.f, 0.f);  // weight 0
+                else
+                    pool[c * kChunk + lane] = (int)kNoPair;
+            }
         }
         // list the chunks grouped by bin (stable): position = chunks of the
         // lower bins + rank inside the bin
@@ -327,6 +412,10 @@ __global__ void __launch_bounds__(kLThreads, 7) k_scan(ListArgs a) {
                 const int pos = __shfl_sync(kFull, off, b) + (t >> 5);
                 if (c < nlist && pos < cap_ch) pord[pos] = c | (b << 26);
             }
+        }
+        if constexpr (DIR) {  // the tags are read: their first nbins ints take the bins' chunk counts
+            __syncwarp();
+            if (lane < B) ptag[lane] = nbc;
         }
         if (lane == 0) a.nchunks[q] = nch < cap_ch ? nch : cap_ch;
         my_total += padd;
@@ -419,6 +508,11 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool vali
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     const int n = valid ? 16 : 0;
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+// 16 bytes past L1
+__device__ __forceinline__ void cp_async16_cg(void* dst, const void* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -675,6 +769,90 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
     }
 }
 
+// The accumulate kernel of plain forwards: the lists hold direction records
+// (k_scan), so a chunk costs one 16-byte copy and one shared-memory load per lane
+// and the harmonics.  Bound by issue: at lmax = 10 a chunk's 55 packed FMAs take
+// two issue cycles each, the recurrences of T_k and (x + iy)^m about 65 more, the
+// list walk about 30; the loop body without any load measures 208 cycles per chunk
+// and SM quarter, the kernel 232 (the form that gathers points from list entries:
+// 310).  200,000 clustered points (L = 696, 4.0e9 pairs, lmax = 10): 25.2 ms
+// against 33.8.  The list words of 32 chunks are held one per lane and read by
+// shuffle (a load per chunk: 25.9 ms).
+constexpr int kDirRing = 8;
+__host__ __device__ constexpr size_t accum_dir_smem_per_warp(int B, int NRP) {
+    return (size_t)B * NRP * 4 + kDirRing * 32 * 16;
+}
+template <int L>
+__global__ void __launch_bounds__(kLThreads, 3) k_accum_dir(ListArgs a) {
+    constexpr int NRP = Shape<L>::NRP;
+    extern __shared__ __align__(16) unsigned char la_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int B = a.bins.nbins;
+    unsigned char* base = la_raw + (size_t)wid * accum_dir_smem_per_warp(B, NRP);
+    float4* ring = reinterpret_cast<float4*>(base) + lane;
+    float* res = reinterpret_cast<float*>(base + kDirRing * 32 * 16);
+    const int qa = a.qrange ? a.qrange[0] : a.qa, qb = a.qrange ? a.qrange[1] : a.qb;
+    for (;;) {
+        int q = 0;
+        if (lane == 0) q = qa + atomicAdd(a.queue, 1);
+        q = __shfl_sync(kFull, q, 0);
+        if (q >= qb) break;
+        const int p = a.plist ? a.plist[q] : q;
+        const float w0 = a.pts[p].w;
+        const int cb = a.base[q] < 0 ? 0 : a.base[q];
+        const int nch = a.nchunks[q];
+        const int nbc = nch > 0 && lane < B ? a.tag[cb + lane] : 0;  // chunks of bin lane
+        const float4* recs = a.dirs + (int64_t)cb * kChunk + lane;
+        const int* ordp = a.ord + cb;
+        for (int k = lane; k < B * NRP; k += 32) res[k] = 0.f;
+        __syncwarp();
+        if (nch > 0) {
+            // every lane copies and reads its own record: the ring needs no barrier
+            auto copy = [&](int i, unsigned o) {
+                cp_async16_cg(ring + (i & (kDirRing - 1)) * 32, recs + (o & 0x3ffffffu) * kChunk);
+            };
+            auto slot = [&](int i) -> unsigned { return i < nch ? (unsigned)__ldg(ordp + i) : 0u; };
+#pragma unroll
+            for (int k = 0; k < kDirRing - 1; ++k) {
+                if (k < nch) copy(k, slot(k));
+                cp_async_commit();
+            }
+            // list words: 32 chunks' in the lanes, the next 32 loading
+            unsigned ow = slot(lane), ow2 = slot(32 + lane);
+            constexpr int NC = Cheb<L>::NC > 0 ? Cheb<L>::NC : 1;
+            int i = 0;
+            for (int b = 0; b < B; ++b) {
+                const int end = i + __shfl_sync(kFull, nbc, b);
+                if (end == i) continue;
+                float acc0[L + 1];
+                float2 accc[NC];
+                static_for<0, L + 1>([&](auto kc) { acc0[decltype(kc)::value] = 0.f; });
+                static_for<0, NC>([&](auto ic) { accc[decltype(ic)::value] = make_float2(0.f, 0.f); });
+                for (; i < end; ++i) {
+                    cp_async_wait<kDirRing - 2>();  // the records of chunk i have landed
+                    const float4 v = ring[(i & (kDirRing - 1)) * 32];
+                    const int ic = i + kDirRing - 1;
+                    if ((ic & 31) == 0) {
+                        ow = ow2;
+                        ow2 = slot(ic + 32 + lane);
+                    }
+                    const unsigned o = __shfl_sync(kFull, ow, ic & 31);
+                    if (ic < nch) copy(ic, o);
+                    cp_async_commit();
+                    accum_pair_cheb<L>(acc0, accc, v.x, v.y, v.z, v.w);
+                }
+                reduce_cheb<L>(acc0, accc, lane, res + b * NRP);
+            }
+            cp_async_wait<0>();
+        }
+        __syncwarp();
+        const int row = a.chunked ? q - a.q0 : a.orig[p];
+        emit_row(a, res, row, p, w0, lane);
+        if (lane == 0) a.wrow[row] = w0;
+        __syncwarp();
+    }
+}
+
 // Adjoint pair pass over the pair lists (the derivative of Sec. 3.1's a_lm
 // with the pair set and bins held fixed).  Per primary i and bin b the adjoint
 // multipoles H_lm = w_i K_lm V_i (V = M A, slot layout) are carried to the
@@ -889,22 +1067,40 @@ int launch_accum_e(const ListArgs& a, int nsm, cudaStream_t st) {
 }
 
 template <int L>
-int launch_accum_t(const ListArgs& a, int nsm, cudaStream_t st) {
-    return a.exact_img ? launch_accum_e<L, true>(a, nsm, st) : launch_accum_e<L, false>(a, nsm, st);
-}
-
-int launch_scan_k(const ListArgs& a, int nsm, cudaStream_t st) {
-    const size_t smem = scan_smem_per_warp(a.bins.nbins) * kLWarps;
-    if (cudaFuncSetAttribute(k_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+int launch_accum_dir_t(const ListArgs& a, int nsm, cudaStream_t st) {
+    const size_t smem = accum_dir_smem_per_warp(a.bins.nbins, Shape<L>::NRP) * kLWarps;
+    if (cudaFuncSetAttribute(k_accum_dir<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return -1;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scan, kLThreads, smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_accum_dir<L>, kLThreads, smem) != cudaSuccess ||
         per_sm < 1)
         return -1;
     int blocks = per_sm * nsm;
     const int need = (a.qb - a.qa + kLWarps - 1) / kLWarps;
+    if (!a.qrange && blocks > need) blocks = need > 0 ? need : 1;
+    k_accum_dir<L><<<blocks, kLThreads, smem, st>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+template <int L>
+int launch_accum_t(const ListArgs& a, int nsm, cudaStream_t st) {
+    if (a.dirs) return launch_accum_dir_t<L>(a, nsm, st);
+    return a.exact_img ? launch_accum_e<L, true>(a, nsm, st) : launch_accum_e<L, false>(a, nsm, st);
+}
+
+template <int MODE>
+int launch_scan_k(const ListArgs& a, int nsm, cudaStream_t st) {
+    const size_t smem = sizeof(ScanSmem<MODE != kEntries>) * kScanWarps;
+    if (cudaFuncSetAttribute(k_scan<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return -1;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scan<MODE>, kScanThreads, smem) != cudaSuccess ||
+        per_sm < 1)
+        return -1;
+    int blocks = per_sm * nsm;
+    const int need = (a.qb - a.qa + kScanWarps - 1) / kScanWarps;
     if (!a.qrange && blocks > need) blocks = need;
-    k_scan<<<blocks, kLThreads, smem, st>>>(a);
+    k_scan<MODE><<<blocks, kScanThreads, smem, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -921,7 +1117,8 @@ int launch_count(const ListArgs& a, int nsm, cudaStream_t st) {
 
 int launch_scan(const ListArgs& a, int nsm, cudaStream_t st) {
     if (!a.qrange && a.qb <= a.qa) return 0;
-    return launch_scan_k(a, nsm, st);
+    if (!a.dirs) return launch_scan_k<kEntries>(a, nsm, st);
+    return a.g.radial ? launch_scan_k<kDirsRadial>(a, nsm, st) : launch_scan_k<kDirs>(a, nsm, st);
 }
 
 size_t plan_scan_tmp_bytes(int64_t n) { return 8 * (size_t)((n + kScan64 - 1) / kScan64 + 1); }
