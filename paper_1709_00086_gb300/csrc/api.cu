@@ -1036,8 +1036,14 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
         std::vector<std::vector<int>> ccats(nchunks);
         std::vector<int64_t> cpad(nchunks, 0);
         int total_segs = 0;
+        auto fp32_seg = [](int64_t len) { return std::max<int64_t>(8192, len / 32); };
         for (int64_t ch = 0; ch < nchunks; ++ch) {
             const int64_t q0 = ch * C, q1 = chunked ? std::min(rows_all, q0 + C) : rows_all;
+            int64_t nbase = 0;  // base segments of this pass's FP32 contraction
+            for (int k = 0; k < c.ncat; ++k) {
+                const int64_t len = chunked ? q1 - q0 : (c.ncat > 1 ? c.offs[k + 1] - c.offs[k] : c.n_primary);
+                nbase += (len + fp32_seg(len) - 1) / fp32_seg(len);
+            }
             for (int k = 0; k < c.ncat; ++k) {
                 if (ch == 0) segfirst[k] = total_segs + (int)csegs[ch].size();
                 // rows of catalog k inside this pass (A-row coordinates)
@@ -1068,15 +1074,17 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
                     }
                     cpad[ch] += plen;
                 } else {
-                    int64_t seg = len / 32;
-                    if (seg < 8192) seg = 8192;
-                    for (int64_t s0 = r0; s0 < r1; s0 += seg) {
-                        Segment sg;
-                        sg.cat = k;
-                        sg.row0 = (int)s0;
-                        sg.row1 = (int)(s0 + seg < r1 ? s0 + seg : r1);
-                        csegs[ch].push_back(sg);
-                    }
+                    // base segments, each cut into parts where there are too few CTAs
+                    const int64_t seg = fp32_seg(len);
+                    const int64_t part = contract_fp32_split(seg, nbase, ntiles, P->nsm);
+                    for (int64_t s0 = r0; s0 < r1; s0 += seg)
+                        for (int64_t p0 = s0, s1 = std::min(r1, s0 + seg); p0 < s1; p0 += part) {
+                            Segment sg;
+                            sg.cat = k;
+                            sg.row0 = (int)p0;
+                            sg.row1 = (int)std::min(s1, p0 + part);
+                            csegs[ch].push_back(sg);
+                        }
                 }
             }
             total_segs += (int)csegs[ch].size();

@@ -16,78 +16,134 @@ namespace g3 {
 
 namespace {
 
-constexpr int kT = 64;       // tile edge
-constexpr int kKC = 32;      // rows per smem stage
-constexpr int kThreads = 256;
-constexpr int kFlushRows = 256;  // FP32 run length before a compensated add
+// One warp per 32 x 32 tile and range of primaries, four warps (row ranges) per
+// CTA; a lane holds 8 x 4 entries of the tile.  Bound by issue: per primary and
+// warp 16 packed FMAs (two issue cycles each) and about 20 other instructions.
+// 32-wide tiles leave 1.5 entries computed per entry of the triangle (64-wide
+// ones 2.1 at B = lmax = 10).  Runs of kFlushRows primaries are summed in FP32, the
+// runs in double-float (head + tail, 2^-48): FP64 additions, at 1/58 of the FP32
+// rate, would take a third of the kernel's time.  20,000 primaries, B = lmax = 10:
+// 0.20 ms (10 row parts, 1,220 CTAs) against 1.29 ms for 64-wide tiles with 4 x 4 scalar
+// FMAs per thread, whose 129 CTAs left most SMs one block of 8,192 rows.
+constexpr int kT = 32;           // tile edge
+constexpr int kKC = 8;           // rows per shared-memory stage
+constexpr int kCWarps = 4;
+constexpr int kThreads = kCWarps * 32;
+constexpr int kFlushRows = 256;  // FP32 run length
+static_assert(kFlushRows % kKC == 0, "a run is whole stages");
 
-__device__ __forceinline__ void two_sum(double& hi, float v) {
-    hi += (double)v;  // FP64 add of an FP32 run sum: error far below FP32 rounding
+struct ContractSmem {
+    float a[kKC][kT];            // weighted rows, left side
+    float b[kKC][kT];
+    float2 tot[32][32];          // [entry of a lane][lane]: sum of the finished runs
+};
+
+__device__ __forceinline__ float2 neg2(float2 x) { return make_float2(-x.x, -x.y); }
+// (h, l) += v for two sums at once: error-free addition to the head, its rounding
+// error into the tail
+__device__ __forceinline__ void run_add(float2& h, float2& l, float2 v) {
+    const float2 s = __fadd2_rn(h, v);
+    const float2 bb = __fadd2_rn(s, neg2(h));
+    const float2 e = __fadd2_rn(__fadd2_rn(h, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(v, neg2(bb)));
+    l = __fadd2_rn(l, e);
+    h = s;
 }
 
-__global__ void __launch_bounds__(kThreads) k_contract_fp32(const float* __restrict__ A, int RLP,
-                                                          const float* __restrict__ wrow,
-                                                          const Tile* tiles, const Segment* segs,
-                                                          double* partials, int part_stride) {
-    __shared__ __align__(16) float sa[kKC][kT];
-    __shared__ __align__(16) float sb[kKC][kT];
+__global__ void __launch_bounds__(kThreads, 4) k_contract_fp32(const float* __restrict__ A, int RLP,
+                                                               const float* __restrict__ wrow,
+                                                               const Tile* tiles, const Segment* segs,
+                                                               double* partials, int part_stride) {
+    extern __shared__ __align__(16) unsigned char cs_raw[];
+    ContractSmem* sm = reinterpret_cast<ContractSmem*>(cs_raw);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    ContractSmem& S = sm[wid];
     const Tile t = tiles[blockIdx.x];
     const Segment sg = segs[blockIdx.y];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4];
-    double tot[4][4];
+    // lane: rows 8 ty .. + 7 and columns 4 tx .. + 3 of the tile
+    const int tx = lane & 7, ty = lane >> 3;
+    // this warp's runs of the segment
+    const int nruns = (sg.row1 - sg.row0 + kFlushRows - 1) / kFlushRows;
+    const int first = sg.row0 + wid * nruns / kCWarps * kFlushRows;
+    const int last = min(sg.row1, sg.row0 + (wid + 1) * nruns / kCWarps * kFlushRows);
+    const bool va = lane < t.rows, vb = lane < t.cols, diag = t.r0 == t.c0;
+    const float* pa = A + (int64_t)first * RLP + t.col0 + t.r0 + (va ? lane : 0);
+    const float* pb = A + (int64_t)first * RLP + t.col0 + t.c0 + (vb ? lane : 0);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int e = 0; e < 32; ++e) S.tot[e][lane] = make_float2(0.f, 0.f);
+    // acc[j][i]: rows 8 ty + 2 i, + 1 (the packed pair) of column 4 tx + j
+    float2 acc[4][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            acc[i][j] = 0.f;
-            tot[i][j] = 0.0;
-        }
-    int since = 0;
-    for (int r0 = sg.row0; r0 < sg.row1; r0 += kKC) {
-        // stage kKC rows of the two column windows (rows weighted on the left)
-        for (int k = threadIdx.x; k < kKC * kT; k += kThreads) {
-            const int rr = k / kT, cc = k % kT;
-            const int row = r0 + rr;
-            float va = 0.f, vb = 0.f;
-            if (row < sg.row1) {
-                const float* Ar = A + (int64_t)row * RLP + t.col0;
-                if (cc < t.rows) va = Ar[t.r0 + cc] * wrow[row];
-                if (cc < t.cols) vb = Ar[t.c0 + cc];
-            }
-            sa[rr][cc] = va;
-            sb[rr][cc] = vb;
-        }
-        __syncthreads();
-#pragma unroll 8
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[j][i] = make_float2(0.f, 0.f);
+    float ra[kKC], rb[kKC], rw[kKC];
+    auto fetch = [&](int r0) {
+#pragma unroll
         for (int k = 0; k < kKC; ++k) {
-            const float4 a4 = *reinterpret_cast<const float4*>(&sa[k][ty * 4]);
-            const float4 b4 = *reinterpret_cast<const float4*>(&sb[k][tx * 4]);
-            const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+            const bool in = r0 + k < last;
+            rw[k] = in ? __ldg(wrow + r0 + k) : 0.f;
+            ra[k] = in && va ? __ldg(pa) : 0.f;
+            rb[k] = diag ? ra[k] : (in && vb ? __ldg(pb) : 0.f);
+            pa += RLP;
+            pb += RLP;
+        }
+    };
+    if (first < last) fetch(first);
+    for (int r0 = first; r0 < last; r0 += kKC) {
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kKC; ++k) {
+            S.a[k][lane] = ra[k] * rw[k];
+            S.b[k][lane] = rb[k];
+        }
+        __syncwarp();
+        if (r0 + kKC < last) fetch(r0 + kKC);
+#pragma unroll
+        for (int k = 0; k < kKC; ++k) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&S.a[k][8 * ty]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&S.a[k][8 * ty + 4]);
+            const float4 b4 = *reinterpret_cast<const float4*>(&S.b[k][4 * tx]);
+            const float2 av[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
+                                  make_float2(a1.z, a1.w)};
             const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+                for (int i = 0; i < 4; ++i) acc[j][i] = __ffma2_rn(av[i], make_float2(bv[j], bv[j]), acc[j][i]);
         }
-        __syncthreads();
-        since += kKC;
-        if (since >= kFlushRows) {
+        if ((r0 + kKC - sg.row0) % kFlushRows == 0 || r0 + kKC >= last) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    two_sum(tot[i][j], acc[i][j]);
-                    acc[i][j] = 0.f;
+                for (int i = 0; i < 4; ++i) {
+                    float2* to = &S.tot[2 * (4 * j + i)][lane];
+                    float2 x = to[0], y = to[32];  // (head, tail) of the pair's two entries
+                    float2 h = make_float2(x.x, y.x), l = make_float2(x.y, y.y);
+                    run_add(h, l, acc[j][i]);
+                    to[0] = make_float2(h.x, l.x);
+                    to[32] = make_float2(h.y, l.y);
+                    acc[j][i] = make_float2(0.f, 0.f);
                 }
-            since = 0;
         }
     }
+    // the four warps' sums, in warp order: warp w takes the lanes' entries 8 w .. + 7
+    __syncthreads();
     double* out = partials + (int64_t)blockIdx.y * part_stride + t.out_off;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int q = 0; q < 8; ++q) {
+        const int e = 8 * wid + q;  // = 2 (4 j + i) + part
+        float h = 0.f, l = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) out[(ty * 4 + i) * kT + tx * 4 + j] = tot[i][j] + (double)acc[i][j];
+        for (int w = 0; w < kCWarps; ++w) {
+            const float2 v = sm[w].tot[e][lane];
+            const float s = __fadd_rn(h, v.x), bb = __fsub_rn(s, h);
+            const float er = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(v.x, bb));
+            l = __fadd_rn(l, __fadd_rn(v.y, er));
+            h = s;
+        }
+        const int j = e >> 3, i = (e >> 1) & 3, part = e & 1;
+        out[(8 * ty + 2 * i + part) * kT + 4 * tx + j] = (double)h + (double)l;
+    }
 }
 
 struct BlockInfo {
@@ -186,6 +242,17 @@ int launch_combine(const double* zeta, int64_t zsize, int ncat, const double* co
 
 int contract_tile_dim_fp32() { return kT; }
 
+// Rows per segment when the base segments (of `seg` rows) alone leave the chip
+// idle: about three CTAs per slot (4 per SM), whole runs for every warp.
+int64_t contract_fp32_split(int64_t seg, int64_t nbase, int ntiles, int nsm) {
+    const int64_t step = (int64_t)kCWarps * kFlushRows;
+    const int64_t have = nbase * ntiles, want = (int64_t)nsm * 4 * 3;
+    if (have <= 0 || have >= want) return seg;
+    const int64_t parts = (want + have - 1) / have;
+    const int64_t rows = ((seg + parts - 1) / parts + step - 1) / step * step;
+    return rows < seg ? rows : seg;
+}
+
 // Tiles of edge T over the upper triangle of every C_m (row-major in (ti, tj)).
 int make_tiles(int nbins, int lmax, int T, Tile* out, int max_tiles) {
     return fill_tiles(nbins, lmax, T, out, max_tiles);
@@ -195,8 +262,11 @@ int launch_contract_fp32(const float* A, int RLP, const float* wrow, const Tile*
                          const Segment* segs, int nsegs, double* partials, int part_stride,
                          cudaStream_t st) {
     if (ntiles <= 0 || nsegs <= 0) return 0;
+    const size_t smem = sizeof(ContractSmem) * kCWarps;
+    if (cudaFuncSetAttribute(k_contract_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return -1;
     dim3 grid(ntiles, nsegs);
-    k_contract_fp32<<<grid, kThreads, 0, st>>>(A, RLP, wrow, tiles, segs, partials, part_stride);
+    k_contract_fp32<<<grid, kThreads, smem, st>>>(A, RLP, wrow, tiles, segs, partials, part_stride);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -291,6 +291,7 @@ __host__ __device__ inline int count_tiles(int nbins, int lmax, int T) {
     return n;
 }
 int contract_tile_dim_fp32();
+int64_t contract_fp32_split(int64_t seg, int64_t nbase, int ntiles, int nsm);
 int launch_contract_fp32(const float* A, int RLP, const float* wrow, const Tile* tiles, int ntiles,
                          const Segment* segs, int nsegs, double* partials, int part_stride,
                          cudaStream_t st);

@@ -112,7 +112,9 @@ int noalloc_zeta_from_alm(int nbins, int lmax, const float* alm, int64_t ld, con
                  part_stride, kNoAllocPartialDoubles);
         return G3PCF_ERR_ARG;
     }
-    int nsegs_max = (int)(kNoAllocPartialDoubles / part_stride);
+    // segments of equal length, as many as fit in partials of 64-wide tiles (the
+    // 32-wide ones take less): the lengths fix where the FP32 runs of the sum end
+    int nsegs_max = (int)(kNoAllocPartialDoubles / ((size_t)count_tiles(nbins, lmax, 64) * 64 * 64));
     if (nsegs_max > kNoAllocMaxSegs) nsegs_max = kNoAllocMaxSegs;
     // segments of primaries: at least 4096 rows each, at most nsegs_max of them
     int64_t seg = 4096;
