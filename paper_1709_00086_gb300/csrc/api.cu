@@ -653,6 +653,7 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     la.A = pa.A;
     la.RLP = pa.RLP;
     la.colconv = P->d_colconv.as<int4>();
+    la.slotconv = P->d_slotconv.as<int4>();
     la.colcoef = P->d_colcoef.as<float>();
     la.RL = pa.RL;
     la.counts = pa.counts;
@@ -674,7 +675,6 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         la.V = pa.V;
         la.dw = pa.dw;
         la.dpos = pa.dpos;
-        la.slotconv = P->d_slotconv.as<int4>();
         la.slotcoef = P->d_slotcoef.as<float>();
         la.Vdf = P->d_Vdf.as<float2>();
     }

@@ -17,16 +17,24 @@
 //                 lane evaluates one pair: the separation from the primary's
 //                 image (FP32 head + tail of the FP64 image, so the difference
 //                 is exact), r^2, 1/r by one Newton step from rsqrt, the unit
-//                 vector, T_k(z) and w (x + iy)^m, all in double-float, into a
-//                 shared-memory record.  Then every lane adds the chunk's 32
-//                 terms T_k w (x + iy)^m to the accumulator slots it owns, two
-//                 slots per packed f32x2 operation (double-float sums, no
-//                 cross-lane reduction).  At a change of bin the slots go to
-//                 double-float shared memory; at the primary's end the
-//                 Chebyshev -> Legendre-form connection (times K_lm, head +
-//                 tail coefficients) is applied in double-float and the row
-//                 of A is stored.  No FP64 arithmetic: the FP64 pipe runs at
-//                 1/58 of the FP32 rate here.
+//                 vector, T_k(z) and w (x + iy)^m, all in double-float.  The m = 0
+//                 sums stay with the lane; the rest goes through a shared-memory
+//                 record to the lanes that own the sums of each m >= 1 (two k of
+//                 one m per lane, several pairs of the chunk side by side where the
+//                 sums fit in part of the warp), added with biased heads
+//                 (bias_fma).  At the end of a bin the Chebyshev ->
+//                 Legendre-form connection (times K_lm, head + tail
+//                 coefficients) is applied in double-float; the row of A is
+//                 stored at the primary's end.  No FP64 arithmetic: the FP64
+//                 pipe runs at 1/58 of the FP32 rate.  Bound by issue, with
+//                 shared memory (records in and out) close behind: 1,250 cycles
+//                 per chunk and SM quarter at lmax = 6.  100,000 clustered
+//                 points, lmax = 6 (7.1e8 pairs): 24 ms, against 40 ms with
+//                 12 instead of 6 operations per term and one sum pair per lane
+//                 (twice the shared-memory bytes per term).  Sums in the
+//                 registers of the pair's lane alone (no records, a
+//                 reduction of every sum per bin) took 23 ms there, but three
+//                 times this kernel's time at 55 pairs per bin and lmax = 10.
 //   k_adj_df   -- per primary (one warp), one pair per lane: the adjoint
 //                 coefficients G_{m,k} = w_i sum_l c^(m)_{l-m,k} K_lm V_lm of
 //                 the primary (FP64 from the FP64 V = M A, held as head + tail
@@ -177,88 +185,104 @@ __device__ __forceinline__ void load_sec(const ListArgs& a, unsigned e, float4& 
 }
 
 // ---- forward ----------------------------------------------------------------
-// The (lmax+1)^2 accumulator slots are handled in pairs, two slots per packed
-// (f32x2) operation: the m = 0 slots k, k + 1 (k even), and for m >= 1 the Re
-// and Im slots of one (m, k).  Per-pair record in shared memory (floats, every
-// group of four 16-byte aligned so that one 128-bit load gives a slot pair's
-// head pair and tail pair):
-//   TA (m = 0), k even:  T_k.h, T_k+1.h, T_k.l, T_k+1.l      (LE = lmax+1 rounded up to even)
-//   TB (m >= 1), k < L:  T_k.h, T_k.h,   T_k.l, T_k.l
-//   W:                   w,     w,       0,     0
-//   CB, m = 1..L:        Re.h,  Im.h,    Re.l,  Im.l         of w (x + iy)^m
-// Row stride RS (floats) a multiple of 4.
-template <int L>
-struct DfRec {
-    static constexpr int LE = (L + 2) & ~1;       // m = 0 slots, padded to even
-    static constexpr int TA = 0;
-    static constexpr int TB = 2 * LE;
-    static constexpr int W = TB + 4 * L;
-    static constexpr int CB = W + 4;
-    static constexpr int N = CB + 4 * L;
-    static constexpr int RS = N;                   // a multiple of 4
-    static constexpr int NP = LE / 2 + L * (L + 1) / 2;  // slot pairs
-    static constexpr int S2 = (NP + 31) / 32;            // slot pairs per lane
-};
-
-__host__ __device__ constexpr size_t accum_df_smem_per_warp(int L, int B, int NRP) {
-    return (size_t)B * NRP * 8 + 54 * 16 + 9 * 8 + 8 + (size_t)32 * (2 * ((L + 2) & ~1) + 8 * L + 4) * 4;
-}
-
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-// Two double-float accumulators at once (.x and .y): (H, Lo) += T * C, the
-// operations of df_acc(acc, df_mul_u(T, C)) lane for lane.
-__device__ __forceinline__ void df_acc_mul2(float2& H, float2& Lo, float4 T, float4 C) {
-    const float2 Th = make_float2(T.x, T.y), Tl = make_float2(T.z, T.w);
-    const float2 Ch = make_float2(C.x, C.y), Cl = make_float2(C.z, C.w);
-    const float2 p = __fmul2_rn(Th, Ch);
-    float2 e = __ffma2_rn(Th, Ch, neg2(p));
-    e = __ffma2_rn(Th, Cl, __ffma2_rn(Tl, Ch, e));
-    const float2 s = __fadd2_rn(H, p);
-    const float2 bb = __fadd2_rn(s, neg2(H));
-    const float2 err = __fadd2_rn(__fadd2_rn(H, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
-    Lo = __fadd2_rn(Lo, __fadd2_rn(err, e));
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+// Biased accumulators.  Two sums at a time (.x and .y), each a head H that carries
+// a bias, so that it stays more than twice as large as any term, and a tail: in
+// s = fl(H + T C) the difference H - s is then exact (Sterbenz), and one more FMA
+// returns what the rounding left.  (H, Lo) += T C with T = (Th, Tl), C = (Ch, Cl)
+// takes 6 packed operations instead of the 12 of an error-free addition to a head
+// of unknown size.
+__device__ __forceinline__ void bias_fma(float2& H, float2& Lo, float2 Th, float2 Tl, float2 Ch, float2 Cl) {
+    const float2 s = __ffma2_rn(Th, Ch, H);
+    const float2 e = __ffma2_rn(Th, Ch, __fadd2_rn(H, neg2(s)));
+    Lo = __ffma2_rn(Th, Cl, __ffma2_rn(Tl, Ch, __fadd2_rn(Lo, e)));
+    H = s;
+}
+// the same with Cl = 0
+__device__ __forceinline__ void bias_fma(float2& H, float2& Lo, float2 Th, float2 Tl, float2 Ch) {
+    const float2 s = __ffma2_rn(Th, Ch, H);
+    const float2 e = __ffma2_rn(Th, Ch, __fadd2_rn(H, neg2(s)));
+    Lo = __ffma2_rn(Tl, Ch, __fadd2_rn(Lo, e));
+    H = s;
+}
+// (H, Lo) += C
+__device__ __forceinline__ void bias_add(float2& H, float2& Lo, float2 Ch, float2 Cl) {
+    const float2 s = __fadd2_rn(H, Ch);
+    const float2 e = __fadd2_rn(__fadd2_rn(H, neg2(s)), Ch);
+    Lo = __fadd2_rn(Lo, __fadd2_rn(e, Cl));
     H = s;
 }
 
+// Forward sums.  The m = 0 sums (reals) stay in the registers of the lane that
+// evaluates the pair and are reduced over the warp once per bin.  For m >= 1 the pair goes
+// to a record in shared memory,
+//   C_m, m = 1..L:      Re.h, Im.h, Re.l, Im.l  of w (x + iy)^m
+//   T_k, k = 0..L:      h, l                     (KE values)
+// and every lane owns two sums (k0, k0 + 1; k0 even) of one m: one 128-bit load
+// gives both T, one the C (LDS returns 128 bytes per cycle whatever is broadcast, so
+// bytes per sum count: 16 here, 32 with one sum per lane).  LPG lanes hold all sums;
+// where they fit in a half, quarter ... of the warp, G groups share the chunk's pairs.
 template <int L>
-__global__ void __launch_bounds__(kDThreads) k_accum_df(ListArgs a) {
+struct DfRec {
+    __host__ __device__ static constexpr int lanes() {
+        int n = 0;
+        for (int m = 1; m <= L; ++m) n += (L - m + 2) / 2;
+        return n;
+    }
+    __host__ __device__ static constexpr int groups() {
+        int g = 1;
+        while (g < 16 && lanes() * g * 2 <= 32) g *= 2;
+        return g;
+    }
+    static constexpr int N = lanes();
+    static constexpr int G = groups();
+    static constexpr int LPG = 32 / G;
+    static constexpr int KE = (L + 1) & ~1;
+    static constexpr int TB = 4 * L;
+    // record stride (floats), an odd number of 16-byte units: conflict-free stores
+    static constexpr int RS = ((4 * L + 2 * KE) / 4 % 2) ? 4 * L + 2 * KE : 4 * L + 2 * KE + 4;
+    static constexpr int M0 = (L + 2) / 2;  // packed pairs of m = 0
+    // bias of a chunk's sums (32 / G terms of size <= 1)
+    static constexpr float kBias = 32.f / G + 8.f;
+};
+// Bias of the m = 0 sums: one term of size <= 1 per chunk and lane, flushed after 32.
+constexpr int kBiasChunks = 32;
+constexpr float kBias0 = 40.f;
+
+__host__ __device__ constexpr size_t accum_df_smem_per_warp(int RL, int RS, int NRP) {
+    return (size_t)32 * RS * 4 + 54 * 16 + 9 * 8 + 8 + (size_t)NRP * 8 + (size_t)((RL + 3) & ~3) * 4;
+}
+
+template <int L>
+__global__ void __launch_bounds__(kDThreads, L <= 8 ? 4 : 3) k_accum_df(ListArgs a) {
     using R_ = DfRec<L>;
-    constexpr int S2 = R_::S2, RS = R_::RS, NP = R_::NP;
-    constexpr int U = S2 == 1 ? 8 : 4;  // pairs per round of the accumulation
-    constexpr int NRP = Shape<L>::NRP;
+    constexpr int RS = R_::RS, G = R_::G, M0 = R_::M0, KE = R_::KE;
+    constexpr int NR = Shape<L>::NR, NRP = Shape<L>::NRP;
+    constexpr int kSteps = 32 / G, U = kSteps < 4 ? kSteps : 4;
     extern __shared__ __align__(16) unsigned char draw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int B = a.bins.nbins;
-    unsigned char* base = draw + (size_t)wid * accum_df_smem_per_warp(L, B, NRP);
-    float2* res = reinterpret_cast<float2*>(base);                          // [B][NRP] head, tail
-    float4* img = reinterpret_cast<float4*>(base + (size_t)B * NRP * 8);    // [54]
-    df* Rd = reinterpret_cast<df*>(base + (size_t)B * NRP * 8 + 54 * 16);   // [9]
-    float* rec = reinterpret_cast<float*>(base + (size_t)B * NRP * 8 + 54 * 16 + 9 * 8 + 8);  // [32][RS]
-    // this lane's slot pairs: record offsets of their T and C operands and their
-    // two slots (slot1 < 0: none, e.g. the padding slot of m = 0)
-    int offT[S2], offC[S2], slot0[S2], slot1[S2];
-#pragma unroll
-    for (int s = 0; s < S2; ++s) {
-        const int sp = lane + 32 * s;
-        offT[s] = 0;
-        offC[s] = R_::W;
-        slot0[s] = slot1[s] = -1;
-        if (sp < R_::LE / 2) {
-            offT[s] = R_::TA + 4 * sp;
-            slot0[s] = 2 * sp;
-            slot1[s] = 2 * sp + 1 <= L ? 2 * sp + 1 : -1;
-        } else if (sp < NP) {
-            int idx = sp - R_::LE / 2, m = 1;
-            while (idx >= L + 1 - m) {
-                idx -= L + 1 - m;
+    unsigned char* base = draw + (size_t)wid * accum_df_smem_per_warp(a.RL, RS, NRP);
+    float* rec = reinterpret_cast<float*>(base);                              // [32][RS]
+    float4* img = reinterpret_cast<float4*>(base + 32 * RS * 4);              // [54]
+    df* Rd = reinterpret_cast<df*>(base + 32 * RS * 4 + 54 * 16);             // [9]
+    float2* res = reinterpret_cast<float2*>(base + 32 * RS * 4 + 54 * 16 + 80);  // [NRP] one bin's sums
+    float* rowbuf = reinterpret_cast<float*>(base + 32 * RS * 4 + 54 * 16 + 80 + NRP * 8);  // [RL]
+    // this lane's order m and first k
+    const int grp = lane / R_::LPG;
+    int m = 0, k0 = 0;
+    {
+        int idx = lane % R_::LPG;
+        if (idx < R_::N) {
+            m = 1;
+            while (idx >= (L - m + 2) / 2) {
+                idx -= (L - m + 2) / 2;
                 ++m;
             }
-            offT[s] = R_::TB + 4 * idx;
-            offC[s] = R_::CB + 4 * (m - 1);
-            slot0[s] = acc_base(L, m) + 2 * idx;
-            slot1[s] = slot0[s] + 1;
+            k0 = 2 * idx;
         }
     }
+    const int offC = m > 0 ? 4 * (m - 1) : 0, offT = R_::TB + 2 * k0;
     const Grid& g = a.g;
     const df boxdf = df_from(g.boxd);  // the box side as head + tail
     const bool radial = g.radial != 0;
@@ -284,141 +308,243 @@ __global__ void __launch_bounds__(kDThreads) k_accum_df(ListArgs a) {
                 Rd[lane] = {(lane % 4 == 0) ? 1.f : 0.f, 0.f};
             }
         }
-        for (int k = lane; k < B * NRP; k += 32) res[k] = make_float2(0.f, 0.f);
+        for (int k = lane; k < a.RL; k += 32) rowbuf[k] = 0.f;
+        for (int k = lane; k < NR; k += 32) res[k] = make_float2(0.f, 0.f);
         const int cb = a.base[q] < 0 ? 0 : a.base[q];
         const int nch = a.nchunks[q];
         const int* chunks = a.chunks + (int64_t)cb * 32;
         const int* ordp = a.ord + cb;
         __syncwarp();
-        float2 accH[S2], accL[S2];
-#pragma unroll
-        for (int s = 0; s < S2; ++s) accH[s] = accL[s] = make_float2(0.f, 0.f);
-        auto flush = [&](int b) {
-#pragma unroll
-            for (int s = 0; s < S2; ++s) {
-                if (slot0[s] >= 0) {
-                    const float2 o = res[b * NRP + slot0[s]];
-                    const df v = df_add({o.x, o.y}, {accH[s].x, accL[s].x});
-                    res[b * NRP + slot0[s]] = make_float2(v.h, v.l);
-                }
-                if (slot1[s] >= 0) {
-                    const float2 o = res[b * NRP + slot1[s]];
-                    const df v = df_add({o.x, o.y}, {accH[s].y, accL[s].y});
-                    res[b * NRP + slot1[s]] = make_float2(v.h, v.l);
-                }
-                accH[s] = accL[s] = make_float2(0.f, 0.f);
-            }
+        // m = 0: packed (k, k + 1); m >= 1: this lane's sums k0 and k0 + 1 as (Re, Im)
+        // (biased: Ha .. Lb; added to SaH .. SbL after every chunk, so that the bias, which
+        // sets the rounding, stays near the sums)
+        float2 H0[M0], L0[M0], Ha, La, Hb, Lb, SaH, SaL, SbH, SbL;
+        auto clear = [&]() {
+            static_for<0, M0>([&](auto ic) {
+                H0[decltype(ic)::value] = dup(kBias0);
+                L0[decltype(ic)::value] = dup(0.f);
+            });
+            Ha = Hb = dup(R_::kBias);
+            La = Lb = SaH = SaL = SbH = SbL = dup(0.f);
         };
-        if (nch > 0) {
-            int curb = (int)((unsigned)__ldg(ordp) >> 26);
-            // entries and points of chunk i + 1 load while chunk i is evaluated
-            unsigned o_n = (unsigned)__ldg(ordp);
-            unsigned e_n = (unsigned)__ldg(chunks + (int64_t)(o_n & 0x3ffffffu) * 32 + lane);
-            float4 q_n = make_float4(0.f, 0.f, 0.f, 0.f);
-            float3 l_n = make_float3(0.f, 0.f, 0.f);
-            if (e_n != kNoPairD) load_sec(a, e_n, q_n, l_n);
-            for (int i = 0; i < nch; ++i) {
-                const unsigned o = o_n, e = e_n;
-                const float4 qv = q_n;
-                const float3 ql = l_n;
-                if (i + 1 < nch) {
-                    o_n = (unsigned)__ldg(ordp + i + 1);
-                    e_n = (unsigned)__ldg(chunks + (int64_t)(o_n & 0x3ffffffu) * 32 + lane);
-                    if (e_n != kNoPairD) load_sec(a, e_n, q_n, l_n);
-                }
-                const int b = (int)(o >> 26);
-                if (b != curb) {
-                    flush(curb);
-                    curb = b;
-                }
-                // this lane's pair -> its record (only valid pairs are read back)
-                float4* my = reinterpret_cast<float4*>(rec + lane * RS);
-                if (e != kNoPairD) {
-                    const int code = (int)(e >> kIdxBits);
-                    const float4 hh = img[code], tt = img[27 + code];
-                    const df dx = sep(qv.x, ql.x, hh.x, tt.x), dy = sep(qv.y, ql.y, hh.y, tt.y),
-                             dz = sep(qv.z, ql.z, hh.z, tt.z);
-                    df ux, uy, uz, rinv;
-                    unit_df(dx, dy, dz, Rd, radial, ux, uy, uz, rinv);
-                    const float w = qv.w;
-                    df T[R_::LE];
-                    T[0] = {1.f, 0.f};
-                    if constexpr (L >= 1) T[1] = uz;
-                    const df z2 = {2.f * uz.h, 2.f * uz.l};
+        clear();
+        auto fold1 = [&](float2& SH, float2& SL, float2& H, float2& Lo) {
+            const float2 x = __fadd2_rn(H, dup(-R_::kBias));  // exact
+            const float2 s = __fadd2_rn(SH, x), bb = __fadd2_rn(s, neg2(SH));
+            const float2 er = __fadd2_rn(__fadd2_rn(SH, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(x, neg2(bb)));
+            SL = __fadd2_rn(SL, __fadd2_rn(er, Lo));
+            SH = s;
+            H = dup(R_::kBias);
+            Lo = dup(0.f);
+        };
+        // |w| <= cap (a power of two fixed by the first weights of a bin; a larger one
+        // flushes the sums): the sums take w / cap
+        unsigned cap = 0u;
+        int cnt = 0;
+        float inv = 1.f, scale = 1.f;
+        // the sums, times cap, into res
+        auto flush = [&]() {
+            if (m > 0 || G > 1) {
+                float h[4] = {SaH.x, SaH.y, SbH.x, SbH.y};
+                float l[4] = {SaL.x, SaL.y, SbL.x, SbL.y};
 #pragma unroll
-                    for (int k = 2; k <= L; ++k) T[k] = df_add(df_mul(z2, T[k - 1]), df_neg(T[k - 2]));
+                for (int o = 16; o >= R_::LPG; o >>= 1)
 #pragma unroll
-                    for (int k = L + 1; k < R_::LE; ++k) T[k] = {0.f, 0.f};
-#pragma unroll
-                    for (int k = 0; k < R_::LE; k += 2)
-                        my[(R_::TA >> 2) + (k >> 1)] = make_float4(T[k].h, T[k + 1].h, T[k].l, T[k + 1].l);
-#pragma unroll
-                    for (int k = 0; k < L; ++k) my[(R_::TB >> 2) + k] = make_float4(T[k].h, T[k].h, T[k].l, T[k].l);
-                    my[R_::W >> 2] = make_float4(w, w, 0.f, 0.f);
-                    if constexpr (L >= 1) {
-                        df cr = df_mulf(ux, w), ci = df_mulf(uy, w);
-#pragma unroll
-                        for (int m = 1; m <= L; ++m) {
-                            my[(R_::CB >> 2) + (m - 1)] = make_float4(cr.h, ci.h, cr.l, ci.l);
-                            if (m < L) {
-                                df nr, ni;
-                                df_cmul(cr, ci, ux, uy, nr, ni);
-                                cr = nr;
-                                ci = ni;
-                            }
-                        }
+                    for (int i = 0; i < 4; ++i) {
+                        const float gh = __shfl_xor_sync(kFull, h[i], o), gl = __shfl_xor_sync(kFull, l[i], o);
+                        const df t = two_sum(h[i], gh);
+                        h[i] = t.h;
+                        l[i] = __fadd_rn(__fadd_rn(l[i], gl), t.l);
                     }
+                if (m > 0 && grp == 0) {
+                    const int s0 = acc_base(L, m) + 2 * k0, n = k0 + 1 <= L - m ? 4 : 2;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (i < n) {
+                            const float2 o = res[s0 + i];
+                            const df v = df_add({o.x, o.y}, fast_two_sum(h[i] * scale, l[i] * scale));
+                            res[s0 + i] = make_float2(v.h, v.l);
+                        }
                 }
+            }
+            // m = 0 over the warp by recursive halving
+            float h[L + 1], l[L + 1];
+            static_for<0, L + 1>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                h[k] = ((k & 1) ? H0[k / 2].y : H0[k / 2].x) - kBias0;
+                l[k] = (k & 1) ? L0[k / 2].y : L0[k / 2].x;
+            });
+            int b0 = 0, size = L + 1;
+            static_for<0, 5>([&](auto rc) {
+                constexpr int r = decltype(rc)::value;
+                constexpr int S = bf_size(L + 1, r);
+                constexpr int hf = (S + 1) / 2;
+                constexpr int o = 16 >> r;
+                const bool hi = (lane & o) != 0;
+                static_for<0, hf>([&](auto ic) {
+                    constexpr int i = decltype(ic)::value;
+                    float uh = 0.f, ul = 0.f;
+                    if constexpr (i + hf < S) {
+                        uh = h[i + hf];
+                        ul = l[i + hf];
+                    }
+                    const float kh = hi ? uh : h[i], kl = hi ? ul : l[i];
+                    const float gh = __shfl_xor_sync(kFull, hi ? h[i] : uh, o);
+                    const float gl = __shfl_xor_sync(kFull, hi ? l[i] : ul, o);
+                    const df t = two_sum(kh, gh);
+                    h[i] = t.h;
+                    l[i] = __fadd_rn(__fadd_rn(kl, gl), t.l);
+                });
+                if (hi) {
+                    b0 += hf;
+                    size -= hf;
+                } else {
+                    size = size < hf ? size : hf;
+                }
+            });
+            if (size > 0) {  // one slot per lane after five halvings of at most 11
+                const float2 o = res[b0];
+                const df v = df_add({o.x, o.y}, fast_two_sum(h[0] * scale, l[0] * scale));
+                res[b0] = make_float2(v.h, v.l);
+            }
+            clear();
+            cnt = 0;
+        };
+        // list words three chunks ahead, entries two, points one
+        auto word = [&](int i) { return (unsigned)__ldg(ordp + (i < nch ? i : nch - 1)); };
+        auto entry = [&](unsigned o) { return (unsigned)__ldg(chunks + (int64_t)(o & 0x3ffffffu) * 32 + lane); };
+        unsigned e = kNoPairD, en = kNoPairD, o0 = 0u, o1 = 0u, o2 = 0u;
+        float4 qv = make_float4(0.f, 0.f, 0.f, 0.f);
+        float3 ql = make_float3(0.f, 0.f, 0.f);
+        if (nch > 0) {
+            o0 = word(0);
+            o1 = word(1);
+            o2 = word(2);
+            e = entry(o0);
+            en = entry(o1);
+            if (e != kNoPairD) load_sec(a, e, qv, ql);
+        }
+        for (int i = 0; i < nch; ++i) {
+            float4 qn = make_float4(0.f, 0.f, 0.f, 0.f);
+            float3 ln = make_float3(0.f, 0.f, 0.f);
+            if (en != kNoPairD) load_sec(a, en, qn, ln);
+            const unsigned en2 = entry(o2), o3 = word(i + 3);
+            const bool v = e != kNoPairD;
+            const unsigned wm = __reduce_max_sync(kFull, v ? __float_as_uint(fabsf(qv.w)) : 0u);
+            const int nv = __popc(__ballot_sync(kFull, v));  // the chunk's pairs, its first lanes
+            if (wm > cap || cnt == kBiasChunks) {
+                if (cnt > 0) flush();
+                if (wm > cap) {
+                    const unsigned ex = min((wm >> 23) + 1u, 253u);
+                    cap = ex << 23;
+                    scale = __uint_as_float(cap);
+                    inv = __uint_as_float((254u - ex) << 23);
+                }
+            }
+            ++cnt;
+            {
+                // this lane's pair -> its record; a padding lane takes a unit separation
+                // and weight 0
+                const int code = (int)min(e >> kIdxBits, 26u);
+                const float4 hh = img[code], tt = img[27 + code];
+                df dx = sep(qv.x, ql.x, hh.x, tt.x), dy = sep(qv.y, ql.y, hh.y, tt.y),
+                   dz = sep(qv.z, ql.z, hh.z, tt.z);
+                if (!v) {
+                    dx = {1.f, 0.f};
+                    dy = dz = {0.f, 0.f};
+                }
+                df ux, uy, uz, rinv;
+                unit_df(dx, dy, dz, Rd, radial, ux, uy, uz, rinv);
+                const float w = v ? qv.w * inv : 0.f;
+                float4* my = reinterpret_cast<float4*>(rec + lane * RS);
+                df T[2 * M0];
+                T[0] = {1.f, 0.f};
+                T[1] = uz;
+                const df z2 = {2.f * uz.h, 2.f * uz.l};
+                static_for<2, 2 * M0>([&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    if constexpr (k <= L)
+                        T[k] = df_add(df_mul(z2, T[k - 1]), df_neg(T[k - 2]));
+                    else
+                        T[k] = {0.f, 0.f};
+                });
+                static_for<0, M0>([&](auto ic) {
+                    constexpr int k = 2 * decltype(ic)::value;
+                    bias_fma(H0[k / 2], L0[k / 2], make_float2(T[k].h, T[k + 1].h), make_float2(T[k].l, T[k + 1].l),
+                             dup(w));
+                    if constexpr (k < KE) my[(R_::TB + 2 * k) / 4] = make_float4(T[k].h, T[k].l, T[k + 1].h, T[k + 1].l);
+                });
+                if constexpr (L >= 1) {
+                    df cr = df_mulf(ux, w), ci = df_mulf(uy, w);
+                    static_for<1, L + 1>([&](auto mc) {
+                        constexpr int mm = decltype(mc)::value;
+                        my[mm - 1] = make_float4(cr.h, ci.h, cr.l, ci.l);
+                        if constexpr (mm < L) {
+                            df nr, ni;
+                            df_cmul(cr, ci, ux, uy, nr, ni);
+                            cr = nr;
+                            ci = ni;
+                        }
+                    });
+                }
+            }
+            if constexpr (L >= 1) {
                 __syncwarp();
-                // every valid pair of the chunk into this lane's slot pairs, U
-                // pairs per round (loads and products of later pairs overlap the
-                // sums of earlier ones; the sums keep the pairs' order)
-                unsigned valid = __ballot_sync(kFull, e != kNoPairD);
-                while (valid) {
-                    int t[U];
+                // the chunk's pairs into this lane's two sums, G pairs per step (the
+                // records past the last pair hold weight 0)
+                const float* rt = rec + grp * RS;
+                const int steps = (nv + G - 1) / G;
+                for (int t = 0; t < steps; t += U, rt += U * G * RS) {
+                    float4 T4[U], C4[U];
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        t[u] = -1;
-                        if (valid) {
-                            t[u] = __ffs(valid) - 1;
-                            valid &= valid - 1;
-                        }
+                        C4[u] = *reinterpret_cast<const float4*>(rt + u * G * RS + offC);
+                        T4[u] = *reinterpret_cast<const float4*>(rt + u * G * RS + offT);
                     }
 #pragma unroll
-                    for (int s = 0; s < S2; ++s) {
-                        if (lane + 32 * s < NP) {
-                            float4 T4[U], C4[U];
-#pragma unroll
-                            for (int u = 0; u < U; ++u) {
-                                if (t[u] >= 0) {
-                                    const float* rt = rec + t[u] * RS;
-                                    T4[u] = *reinterpret_cast<const float4*>(rt + offT[s]);
-                                    C4[u] = *reinterpret_cast<const float4*>(rt + offC[s]);
-                                }
-                            }
-#pragma unroll
-                            for (int u = 0; u < U; ++u)
-                                if (t[u] >= 0) df_acc_mul2(accH[s], accL[s], T4[u], C4[u]);
-                        }
+                    for (int u = 0; u < U; ++u) {
+                        const float2 Ch = make_float2(C4[u].x, C4[u].y), Cl = make_float2(C4[u].z, C4[u].w);
+                        bias_fma(Ha, La, dup(T4[u].x), dup(T4[u].y), Ch, Cl);
+                        bias_fma(Hb, Lb, dup(T4[u].z), dup(T4[u].w), Ch, Cl);
                     }
                 }
+                fold1(SaH, SaL, Ha, La);
+                fold1(SbH, SbL, Hb, Lb);
                 __syncwarp();
             }
-            flush(curb);
+            if (i + 1 == nch || (o0 ^ o1) >> 26) {  // the bin's last chunk: its columns of the row
+                flush();
+                cap = 0u;
+                __syncwarp();
+                const int b = (int)(o0 >> 26);
+                for (int sl = lane; sl < NR; sl += 32) {
+                    const int col = __ldg(&a.slotconv[sl].x) + b;
+                    const int4 cv = __ldg(a.colconv + col);
+                    const float2* cf = a.colcoefdf + cv.w;
+                    const float2* rs = res + (cv.x - b * NRP);
+                    df v2 = {0.f, 0.f};
+                    for (int k = 0; k < cv.z; ++k) {
+                        const float2 c = __ldg(cf + k), r = rs[cv.y * k];
+                        v2 = df_add(v2, df_mul({c.x, c.y}, {r.x, r.y}));
+                    }
+                    rowbuf[col] = __fadd_rn(v2.h, v2.l);
+                }
+                __syncwarp();
+                for (int k = lane; k < NR; k += 32) res[k] = make_float2(0.f, 0.f);
+                __syncwarp();
+            }
+            e = en;
+            qv = qn;
+            ql = ln;
+            en = en2;
+            o0 = o1;
+            o1 = o2;
+            o2 = o3;
         }
         __syncwarp();
         const int row = a.chunked ? q - a.q0 : a.orig[p];
         float* Arow = a.A + (int64_t)row * a.RLP;
-        for (int col = lane; col < a.RL; col += 32) {
-            const int4 cv = __ldg(a.colconv + col);
-            const float2* cf = a.colcoefdf + cv.w;
-            df v = {0.f, 0.f};
-            for (int k = 0; k < cv.z; ++k) {
-                const float2 c = __ldg(cf + k), r = res[cv.x + cv.y * k];
-                v = df_add(v, df_mul({c.x, c.y}, {r.x, r.y}));
-            }
-            Arow[col] = __fadd_rn(v.h, v.l);
-        }
+        for (int col = lane; col < a.RL; col += 32) Arow[col] = rowbuf[col];
         if (lane == 0) a.wrow[row] = P0.w;
         __syncwarp();
     }
@@ -428,6 +554,21 @@ __global__ void __launch_bounds__(kDThreads) k_accum_df(ListArgs a) {
 __host__ __device__ constexpr size_t adj_df_smem_per_warp(int B, int NRP) {
     return (size_t)B * NRP * 8 + 54 * 16;
 }
+// Two double-float accumulators at once (.x and .y): (H, Lo) += T * C, the
+// operations of df_acc(acc, df_mul_u(T, C)) lane for lane.
+__device__ __forceinline__ void df_acc_mul2(float2& H, float2& Lo, float4 T, float4 C) {
+    const float2 Th = make_float2(T.x, T.y), Tl = make_float2(T.z, T.w);
+    const float2 Ch = make_float2(C.x, C.y), Cl = make_float2(C.z, C.w);
+    const float2 p = __fmul2_rn(Th, Ch);
+    float2 e = __ffma2_rn(Th, Ch, neg2(p));
+    e = __ffma2_rn(Th, Cl, __ffma2_rn(Tl, Ch, e));
+    const float2 s = __fadd2_rn(H, p);
+    const float2 bb = __fadd2_rn(s, neg2(H));
+    const float2 err = __fadd2_rn(__fadd2_rn(H, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
+    Lo = __fadd2_rn(Lo, __fadd2_rn(err, e));
+    H = s;
+}
+
 // a double-float value (head, tail) as the duplicated operand (h, h, t, t) of a
 // packed product
 __device__ __forceinline__ float4 dup2(float2 v) { return make_float4(v.x, v.x, v.y, v.y); }
@@ -608,7 +749,7 @@ int launch_persistent(K kern, const ListArgs& a, size_t smem, int nsm, cudaStrea
 
 template <int L>
 int launch_accum_df_t(const ListArgs& a, int nsm, cudaStream_t st) {
-    return launch_persistent(k_accum_df<L>, a, accum_df_smem_per_warp(L, a.bins.nbins, Shape<L>::NRP) * kDWarps,
+    return launch_persistent(k_accum_df<L>, a, accum_df_smem_per_warp(a.RL, DfRec<L>::RS, Shape<L>::NRP) * kDWarps,
                              nsm, st);
 }
 template <int L>
