@@ -551,37 +551,33 @@ __global__ void __launch_bounds__(kDThreads, L <= 8 ? 4 : 3) k_accum_df(ListArgs
 }
 
 // ---- adjoint ----------------------------------------------------------------
-__host__ __device__ constexpr size_t adj_df_smem_per_warp(int B, int NRP) {
-    return (size_t)B * NRP * 8 + 54 * 16;
+// Coefficients of one bin in shared memory (floats): for m >= 1 the pair (m, k) as
+// Re.h, Im.h, Re.l, Im.l at 4 (cidx(m) + k), so that one broadcast load gives both
+// operands of a packed operation; then G_{0,k} as h, l.
+template <int L>
+struct AdjG {
+    static constexpr int NC = L * (L + 1) / 2;
+    static constexpr int Z = 4 * NC;
+    static constexpr int N = (Z + 2 * (L + 1) + 3) & ~3;  // floats per bin
+    __host__ __device__ static constexpr int cidx(int m) { return (m - 1) * (L + 1) - (m - 1) * m / 2; }
+};
+__host__ __device__ constexpr size_t adj_df_smem_per_warp(int B, int N) {
+    return (size_t)B * N * 4 + 54 * 16 + (size_t)((B + 1) & ~1) * 8;
 }
-// Two double-float accumulators at once (.x and .y): (H, Lo) += T * C, the
-// operations of df_acc(acc, df_mul_u(T, C)) lane for lane.
-__device__ __forceinline__ void df_acc_mul2(float2& H, float2& Lo, float4 T, float4 C) {
-    const float2 Th = make_float2(T.x, T.y), Tl = make_float2(T.z, T.w);
-    const float2 Ch = make_float2(C.x, C.y), Cl = make_float2(C.z, C.w);
-    const float2 p = __fmul2_rn(Th, Ch);
-    float2 e = __ffma2_rn(Th, Ch, neg2(p));
-    e = __ffma2_rn(Th, Cl, __ffma2_rn(Tl, Ch, e));
-    const float2 s = __fadd2_rn(H, p);
-    const float2 bb = __fadd2_rn(s, neg2(H));
-    const float2 err = __fadd2_rn(__fadd2_rn(H, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
-    Lo = __fadd2_rn(Lo, __fadd2_rn(err, e));
-    H = s;
-}
-
-// a double-float value (head, tail) as the duplicated operand (h, h, t, t) of a
-// packed product
-__device__ __forceinline__ float4 dup2(float2 v) { return make_float4(v.x, v.x, v.y, v.y); }
+// the value of a biased sum as head (exact) and tail
+__device__ __forceinline__ float2 unbias(float2 H, float b) { return __fadd2_rn(H, dup(-b)); }
 
 template <int L>
-__global__ void __launch_bounds__(kDThreads) k_adj_df(ListArgs a) {
-    constexpr int NR = Shape<L>::NR, NRP = Shape<L>::NRP;
+__global__ void __launch_bounds__(kDThreads, L <= 6 ? 4 : (L <= 8 ? 3 : 2)) k_adj_df(ListArgs a) {
+    constexpr int NR = Shape<L>::NR;
+    using G_ = AdjG<L>;
     extern __shared__ __align__(16) unsigned char draw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int B = a.bins.nbins;
-    unsigned char* base = draw + (size_t)wid * adj_df_smem_per_warp(B, NRP);
-    float2* G = reinterpret_cast<float2*>(base);                           // [B][NRP] head, tail
-    float4* img = reinterpret_cast<float4*>(base + (size_t)B * NRP * 8);   // [54]
+    unsigned char* base = draw + (size_t)wid * adj_df_smem_per_warp(B, G_::N);
+    float* G = reinterpret_cast<float*>(base);                                  // [B][N]
+    float4* img = reinterpret_cast<float4*>(base + (size_t)B * G_::N * 4);      // [54]
+    float2* bias = reinterpret_cast<float2*>(base + (size_t)B * G_::N * 4 + 54 * 16);  // [B]
     const Grid& g = a.g;
     const df boxdf = df_from(g.boxd);  // the box side as head + tail
     const int qa = a.qrange ? a.qrange[0] : a.qa, qb = a.qrange ? a.qrange[1] : a.qb;
@@ -595,16 +591,47 @@ __global__ void __launch_bounds__(kDThreads) k_adj_df(ListArgs a) {
         if (lane < 27) image_df(img, lane, P0, a.pts64, p, g.boxd, boxdf);
         const int row = a.orig[p];
         const float2* Vrow = a.Vdf + (int64_t)(a.chunked ? q - a.q0 : row) * a.RLP;
-        for (int idx = lane; idx < B * NR; idx += 32) {
-            const int b = idx / NR, sl = idx - b * NR;
-            const int4 cv = __ldg(a.slotconv + sl);
-            df v = {0.f, 0.f};
-            for (int t = 0; t < cv.z; ++t) {
-                const float2 c = __ldg(a.slotcoefdf + cv.w + t), x = Vrow[cv.x + b + t * cv.y];
-                v = df_add(v, df_mul({c.x, c.y}, {x.x, x.y}));
+        for (int b = 0; b < B; ++b) {
+            // this bin's coefficients, and bounds of its sums: s1 over |G|, s2 over
+            // k^2 |G| (|T_k| <= 1, |T_k'| <= k^2)
+            float s1 = 0.f, s2 = 0.f;
+            for (int sl = lane; sl < NR; sl += 32) {
+                int m = 0, k = sl, part = 0;
+                if (sl > L) {
+                    int r = sl - (L + 1);
+                    m = 1;
+                    while (r >= 2 * (L + 1 - m)) {
+                        r -= 2 * (L + 1 - m);
+                        ++m;
+                    }
+                    k = r >> 1;
+                    part = r & 1;
+                }
+                const int4 cv = __ldg(a.slotconv + sl);
+                df v = {0.f, 0.f};
+                for (int t = 0; t < cv.z; ++t) {
+                    const float2 c = __ldg(a.slotcoefdf + cv.w + t), x = Vrow[cv.x + b + t * cv.y];
+                    v = df_add(v, df_mul({c.x, c.y}, {x.x, x.y}));
+                }
+                const df gv = df_mulf(v, P0.w);
+                float* Gb = G + b * G_::N;
+                if (m == 0) {
+                    Gb[G_::Z + 2 * k] = gv.h;
+                    Gb[G_::Z + 2 * k + 1] = gv.l;
+                } else {
+                    Gb[4 * (G_::cidx(m) + k) + part] = gv.h;
+                    Gb[4 * (G_::cidx(m) + k) + 2 + part] = gv.l;
+                }
+                s1 += fabsf(gv.h);
+                s2 = fmaf((float)(k * k), fabsf(gv.h), s2);
             }
-            const df gv = df_mulf(v, P0.w);
-            G[b * NRP + sl] = make_float2(gv.h, gv.l);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                s1 += __shfl_xor_sync(kFull, s1, o);
+                s2 += __shfl_xor_sync(kFull, s2, o);
+            }
+            // biases: three times the bound keeps every head above twice any term
+            if (lane == 0) bias[b] = make_float2(3.f * s1, 3.f * s2);
         }
         const int cb = a.base[q] < 0 ? 0 : a.base[q];
         const int nch = a.nchunks[q];
@@ -612,109 +639,143 @@ __global__ void __launch_bounds__(kDThreads) k_adj_df(ListArgs a) {
         const int* ordp = a.ord + cb;
         __syncwarp();
         df pix = {0.f, 0.f}, piy = {0.f, 0.f}, piz = {0.f, 0.f};  // the primary's share (this lane)
-        unsigned o_n = nch > 0 ? (unsigned)__ldg(ordp) : 0u;
-        unsigned e_n = nch > 0 ? (unsigned)__ldg(chunks + (int64_t)(o_n & 0x3ffffffu) * 32 + lane) : kNoPairD;
-        float4 q_n = make_float4(0.f, 0.f, 0.f, 0.f);
-        float3 l_n = make_float3(0.f, 0.f, 0.f);
-        if (e_n != kNoPairD) load_sec(a, e_n, q_n, l_n);
+        // list words three chunks ahead, entries two, points one
+        auto word = [&](int i) { return (unsigned)__ldg(ordp + (i < nch ? i : nch - 1)); };
+        auto entry = [&](unsigned o) { return (unsigned)__ldg(chunks + (int64_t)(o & 0x3ffffffu) * 32 + lane); };
+        unsigned e = kNoPairD, en = kNoPairD, o0 = 0u, o1 = 0u, o2 = 0u;
+        float4 qv = make_float4(0.f, 0.f, 0.f, 0.f);
+        float3 ql = make_float3(0.f, 0.f, 0.f);
+        if (nch > 0) {
+            o0 = word(0);
+            o1 = word(1);
+            o2 = word(2);
+            e = entry(o0);
+            en = entry(o1);
+            if (e != kNoPairD) load_sec(a, e, qv, ql);
+        }
         for (int i = 0; i < nch; ++i) {
-            const unsigned o = o_n, e = e_n;
-            const float4 qv = q_n;
-            const float3 ql = l_n;
-            if (i + 1 < nch) {
-                o_n = (unsigned)__ldg(ordp + i + 1);
-                e_n = (unsigned)__ldg(chunks + (int64_t)(o_n & 0x3ffffffu) * 32 + lane);
-                if (e_n != kNoPairD) load_sec(a, e_n, q_n, l_n);
-            }
-            if (e == kNoPairD) continue;
-            const int b = (int)(o >> 26);
-            const float2* Gb = G + b * NRP;
-            const int code = (int)(e >> kIdxBits);
-            const float4 hh = img[code], tt = img[27 + code];
-            const df dx = sep(qv.x, ql.x, hh.x, tt.x), dy = sep(qv.y, ql.y, hh.y, tt.y), dz = sep(qv.z, ql.z, hh.z, tt.z);
-            df ux, uy, z, rinv;
-            unit_df(dx, dy, dz, nullptr, false, ux, uy, z, rinv);
-            // T_k(z) and T_k'(z) = k U_{k-1}(z)
-            df T[L + 1], D[L + 1];
-            T[0] = {1.f, 0.f};
-            D[0] = {0.f, 0.f};
-            if constexpr (L >= 1) {
-                T[1] = z;
-                D[1] = {1.f, 0.f};
-                const df z2 = {2.f * z.h, 2.f * z.l};
-                df u0 = {1.f, 0.f}, u1 = z2;  // U_0, U_1
-                static_for<2, L + 1>([&](auto kc) {
-                    constexpr int k = decltype(kc)::value;
-                    T[k] = df_add(df_mul(z2, T[k - 1]), df_neg(T[k - 2]));
-                    D[k] = df_mulf(u1, (float)k);
-                    const df u2 = df_add(df_mul(z2, u1), df_neg(u0));
-                    u0 = u1;
-                    u1 = u2;
-                });
-            }
-            // (T_k, T_k') side by side: the second operand of the packed products
-            float4 TD[L + 1];
-            static_for<0, L + 1>([&](auto kc) {
-                constexpr int k = decltype(kc)::value;
-                TD[k] = make_float4(T[k].h, D[k].h, T[k].l, D[k].l);
-            });
-            // (F, Fz) in one packed double-float accumulator (.x = F, .y = Fz), and per
-            // m the pairs (gmr, gzr) and (gmi, gzi): every component takes the
-            // operations and order of its own scalar sum
-            float2 FH = make_float2(0.f, 0.f), FL = make_float2(0.f, 0.f);
-            df Fx = {0.f, 0.f}, Fy = {0.f, 0.f};
-            static_for<0, L + 1>([&](auto kc) {
-                constexpr int k = decltype(kc)::value;
-                df_acc_mul2(FH, FL, dup2(Gb[k]), TD[k]);
-            });
-            df pr = {1.f, 0.f}, pim = {0.f, 0.f};  // (x + iy)^(m-1)
-            static_for<1, L + 1>([&](auto mc) {
-                constexpr int m = decltype(mc)::value;
-                constexpr int b0 = acc_base(L, m);
-                float2 RH = make_float2(0.f, 0.f), RL = make_float2(0.f, 0.f);  // (gmr, gzr)
-                float2 IH = make_float2(0.f, 0.f), IL = make_float2(0.f, 0.f);  // (gmi, gzi)
-                static_for<0, L - m + 1>([&](auto kc) {
-                    constexpr int k = decltype(kc)::value;
-                    df_acc_mul2(RH, RL, dup2(Gb[b0 + 2 * k]), TD[k]);
-                    df_acc_mul2(IH, IL, dup2(Gb[b0 + 2 * k + 1]), TD[k]);
-                });
-                df ur, ui;  // (x + iy)^m
-                if constexpr (m == 1) {
-                    ur = ux;
-                    ui = uy;
-                } else {
-                    df_cmul(pr, pim, ux, uy, ur, ui);
+            float4 qn = make_float4(0.f, 0.f, 0.f, 0.f);
+            float3 ln = make_float3(0.f, 0.f, 0.f);
+            if (en != kNoPairD) load_sec(a, en, qn, ln);
+            const unsigned en2 = entry(o2), o3 = word(i + 3);
+            if (e != kNoPairD) {
+                const int b = (int)(o0 >> 26);
+                const float* Gb = G + b * G_::N;
+                const float B1 = bias[b].x, B2 = bias[b].y, BF = (float)(L > 0 ? L : 1) * B1;
+                const int jj = __ldg(a.orig + (e & kIdxMask));
+                const int code = (int)(e >> kIdxBits);
+                const float4 hh = img[code], tt = img[27 + code];
+                const df dx = sep(qv.x, ql.x, hh.x, tt.x), dy = sep(qv.y, ql.y, hh.y, tt.y),
+                         dz = sep(qv.z, ql.z, hh.z, tt.z);
+                df ux, uy, z, rinv;
+                unit_df(dx, dy, dz, nullptr, false, ux, uy, z, rinv);
+                // T_k(z) and T_k'(z) = k U_{k-1}(z), heads and tails
+                df T[L + 1], D[L + 1];
+                T[0] = {1.f, 0.f};
+                D[0] = {0.f, 0.f};
+                if constexpr (L >= 1) {
+                    T[1] = z;
+                    D[1] = {1.f, 0.f};
+                    const df z2 = {2.f * z.h, 2.f * z.l};
+                    df u0 = {1.f, 0.f}, u1 = z2;  // U_0, U_1
+                    static_for<2, L + 1>([&](auto kc) {
+                        constexpr int k = decltype(kc)::value;
+                        T[k] = df_add(df_mul(z2, T[k - 1]), df_neg(T[k - 2]));
+                        D[k] = df_mulf(u1, (float)k);
+                        if constexpr (k < L) {
+                            const df u2 = df_add(df_mul(z2, u1), df_neg(u0));
+                            u0 = u1;
+                            u1 = u2;
+                        }
+                    });
                 }
-                // F += Re(conj(gm) u^m), Fz likewise with gz, and the derivatives of
-                // u^m: d/dx = m u^(m-1), d/dy = i m u^(m-1)
-                df_acc_mul2(FH, FL, make_float4(RH.x, RH.y, RL.x, RL.y), make_float4(ur.h, ur.h, ur.l, ur.l));
-                df_acc_mul2(FH, FL, make_float4(IH.x, IH.y, IL.x, IL.y), make_float4(ui.h, ui.h, ui.l, ui.l));
-                const df gmr = {RH.x, RL.x}, gmi = {IH.x, IL.x};
-                const df ax = df_add(df_mul_u(gmr, pr), df_mul_u(gmi, pim));
-                const df ay = df_add(df_mul_u(gmi, pr), df_neg(df_mul_u(gmr, pim)));
-                df_acc(Fx, df_mulf(ax, (float)m));
-                df_acc(Fy, df_mulf(ay, (float)m));
-                pr = ur;
-                pim = ui;
-            });
-            const df F = {FH.x, FL.x}, Fz = {FH.y, FL.y};
-            // tangential gradient: (2 w_j / r) (grad F - (grad F . u) u), formed in
-            // double-float and rounded once: a per-pair relative error of an FP32
-            // ulp is not amplified by the sums over pairs
-            const df gdr = df_add(df_add(df_mul(Fx, ux), df_mul(Fy, uy)), df_mul(Fz, z));
-            const float tx = df_add(Fx, df_neg(df_mul(gdr, ux))).h;
-            const float ty = df_add(Fy, df_neg(df_mul(gdr, uy))).h;
-            const float tz = df_add(Fz, df_neg(df_mul(gdr, z))).h;
-            const float sc = __fmul_rn(2.f * qv.w, __fadd_rn(rinv.h, rinv.l));
-            const float gx = __fmul_rn(sc, tx), gy = __fmul_rn(sc, ty), gz3 = __fmul_rn(sc, tz);
-            const int jj = __ldg(a.orig + (e & kIdxMask));
-            atomicAdd(a.dw + jj, f2d_exact(__fmul_rn(2.f, __fadd_rn(F.h, F.l))));
-            atomicAdd(a.dpos + 3 * (int64_t)jj, f2d_exact(gx));
-            atomicAdd(a.dpos + 3 * (int64_t)jj + 1, f2d_exact(gy));
-            atomicAdd(a.dpos + 3 * (int64_t)jj + 2, f2d_exact(gz3));
-            df_acc(pix, {gx, 0.f});
-            df_acc(piy, {gy, 0.f});
-            df_acc(piz, {gz3, 0.f});
+                // m = 0: (F, Fz) += G_k (T_k, T_k')
+                float2 FH = make_float2(B1, B2), FL = dup(0.f);
+                static_for<0, L + 1>([&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    const float2 gk = *reinterpret_cast<const float2*>(Gb + G_::Z + 2 * k);
+                    bias_fma(FH, FL, dup(gk.x), dup(gk.y), make_float2(T[k].h, D[k].h), make_float2(T[k].l, D[k].l));
+                });
+                // powers of u = x + iy
+                df pr[L + 1], pi[L + 1];
+                pr[0] = {1.f, 0.f};
+                pi[0] = {0.f, 0.f};
+                if constexpr (L >= 2) {
+                    pr[1] = ux;
+                    pi[1] = uy;
+                    static_for<2, L>([&](auto mc) {
+                        constexpr int m = decltype(mc)::value;
+                        df_cmul(pr[m - 1], pi[m - 1], ux, uy, pr[m], pi[m]);
+                    });
+                }
+                // With g_m = sum_k G_{m,k} T_k, h_m likewise with T_k', as (Re, Im) pairs, and
+                // p = u^{m-1}: conj(g_m) p = a_m - i b_m.  SA sums (a, b), SZ the same of h, and
+                // SF the partial sums of SA as m descends, which is sum m (a_m, b_m); so
+                //   F  = F_0 + SA.x x + SA.y y,  dF/dx = SF.x, dF/dy = SF.y,
+                //   dF/dz = Fz_0 + SZ.x x + SZ.y y.
+                float2 SAH = dup(B1), SAL = dup(0.f), SZH = dup(B2), SZL = dup(0.f), SFH = dup(BF), SFL = dup(0.f);
+                static_for<0, L>([&](auto jc) {
+                    constexpr int m = L - decltype(jc)::value;
+                    float2 gH = dup(B1), gL = dup(0.f), hH = dup(B2), hL = dup(0.f);
+                    static_for<0, L - m + 1>([&](auto kc) {
+                        constexpr int k = decltype(kc)::value;
+                        const float4 gg = *reinterpret_cast<const float4*>(Gb + 4 * (G_::cidx(m) + k));
+                        const float2 Gh = make_float2(gg.x, gg.y), Gl = make_float2(gg.z, gg.w);
+                        if constexpr (k == 0)
+                            bias_add(gH, gL, Gh, Gl);
+                        else
+                            bias_fma(gH, gL, dup(T[k].h), dup(T[k].l), Gh, Gl);
+                        if constexpr (k == 1)
+                            bias_add(hH, hL, Gh, Gl);
+                        else if constexpr (k > 1)
+                            bias_fma(hH, hL, dup(D[k].h), dup(D[k].l), Gh, Gl);
+                    });
+                    const float2 gh = unbias(gH, B1), zh = unbias(hH, B2);
+                    if constexpr (m == 1) {  // p = 1
+                        bias_add(SAH, SAL, gh, gL);
+                        bias_add(SZH, SZL, zh, hL);
+                    } else {
+                        const float2 prh = dup(pr[m - 1].h), prl = dup(pr[m - 1].l);
+                        const float2 pih = dup(pi[m - 1].h), pil = dup(pi[m - 1].l);
+                        bias_fma(SAH, SAL, prh, prl, gh, gL);
+                        bias_fma(SAH, SAL, pih, pil, make_float2(gh.y, -gh.x), make_float2(gL.y, -gL.x));
+                        if constexpr (L - m >= 1) {  // (h_L = 0)
+                            bias_fma(SZH, SZL, prh, prl, zh, hL);
+                            bias_fma(SZH, SZL, pih, pil, make_float2(zh.y, -zh.x), make_float2(hL.y, -hL.x));
+                        }
+                    }
+                    bias_add(SFH, SFL, unbias(SAH, B1), SAL);
+                });
+                const float2 sa = unbias(SAH, B1), sz = unbias(SZH, B2), sf = unbias(SFH, BF);
+                const df F0 = fast_two_sum(FH.x - B1, FL.x), Fz0 = fast_two_sum(FH.y - B2, FL.y);
+                const df ax = {sa.x, SAL.x}, ay = {sa.y, SAL.y}, zx = {sz.x, SZL.x}, zy = {sz.y, SZL.y};
+                const df F = df_add(F0, df_add(df_mul_u(ax, ux), df_mul_u(ay, uy)));
+                const df Fz = df_add(Fz0, df_add(df_mul_u(zx, ux), df_mul_u(zy, uy)));
+                const df Fx = two_sum(sf.x, SFL.x), Fy = two_sum(sf.y, SFL.y);
+                // tangential gradient: (2 w_j / r) (grad F - (grad F . u) u), formed in
+                // double-float and rounded once: a per-pair relative error of an FP32
+                // ulp is not amplified by the sums over pairs
+                const df gdr = df_add(df_add(df_mul(Fx, ux), df_mul(Fy, uy)), df_mul(Fz, z));
+                const float tx = df_add(Fx, df_neg(df_mul(gdr, ux))).h;
+                const float ty = df_add(Fy, df_neg(df_mul(gdr, uy))).h;
+                const float tz = df_add(Fz, df_neg(df_mul(gdr, z))).h;
+                const float sc = __fmul_rn(2.f * qv.w, __fadd_rn(rinv.h, rinv.l));
+                const float gx = __fmul_rn(sc, tx), gy = __fmul_rn(sc, ty), gz3 = __fmul_rn(sc, tz);
+                atomicAdd(a.dw + jj, f2d_exact(__fmul_rn(2.f, __fadd_rn(F.h, F.l))));
+                atomicAdd(a.dpos + 3 * (int64_t)jj, f2d_exact(gx));
+                atomicAdd(a.dpos + 3 * (int64_t)jj + 1, f2d_exact(gy));
+                atomicAdd(a.dpos + 3 * (int64_t)jj + 2, f2d_exact(gz3));
+                df_acc(pix, {gx, 0.f});
+                df_acc(piy, {gy, 0.f});
+                df_acc(piz, {gz3, 0.f});
+            }
+            e = en;
+            qv = qn;
+            ql = ln;
+            en = en2;
+            o0 = o1;
+            o1 = o2;
+            o2 = o3;
         }
         double di0 = -df_to(pix), di1 = -df_to(piy), di2 = -df_to(piz);
 #pragma unroll
@@ -754,7 +815,7 @@ int launch_accum_df_t(const ListArgs& a, int nsm, cudaStream_t st) {
 }
 template <int L>
 int launch_adj_df_t(const ListArgs& a, int nsm, cudaStream_t st) {
-    return launch_persistent(k_adj_df<L>, a, adj_df_smem_per_warp(a.bins.nbins, Shape<L>::NRP) * kDWarps, nsm, st);
+    return launch_persistent(k_adj_df<L>, a, adj_df_smem_per_warp(a.bins.nbins, AdjG<L>::N) * kDWarps, nsm, st);
 }
 
 }  // namespace
