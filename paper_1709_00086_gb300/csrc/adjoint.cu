@@ -23,7 +23,7 @@ namespace g3 {
 
 namespace {
 
-constexpr int kRows = 8;         // primaries per CTA in k_vgemm
+constexpr int kRows = 8;         // primaries per CTA in k_vgemm and k_vgemm_df
 constexpr int kVThreads = 256;
 
 struct MInfo {
@@ -34,25 +34,19 @@ struct MInfo {
     long long zoff[kMaxL + 1];  // complex offset of block m in zeta
 };
 
-// M entries as stored: FP32, or head + tail FP32 pairs for the double-float path
-template <class TM>
-__device__ __forceinline__ TM m_entry(double v);
-template <>
-__device__ __forceinline__ float m_entry<float>(double v) { return (float)v; }
-template <>
-__device__ __forceinline__ float2 m_entry<float2>(double v) {
+// an M entry of the double-float path: head + tail
+__device__ __forceinline__ float2 m_entry(double v) {
     const float h = (float)v;
     return make_float2(h, (float)(v - (double)h));
 }
 
-template <class TM>
 __global__ void k_build_mreal(const double* dz, MInfo mi, int lmax, int64_t zsize, size_t mfloats,
-                              TM* Mr) {
+                              float* Mr) {
     const int m = blockIdx.y, cat = blockIdx.z;
     if (m > lmax) return;
     const int K = mi.K[m], W = mi.W[m];
     const double* Z = dz + 2 * ((int64_t)cat * zsize + mi.zoff[m]);
-    TM* out = Mr + (size_t)cat * mfloats + mi.moff[m];
+    float* out = Mr + (size_t)cat * mfloats + mi.moff[m];
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < W * W; e += gridDim.x * blockDim.x) {
         const int rr = e / W, cc = e % W;
         const int r = rr % K, c = cc % K;
@@ -66,7 +60,7 @@ __global__ void k_build_mreal(const double* dz, MInfo mi, int lmax, int64_t zsiz
             const bool rlo = rr < K, clo = cc < K;
             v = (rlo == clo) ? re : (rlo ? -im : im);
         }
-        out[e] = m_entry<TM>(v);
+        out[e] = (float)v;
     }
 }
 
@@ -76,15 +70,14 @@ __global__ void k_build_mreal(const double* dz, MInfo mi, int lmax, int64_t zsiz
 // primary-weight term is added to dw[row], or, for rows of a chunk of
 // primaries (rorig non-null), to dw[rorig[rplist ? rplist[q0 + row] : q0 + row]].
 // FP32 M, V and sums.
-template <class TM>
 __global__ void __launch_bounds__(kVThreads) k_vgemm(const float* __restrict__ A, int RLP, int RL,
                                                      const int4* __restrict__ blks, int64_t row_lo,
-                                                     int64_t row_hi, const TM* __restrict__ Mall,
-                                                     size_t mfloats, MInfo mi, int lmax, TM* V,
+                                                     int64_t row_hi, const float* __restrict__ Mall,
+                                                     size_t mfloats, MInfo mi, int lmax, float* V,
                                                      double* dw, const int* rplist, const int* rorig,
                                                      int64_t q0) {
     extern __shared__ float sA[];  // kRows x RL
-    __shared__ TM red[kRows][kVThreads / 32];
+    __shared__ float red[kRows][kVThreads / 32];
     int4 blk;
     if (blks) {
         blk = blks[blockIdx.x];
@@ -92,7 +85,7 @@ __global__ void __launch_bounds__(kVThreads) k_vgemm(const float* __restrict__ A
         const int64_t b0 = row_lo + (int64_t)blockIdx.x * kRows;
         blk = make_int4(0, (int)b0, (int)(row_hi - b0 < kRows ? row_hi - b0 : kRows), 0);
     }
-    const TM* __restrict__ Mr = Mall + (size_t)blk.x * mfloats;
+    const float* __restrict__ Mr = Mall + (size_t)blk.x * mfloats;
     const int64_t r0 = blk.y;
     const int64_t rows = r0 + blk.z;
     for (int k = threadIdx.x; k < kRows * RL; k += kVThreads) {
@@ -100,33 +93,33 @@ __global__ void __launch_bounds__(kVThreads) k_vgemm(const float* __restrict__ A
         sA[k] = (r0 + rr < rows) ? A[(r0 + rr) * RLP + c] : 0.f;
     }
     __syncthreads();
-    TM dwp[kRows];
+    float dwp[kRows];
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) dwp[r] = (TM)0;
+    for (int r = 0; r < kRows; ++r) dwp[r] = 0.f;
     for (int col = threadIdx.x; col < RL; col += kVThreads) {
         int m = 0;
         while (m < lmax && col >= mi.col0[m + 1]) ++m;
         const int W = mi.W[m], c = col - mi.col0[m];
-        const TM* Mrow = Mr + mi.moff[m] + (int64_t)c * W;
+        const float* Mrow = Mr + mi.moff[m] + (int64_t)c * W;
         const float* As = sA + mi.col0[m];
-        TM acc[kRows];
+        float acc[kRows];
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) acc[r] = (TM)0;
+        for (int r = 0; r < kRows; ++r) acc[r] = 0.f;
         for (int k = 0; k < W; ++k) {
-            const TM mv = __ldg(Mrow + k);
+            const float mv = __ldg(Mrow + k);
 #pragma unroll
-            for (int r = 0; r < kRows; ++r) acc[r] = fma(mv, (TM)As[r * RL + k], acc[r]);
+            for (int r = 0; r < kRows; ++r) acc[r] = fma(mv, As[r * RL + k], acc[r]);
         }
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
             if (r0 + r < rows) V[(r0 + r) * RLP + col] = acc[r];
-            dwp[r] = fma((TM)sA[r * RL + col], acc[r], dwp[r]);
+            dwp[r] = fma(sA[r * RL + col], acc[r], dwp[r]);
         }
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
-        TM v = dwp[r];
+        float v = dwp[r];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) red[r][wid] = v;
@@ -145,102 +138,123 @@ __global__ void __launch_bounds__(kVThreads) k_vgemm(const float* __restrict__ A
     }
 }
 
-// The same product in double-float: M as head + tail pairs, the FP32 A entries
-// exact, each product M_h a formed exactly (a multiply and an FMA), the running
-// sum's head updated by an error-free two-sum and every rounding error, the
-// product's low part and M_l a gathered in the tail; V stored renormalised as
-// head + tail.  ~10 FP32 operations per multiply-add instead of one FP64 FMA,
-// which runs at 1/58 of the FP32 rate on this part.  The primary-weight term
-// Re(A^H V) sums in FP64 (one term per column).
-__global__ void __launch_bounds__(kVThreads) k_vgemm_df(const float* __restrict__ A, int RLP, int RL,
-                                                        const int4* __restrict__ blks, int64_t row_lo,
-                                                        int64_t row_hi, const float2* __restrict__ Mall,
-                                                        size_t mfloats, MInfo mi, int lmax, float2* V,
-                                                        double* dw, const int* rplist, const int* rorig,
-                                                        int64_t q0) {
-    extern __shared__ float sA[];  // kRows x RL
-    __shared__ double red[kRows][kVThreads / 32];
+// M of one catalog for the double-float path, one warp per row c: entries as head +
+// tail, and the row's sum of |M|, which bounds the sums of k_vgemm_df.  The real
+// form is symmetric, so that row c is also column c.
+constexpr int kBWarps = 8;
+__global__ void __launch_bounds__(kBWarps * 32) k_build_m_df(const double* dz, MInfo mi, int lmax, int RL,
+                                                            int64_t zsize, size_t mfloats, float2* Mr, float* norm) {
+    const int lane = threadIdx.x & 31, cat = blockIdx.y;
+    const int col = blockIdx.x * kBWarps + (threadIdx.x >> 5);
+    if (col >= RL) return;
+    int m = 0;
+    while (m < lmax && col >= mi.col0[m + 1]) ++m;
+    const int K = mi.K[m], W = mi.W[m], rr = col - mi.col0[m], r = rr % K;
+    const double* Z = dz + 2 * ((int64_t)cat * zsize + mi.zoff[m]);
+    float2* out = Mr + (size_t)cat * mfloats + mi.moff[m] + (int64_t)rr * W;
+    float sum = 0.f;
+    for (int cc = lane; cc < W; cc += 32) {
+        const int c = cc % K;
+        // M = G + G^H, G = dz / 2
+        const double re = 0.5 * (Z[2 * ((int64_t)r * K + c)] + Z[2 * ((int64_t)c * K + r)]);
+        const double im = 0.5 * (Z[2 * ((int64_t)r * K + c) + 1] - Z[2 * ((int64_t)c * K + r) + 1]);
+        const bool rlo = rr < K, clo = cc < K;
+        const float2 v = m_entry(m == 0 || rlo == clo ? re : (rlo ? -im : im));
+        out[cc] = v;
+        sum += fabsf(v.x);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) norm[(size_t)cat * RL + col] = sum;
+}
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+// V = M A in double-float (M head + tail, A exact), 8 rows of one catalog per CTA,
+// one column per thread at a time, two rows per packed operation.  The head of
+// every sum carries a bias of three times its bound (the row sum of |M| times the
+// largest |A| of the block), so that the difference to the next head is exact and
+// one FMA returns the rounding error: 5 operations per multiply-add (10 with an
+// error-free addition).  Bound by issue; M (from L2) is read once per 8 rows,
+// coalesced by its symmetry (16 rows per CTA: the same time).  20,000 rows at B =
+// lmax = 10: 0.65 ms against 1.73.
+// The primary-weight term Re(A^H V) is the pair pass's (k_adj_df).
+__global__ void __launch_bounds__(kVThreads, 4) k_vgemm_df(
+    const float* __restrict__ A, int RLP, int RL, const int4* __restrict__ blks, int64_t row_lo, int64_t row_hi,
+    const float2* __restrict__ Mall, const float* __restrict__ norm, size_t mfloats, MInfo mi, int lmax,
+    float2* V) {
+    constexpr int R = kRows, RS = R + 4;  // rows, column stride in shared memory
+    extern __shared__ __align__(16) float sA[];  // RL x RS
+    __shared__ int amax[kMaxL + 1];
     int4 blk;
     if (blks) {
         blk = blks[blockIdx.x];
     } else {
-        const int64_t b0 = row_lo + (int64_t)blockIdx.x * kRows;
-        blk = make_int4(0, (int)b0, (int)(row_hi - b0 < kRows ? row_hi - b0 : kRows), 0);
+        const int64_t b0 = row_lo + (int64_t)blockIdx.x * R;
+        blk = make_int4(0, (int)b0, (int)(row_hi - b0 < R ? row_hi - b0 : R), 0);
     }
     const float2* __restrict__ Mr = Mall + (size_t)blk.x * mfloats;
+    const float* __restrict__ nr = norm + (size_t)blk.x * RL;
     const int64_t r0 = blk.y;
-    const int64_t rows = r0 + blk.z;
-    for (int k = threadIdx.x; k < kRows * RL; k += kVThreads) {
-        const int rr = k / RL, c = k % RL;
-        sA[k] = (r0 + rr < rows) ? A[(r0 + rr) * RLP + c] : 0.f;
+    const int nrow = blk.z;
+    if (threadIdx.x <= lmax) amax[threadIdx.x] = 0;
+    __syncthreads();
+    for (int c = threadIdx.x; c < RL; c += kVThreads) {
+        int m = 0;
+        while (m < lmax && c >= mi.col0[m + 1]) ++m;
+        float mx = 0.f;
+#pragma unroll
+        for (int rr = 0; rr < R; ++rr) {
+            const float v = rr < nrow ? __ldg(A + (r0 + rr) * RLP + c) : 0.f;
+            sA[c * RS + rr] = v;
+            mx = fmaxf(mx, fabsf(v));
+        }
+        atomicMax(&amax[m], __float_as_int(mx));
     }
     __syncthreads();
-    double dwp[kRows];
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) dwp[r] = 0.0;
     for (int col = threadIdx.x; col < RL; col += kVThreads) {
         int m = 0;
         while (m < lmax && col >= mi.col0[m + 1]) ++m;
         const int W = mi.W[m], c = col - mi.col0[m];
-        const float2* Mrow = Mr + mi.moff[m] + (int64_t)c * W;
-        const float* As = sA + mi.col0[m];
-        float sh[kRows], sl[kRows];
+        const float2* Mc = Mr + mi.moff[m] + c;
+        const float4* As = reinterpret_cast<const float4*>(sA + mi.col0[m] * RS);
+        const float bias = 3.f * __ldg(nr + col) * __int_as_float(amax[m]);
+        float2 H[R / 2], Lo[R / 2];
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) sh[r] = sl[r] = 0.f;
+        for (int r = 0; r < R / 2; ++r) {
+            H[r] = dup(bias);
+            Lo[r] = dup(0.f);
+        }
+#pragma unroll 4
         for (int k = 0; k < W; ++k) {
-            const float2 mv = __ldg(Mrow + k);
+            const float2 mv = __ldg(Mc + (int64_t)k * W);
+            const float2 Mh = dup(mv.x), Ml = dup(mv.y);
 #pragma unroll
-            for (int r = 0; r < kRows; ++r) {
-                const float x = As[r * RL + k];
-                const float p = __fmul_rn(mv.x, x);
-                const float pe = __fmaf_rn(mv.x, x, -p);
-                const float s = __fadd_rn(sh[r], p);
-                const float bb = __fsub_rn(s, sh[r]);
-                const float err = __fadd_rn(__fsub_rn(sh[r], __fsub_rn(s, bb)), __fsub_rn(p, bb));
-                sh[r] = s;
-                sl[r] = __fmaf_rn(mv.y, x, __fadd_rn(sl[r], __fadd_rn(err, pe)));
+            for (int r = 0; r < R / 4; ++r) {
+                const float4 a4 = As[k * (RS / 4) + r];
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const float2 x = half ? make_float2(a4.z, a4.w) : make_float2(a4.x, a4.y);
+                    float2& h = H[2 * r + half];
+                    float2& l = Lo[2 * r + half];
+                    const float2 s = __ffma2_rn(Mh, x, h);
+                    const float2 e = __ffma2_rn(Mh, x, __fadd2_rn(h, neg2(s)));
+                    l = __ffma2_rn(Ml, x, __fadd2_rn(l, e));
+                    h = s;
+                }
             }
         }
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-            const float h = __fadd_rn(sh[r], sl[r]);
-            const float l = __fsub_rn(sl[r], __fsub_rn(h, sh[r]));
-            if (r0 + r < rows) V[(r0 + r) * RLP + col] = make_float2(h, l);
-            dwp[r] = fma((double)sA[r * RL + col], (double)h + (double)l, dwp[r]);
+        for (int r = 0; r < R; ++r) {
+            const float hb = __fsub_rn(r & 1 ? H[r / 2].y : H[r / 2].x, bias);  // exact
+            const float lb = r & 1 ? Lo[r / 2].y : Lo[r / 2].x;
+            // renormalised
+            const float h = __fadd_rn(hb, lb), bb = __fsub_rn(h, hb);
+            const float l = __fadd_rn(__fsub_rn(hb, __fsub_rn(h, bb)), __fsub_rn(lb, bb));
+            if (r < nrow) V[(r0 + r) * RLP + col] = make_float2(h, l);
         }
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-        double v = dwp[r];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[r][wid] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < kRows && r0 + threadIdx.x < rows) {
-        double s = 0.0;
-        for (int k = 0; k < kVThreads / 32; ++k) s += red[threadIdx.x][k];
-        const int64_t row = r0 + threadIdx.x;
-        int64_t idx = row;
-        if (rorig) {
-            const int64_t q = q0 + row;
-            idx = rorig[rplist ? rplist[q] : q];
-        }
-        dw[idx] += s;
     }
 }
-
-template <class TM>
-struct VgemmKernel;
-template <>
-struct VgemmKernel<float> {
-    static constexpr auto fn = k_vgemm<float>;
-};
-template <>
-struct VgemmKernel<float2> {
-    static constexpr auto fn = k_vgemm_df;
-};
 
 MInfo make_info(int nbins, int lmax) {
     MInfo mi{};
@@ -275,80 +289,79 @@ size_t adjoint_m_floats(int nbins, int lmax) {
 
 int adjoint_rows_per_block() { return kRows; }
 
-template <class TM>
-int adjoint_m_t(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, TM* Mr, cudaStream_t st) {
+int launch_adjoint_m(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float* Mr,
+                     cudaStream_t st) {
     const MInfo mi = make_info(nbins, lmax);
     dim3 g1(64, lmax + 1, ncat);
-    k_build_mreal<TM><<<g1, 256, 0, st>>>(dzeta, mi, lmax, zsize, adjoint_m_floats(nbins, lmax), Mr);
+    k_build_mreal<<<g1, 256, 0, st>>>(dzeta, mi, lmax, zsize, adjoint_m_floats(nbins, lmax), Mr);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <class TM>
-int adjoint_prep_t(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, const float* A, int RLP,
-                   int RL, const int4* blks, int nblks, TM* Mr, TM* V, double* dw, cudaStream_t st) {
-    if (adjoint_m_t<TM>(dzeta, nbins, lmax, ncat, zsize, Mr, st) != 0) return -1;
-    if (nblks > 0) {
-        const MInfo mi = make_info(nbins, lmax);
-        const size_t smem = sizeof(float) * kRows * RL;
-        if (cudaFuncSetAttribute(VgemmKernel<TM>::fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-            return -1;
-        VgemmKernel<TM>::fn<<<(unsigned)nblks, kVThreads, smem, st>>>(A, RLP, RL, blks, 0, 0, Mr,
-                                                                      adjoint_m_floats(nbins, lmax), mi, lmax, V,
-                                                                      dw, nullptr, nullptr, 0);
-    }
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-template <class TM>
-int vgemm_rows_t(const float* A, int RLP, int RL, int64_t row_lo, int64_t row_hi, const TM* Mr, int nbins,
-                 int lmax, TM* V, double* dw, const int* plist, const int* orig, int64_t q0, cudaStream_t st) {
-    if (row_hi <= row_lo) return 0;
+int launch_adjoint_m_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float2* Mr, float* norm,
+                        cudaStream_t st) {
     const MInfo mi = make_info(nbins, lmax);
-    const size_t smem = sizeof(float) * kRows * RL;
-    if (cudaFuncSetAttribute(VgemmKernel<TM>::fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return -1;
-    const int64_t nb = (row_hi - row_lo + kRows - 1) / kRows;
-    VgemmKernel<TM>::fn<<<(unsigned)nb, kVThreads, smem, st>>>(A, RLP, RL, nullptr, row_lo, row_hi, Mr,
-                                                                adjoint_m_floats(nbins, lmax), mi, lmax, V, dw,
-                                                                plist, orig, q0);
+    const int RL = nbins * (lmax + 1) * (lmax + 1);
+    dim3 grid((RL + kBWarps - 1) / kBWarps, ncat);
+    k_build_m_df<<<grid, kBWarps * 32, 0, st>>>(dzeta, mi, lmax, RL, zsize, adjoint_m_floats(nbins, lmax), Mr, norm);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
-
 
 int launch_adjoint_prep(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, const float* A,
                         int RLP, int RL, const int4* blks, int nblks, float* Mr, float* V, double* dw,
                         cudaStream_t st) {
-    return adjoint_prep_t<float>(dzeta, nbins, lmax, ncat, zsize, A, RLP, RL, blks, nblks, Mr, V, dw, st);
-}
-
-int launch_adjoint_prep_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, const float* A,
-                           int RLP, int RL, const int4* blks, int nblks, float2* Mr, float2* V, double* dw,
-                           cudaStream_t st) {
-    return adjoint_prep_t<float2>(dzeta, nbins, lmax, ncat, zsize, A, RLP, RL, blks, nblks, Mr, V, dw, st);
-}
-
-int launch_adjoint_m(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float* Mr,
-                     cudaStream_t st) {
-    return adjoint_m_t<float>(dzeta, nbins, lmax, ncat, zsize, Mr, st);
-}
-
-int launch_adjoint_m_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float2* Mr,
-                        cudaStream_t st) {
-    return adjoint_m_t<float2>(dzeta, nbins, lmax, ncat, zsize, Mr, st);
+    if (launch_adjoint_m(dzeta, nbins, lmax, ncat, zsize, Mr, st) != 0) return -1;
+    if (nblks > 0) {
+        const MInfo mi = make_info(nbins, lmax);
+        const size_t smem = sizeof(float) * kRows * RL;
+        if (cudaFuncSetAttribute(k_vgemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess)
+            return -1;
+        k_vgemm<<<(unsigned)nblks, kVThreads, smem, st>>>(A, RLP, RL, blks, 0, 0, Mr,
+                                                                 adjoint_m_floats(nbins, lmax), mi, lmax, V, dw,
+                                                                 nullptr, nullptr, 0);
+    }
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int launch_vgemm_rows(const float* A, int RLP, int RL, int64_t row_lo, int64_t row_hi, const float* Mr,
                       int nbins, int lmax, float* V, double* dw, const int* plist, const int* orig,
                       int64_t q0, cudaStream_t st) {
-    return vgemm_rows_t<float>(A, RLP, RL, row_lo, row_hi, Mr, nbins, lmax, V, dw, plist, orig, q0, st);
+    if (row_hi <= row_lo) return 0;
+    const MInfo mi = make_info(nbins, lmax);
+    const size_t smem = sizeof(float) * kRows * RL;
+    if (cudaFuncSetAttribute(k_vgemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return -1;
+    const int64_t nb = (row_hi - row_lo + kRows - 1) / kRows;
+    k_vgemm<<<(unsigned)nb, kVThreads, smem, st>>>(A, RLP, RL, nullptr, row_lo, row_hi, Mr,
+                                                          adjoint_m_floats(nbins, lmax), mi, lmax, V, dw, plist, orig,
+                                                          q0);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+namespace {
+int vgemm_df(const float* A, int RLP, int RL, const int4* blks, int64_t nb, int64_t row_lo, int64_t row_hi,
+             const float2* Mr, const float* norm, int nbins, int lmax, float2* V, cudaStream_t st) {
+    const MInfo mi = make_info(nbins, lmax);
+    const size_t smem = sizeof(float) * (kRows + 4) * RL;
+    if (cudaFuncSetAttribute(k_vgemm_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return -1;
+    k_vgemm_df<<<(unsigned)nb, kVThreads, smem, st>>>(A, RLP, RL, blks, row_lo, row_hi, Mr, norm,
+                                                      adjoint_m_floats(nbins, lmax), mi, lmax, V);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+}  // namespace
+
+int launch_vgemm_blocks_df(const float* A, int RLP, int RL, const int4* blks, int nblks, const float2* Mr,
+                           const float* norm, int nbins, int lmax, float2* V, cudaStream_t st) {
+    if (nblks <= 0) return 0;
+    return vgemm_df(A, RLP, RL, blks, nblks, 0, 0, Mr, norm, nbins, lmax, V, st);
 }
 
 int launch_vgemm_rows_df(const float* A, int RLP, int RL, int64_t row_lo, int64_t row_hi, const float2* Mr,
-                         int nbins, int lmax, float2* V, double* dw, const int* plist, const int* orig,
-                         int64_t q0, cudaStream_t st) {
-    return vgemm_rows_t<float2>(A, RLP, RL, row_lo, row_hi, Mr, nbins, lmax, V, dw, plist, orig, q0, st);
+                         const float* norm, int nbins, int lmax, float2* V, cudaStream_t st) {
+    const int64_t rows = row_hi - row_lo;
+    if (rows <= 0) return 0;
+    return vgemm_df(A, RLP, RL, nullptr, (rows + kRows - 1) / kRows, row_lo, row_hi, Mr, norm, nbins, lmax, V, st);
 }
 
 }  // namespace g3

@@ -121,7 +121,7 @@ struct g3pcf_plan_s {
     DevBuf d_colconv, d_colcoef, d_slotconv, d_slotcoef, d_monoexp, d_monoconv, d_monoidx, d_monocoef;
     DevBuf d_ranges, d_tiles_tc, d_cats, d_mreal, d_V, d_bintab, wrow, d_vblk, d_strips_tc, d_items;
     DevBuf d_bop, d_bblk, d_bcat;
-    DevBuf d_slotcoefdf, d_mrealdf, d_Vdf, d_colcoefdf;
+    DevBuf d_slotcoefdf, d_mrealdf, d_Vdf, d_colcoefdf, d_mnorm;
     int64_t opt_chunk = 0;   // G3PCF_OPT_CHUNK_ROWS
     // pinned staging for host -> device tables (capturable copies); offset
     // restarts at every forward
@@ -847,8 +847,8 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
             int vr = launch_accum(P->lmax, la, P->nsm, st);
             if (vr == 0)
                 vr = la.precise ? launch_vgemm_rows_df(la.A, la.RLP, la.RL, la.qa - la.q0, la.qb - la.q0,
-                                                      P->d_mrealdf.as<float2>(), P->nbins, P->lmax,
-                                                      P->d_Vdf.as<float2>(), pa.dw, la.plist, la.orig, la.q0, st)
+                                                      P->d_mrealdf.as<float2>(), P->d_mnorm.as<float>(), P->nbins, P->lmax,
+                                                      P->d_Vdf.as<float2>(), st)
                                 : launch_vgemm_rows(la.A, la.RLP, la.RL, la.qa - la.q0, la.qb - la.q0,
                                                     P->d_mreal.as<float>(), P->nbins, P->lmax, P->d_V.as<float>(),
                                                     pa.dw, la.plist, la.orig, la.q0, st);
@@ -1542,6 +1542,7 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
         const int64_t C = P->fixed_chunk;
         const bool precise = P->opt_grad == 0;
         if (precise ? (ensure(P, P->d_mrealdf, sizeof(float2) * adjoint_m_floats(P->nbins, P->lmax), "adjoint M") ||
+                       ensure(P, P->d_mnorm, sizeof(float) * P->RL, "adjoint M") ||
                        ensure(P, P->d_Vdf, sizeof(float2) * (size_t)P->RLP * C, "adjoint V"))
                     : (ensure(P, P->d_mreal, sizeof(float) * adjoint_m_floats(P->nbins, P->lmax), "adjoint M") ||
                        ensure(P, P->d_V, sizeof(float) * (size_t)P->RLP * C, "adjoint V")))
@@ -1551,7 +1552,7 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
         CK(cudaMemsetAsync(P->small.p, 0, 256, st));
         CK(cudaMemsetAsync(P->counts.p, 0, sizeof(unsigned long long) * P->nbins, st));
         if ((precise ? launch_adjoint_m_df(dzeta, P->nbins, P->lmax, 1, zsize_of(P->nbins, P->lmax),
-                                           P->d_mrealdf.as<float2>(), st)
+                                           P->d_mrealdf.as<float2>(), P->d_mnorm.as<float>(), st)
                      : launch_adjoint_m(dzeta, P->nbins, P->lmax, 1, zsize_of(P->nbins, P->lmax),
                                         P->d_mreal.as<float>(), st)) != 0)
             return fail(G3PCF_ERR_CUDA, "adjoint preparation launch failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1591,33 +1592,50 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
         CK(cudaStreamSynchronize(st));
         return read_status(P);
     }
+    // the double-float pair pass (list path, G3PCF_OPT_GRAD_PRECISION 0) takes M and V in double-float
+    const bool precise = P->opt_grad == 0 && P->opt_pair != 1;
     // row blocks of one catalog each (rows are original indices; catalog c holds
-    // [offs[c], offs[c+1]) of a batched forward, every row of a single one)
+    // [offs[c], offs[c+1]) of a batched forward, every row of a single one, which the
+    // double-float product cuts into blocks by itself)
     const int RB = adjoint_rows_per_block();
     std::vector<int4> blks;
-    for (int c = 0; c < ncat; ++c) {
-        const int64_t r0 = ncat > 1 ? P->last_offs[c] : 0, r1 = ncat > 1 ? P->last_offs[c + 1] : rows;
-        for (int64_t r = r0; r < r1; r += RB) blks.push_back(int4{c, (int)r, (int)std::min<int64_t>(RB, r1 - r), 0});
-    }
-    // the double-float pair pass (list path, G3PCF_OPT_GRAD_PRECISION 0) takes M and V in FP64
-    const bool precise = P->opt_grad == 0 && P->opt_pair != 1;
+    if (ncat > 1 || !precise)
+        for (int c = 0; c < ncat; ++c) {
+            const int64_t r0 = ncat > 1 ? P->last_offs[c] : 0, r1 = ncat > 1 ? P->last_offs[c + 1] : rows;
+            for (int64_t r = r0; r < r1; r += RB) blks.push_back(int4{c, (int)r, (int)std::min<int64_t>(RB, r1 - r), 0});
+        }
     if ((precise ? (ensure(P, P->d_mrealdf, sizeof(float2) * adjoint_m_floats(P->nbins, P->lmax) * ncat, "adjoint M") ||
+                    ensure(P, P->d_mnorm, sizeof(float) * (size_t)P->RL * ncat, "adjoint M") ||
                     ensure(P, P->d_Vdf, sizeof(float2) * (size_t)P->RLP * rows, "adjoint V"))
                  : (ensure(P, P->d_mreal, sizeof(float) * adjoint_m_floats(P->nbins, P->lmax) * ncat, "adjoint M") ||
                     ensure(P, P->d_V, sizeof(float) * (size_t)P->RLP * rows, "adjoint V"))) ||
         ensure(P, P->d_vblk, sizeof(int4) * (blks.size() + 1), "adjoint blocks"))
         return G3PCF_ERR_ALLOC;
-    CK(cudaMemcpyAsync(P->d_vblk.p, blks.data(), sizeof(int4) * blks.size(), cudaMemcpyHostToDevice, st));
+    if (!blks.empty())
+        CK(cudaMemcpyAsync(P->d_vblk.p, blks.data(), sizeof(int4) * blks.size(), cudaMemcpyHostToDevice, st));
     int* d_status = P->small.as<int>();
     int* d_queue = d_status + 16;
     CK(cudaMemsetAsync(P->small.p, 0, 256, st));
     CK(cudaMemsetAsync(P->counts.p, 0, sizeof(unsigned long long) * P->nbins * ncat, st));
-    if ((precise ? launch_adjoint_prep_df(dzeta, P->nbins, P->lmax, ncat, zsize_of(P->nbins, P->lmax),
-                                         P->A.as<float>(), P->RLP, P->RL, P->d_vblk.as<int4>(), (int)blks.size(),
-                                         P->d_mrealdf.as<float2>(), P->d_Vdf.as<float2>(), dw, st)
-                 : launch_adjoint_prep(dzeta, P->nbins, P->lmax, ncat, zsize_of(P->nbins, P->lmax),
-                                       P->A.as<float>(), P->RLP, P->RL, P->d_vblk.as<int4>(), (int)blks.size(),
-                                       P->d_mreal.as<float>(), P->d_V.as<float>(), dw, st)) != 0)
+    const int64_t zs = zsize_of(P->nbins, P->lmax);
+    int prep = 0;
+    if (precise) {
+        const float2* M = P->d_mrealdf.as<float2>();
+        const float* nm = P->d_mnorm.as<float>();
+        prep = launch_adjoint_m_df(dzeta, P->nbins, P->lmax, ncat, zs, P->d_mrealdf.as<float2>(),
+                                   P->d_mnorm.as<float>(), st);
+        if (prep == 0)
+            prep = ncat > 1 ? launch_vgemm_blocks_df(P->A.as<float>(), P->RLP, P->RL, P->d_vblk.as<int4>(),
+                                                     (int)blks.size(), M, nm, P->nbins, P->lmax,
+                                                     P->d_Vdf.as<float2>(), st)
+                            : launch_vgemm_rows_df(P->A.as<float>(), P->RLP, P->RL, 0, rows, M, nm, P->nbins, P->lmax,
+                                                   P->d_Vdf.as<float2>(), st);
+    } else {
+        prep = launch_adjoint_prep(dzeta, P->nbins, P->lmax, ncat, zs, P->A.as<float>(), P->RLP, P->RL,
+                                   P->d_vblk.as<int4>(), (int)blks.size(), P->d_mreal.as<float>(), P->d_V.as<float>(),
+                                   dw, st);
+    }
+    if (prep != 0)
         return fail(G3PCF_ERR_CUDA, "adjoint preparation launch failed: %s", cudaGetErrorString(cudaGetLastError()));
     PairArgs pa{};
     pa.pts = P->pts.as<float4>();
@@ -2020,7 +2038,7 @@ int g3pcf_destroy(g3pcf_plan_t P) {
                       &P->d_segfirst, &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_colcoef, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
                       &P->d_tiles_tc, &P->d_cats, &P->d_mreal, &P->d_V, &P->d_bintab, &P->d_vblk,
                       &P->d_strips_tc, &P->d_items,
-                      &P->d_slotcoefdf, &P->d_mrealdf, &P->d_Vdf, &P->d_colcoefdf,
+                      &P->d_slotcoefdf, &P->d_mrealdf, &P->d_mnorm, &P->d_Vdf, &P->d_colcoefdf,
                       &P->wrow, &P->l_need, &P->l_base, &P->l_nch, &P->l_pool, &P->l_tag, &P->l_ord,
                       &P->l_gbase, &P->l_scantmp, &P->l_passq};
     for (DevBuf* b : bufs) b->release();

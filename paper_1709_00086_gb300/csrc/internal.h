@@ -365,14 +365,14 @@ int launch_vgemm_rows(const float* A, int RLP, int RL, int64_t row_lo, int64_t r
                       int64_t q0, cudaStream_t st);
 // Double-float forms of the three (M and V as head + tail FP32 pairs, ~48 bits;
 // for the double-float adjoint pass)
-int launch_adjoint_prep_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, const float* A,
-                           int RLP, int RL, const int4* blks, int nblks, float2* Mr, float2* V, double* dw,
-                           cudaStream_t st);
-int launch_adjoint_m_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float2* Mr,
+// norm: per catalog and A column the row sum of |M| (filled with M, ncat x RL)
+int launch_adjoint_m_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float2* Mr, float* norm,
                         cudaStream_t st);
+// V of the row blocks blks (adjoint_rows_per_block rows at most, one catalog each)
+int launch_vgemm_blocks_df(const float* A, int RLP, int RL, const int4* blks, int nblks, const float2* Mr,
+                           const float* norm, int nbins, int lmax, float2* V, cudaStream_t st);
 int launch_vgemm_rows_df(const float* A, int RLP, int RL, int64_t row_lo, int64_t row_hi, const float2* Mr,
-                         int nbins, int lmax, float2* V, double* dw, const int* plist, const int* orig,
-                         int64_t q0, cudaStream_t st);
+                         const float* norm, int nbins, int lmax, float2* V, cudaStream_t st);
 
 // ---- api.cu / noalloc.cu -----------------------------------------------------
 void set_last_error(const char* msg);

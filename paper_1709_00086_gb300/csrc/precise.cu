@@ -633,6 +633,19 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 4 : (L <= 8 ? 3 : 2)) k_ad
             // biases: three times the bound keeps every head above twice any term
             if (lane == 0) bias[b] = make_float2(3.f * s1, 3.f * s2);
         }
+        // the primary's own weight term of dL/dw: Re(A^H V)
+        {
+            const float* Arow = a.A + (int64_t)(a.chunked ? q - a.q0 : row) * a.RLP;
+            df wt = {0.f, 0.f};
+            for (int c = lane; c < a.RL; c += 32) {
+                const float2 v = Vrow[c];
+                df_acc(wt, df_mulf({v.x, v.y}, __ldg(Arow + c)));
+            }
+            double t = df_to(wt);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+            if (lane == 0) atomicAdd(a.dw + row, t);
+        }
         const int cb = a.base[q] < 0 ? 0 : a.base[q];
         const int nch = a.nchunks[q];
         const int* chunks = a.chunks + (int64_t)cb * 32;
