@@ -115,7 +115,7 @@ struct g3pcf_plan_s {
     int T = 0, T_tc = 0;
     int kflush = 16;
     // device buffers
-    DevBuf key_a, key_b, val_a, val_b, hist, hist_off, scan_tmp, pts, pts64, orig, cstart, plist;
+    DevBuf key_a, key_b, val_a, val_b, idx_scratch, pts, pts64, orig, cstart, plist;
     DevBuf small;       // status, queue
     DevBuf counts, A, partials, d_tiles, d_segs, d_segfirst, d_colmap, d_colscale, d_catoff;
     DevBuf d_colconv, d_colcoef, d_slotconv, d_slotcoef, d_monoexp, d_monoconv, d_monoidx, d_monocoef;
@@ -913,12 +913,9 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
     int64_t nprim = 0;
     if (n > 0) {
         // ---- workspace
-        const size_t hist_ints = radix_hist_ints(n);
-        const size_t off_ints = (hist_ints > (size_t)n ? hist_ints : (size_t)n) + 1;
         if (ensure(P, P->key_a, 4 * n, "keys") || ensure(P, P->key_b, 4 * n, "keys") ||
             ensure(P, P->val_a, 4 * n, "vals") || ensure(P, P->val_b, 4 * n, "vals") ||
-            ensure(P, P->hist, 4 * hist_ints, "hist") || ensure(P, P->hist_off, 4 * off_ints, "hist") ||
-            ensure(P, P->scan_tmp, 4 * (scan_tmp_ints(off_ints) + 16), "scan") ||
+            ensure(P, P->idx_scratch, 4 * index_scratch_ints(n), "index") ||
             ensure(P, P->pts, 16 * n, "points") || ensure(P, P->orig, 4 * n, "orig") ||
             ensure(P, P->cstart, 4 * (ncells + 1), "cells") || ensure(P, P->plist, 4 * n, "plist"))
             return G3PCF_ERR_ALLOC;
@@ -928,9 +925,7 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
         ib.key_b = P->key_b.as<unsigned>();
         ib.val_a = P->val_a.as<int>();
         ib.val_b = P->val_b.as<int>();
-        ib.hist = P->hist.as<int>();
-        ib.hist_off = P->hist_off.as<int>();
-        ib.scan_tmp = P->scan_tmp.as<int>();
+        ib.scratch = P->idx_scratch.as<int>();
         ib.pts = P->pts.as<float4>();
         ib.pts64 = c.pos_f64 ? P->pts64.as<double>() : nullptr;
         ib.orig = P->orig.as<int>();
@@ -2032,8 +2027,8 @@ int g3pcf_destroy(g3pcf_plan_t P) {
     g_err.clear();
     if (!P) return G3PCF_OK;
     if (P->device >= 0) cudaStreamSynchronize(P->stream);
-    DevBuf* bufs[] = {&P->key_a, &P->key_b, &P->val_a, &P->val_b, &P->hist, &P->hist_off,
-                      &P->scan_tmp, &P->pts, &P->pts64, &P->orig, &P->cstart, &P->plist,
+    DevBuf* bufs[] = {&P->key_a, &P->key_b, &P->val_a, &P->val_b, &P->idx_scratch,
+                      &P->pts, &P->pts64, &P->orig, &P->cstart, &P->plist,
                       &P->small, &P->counts, &P->A, &P->partials, &P->d_tiles, &P->d_segs,
                       &P->d_segfirst, &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_colcoef, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
                       &P->d_tiles_tc, &P->d_cats, &P->d_mreal, &P->d_V, &P->d_bintab, &P->d_vblk,

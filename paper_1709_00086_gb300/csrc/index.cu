@@ -15,9 +15,11 @@ namespace g3 {
 
 namespace {
 
+// Radix tiles of 256 x ITEMS keys: 4 items per thread up to kSmallSort points, so
+// that a small catalog still spreads over the chip, else 16.
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kTile = kSortThreads * kSortItems;  // 4096 keys per tile
+constexpr int64_t kSmallSort = 1 << 16;
+constexpr int kPrimTile = 1024;  // slots per counter of the primaries' compaction
 constexpr int kScanBlock = 1024;
 
 __device__ __forceinline__ unsigned lanemask_lt() {
@@ -26,13 +28,8 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
-// ---- keys ----------------------------------------------------------------
-
-__global__ void k_keys(IndexArgs a, const int64_t* cat_off, int ncat, unsigned* key,
-                       int* val, int* status) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    double x[3];
+// Position i of the input in FP64 (0 where it is out of range: flagged in k_keys).
+__device__ __forceinline__ bool load_pos(const IndexArgs& a, int64_t i, double (&x)[3]) {
     if (a.pos_f64) {
         const double* p = static_cast<const double*>(a.pos) + 3 * i;
         x[0] = p[0]; x[1] = p[1]; x[2] = p[2];
@@ -40,32 +37,58 @@ __global__ void k_keys(IndexArgs a, const int64_t* cat_off, int ncat, unsigned* 
         const float* p = static_cast<const float*>(a.pos) + 3 * i;
         x[0] = p[0]; x[1] = p[1]; x[2] = p[2];
     }
-    float w = a.w[i];
-    bool bad = !isfinite(w);
-    int c[3];
-    for (int d = 0; d < 3; ++d) {
+    bool ok = true;
+    for (int d = 0; d < 3; ++d)
         if (!(x[d] >= 0.0 && x[d] < a.g.boxd)) {  // also catches NaN
-            bad = true;
+            ok = false;
             x[d] = 0.0;
         }
-        const float xf = (float)x[d];
-        const int n = d == 0 ? a.g.ncx : a.g.nc;
-        const int cc = (int)(xf * (d == 0 ? a.g.inv_cellx : a.g.inv_cell));
-        c[d] = cc < 0 ? 0 : (cc >= n ? n - 1 : cc);
-    }
-    if (bad) atomicOr(status, kStatusRange);
-    long long cat = 0;
-    if (cat_off) {
-        int lo = 0, hi = ncat - 1;  // last catalog with cat_off[c] <= i
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (cat_off[mid] <= i) lo = mid; else hi = mid - 1;
+    return ok;
+}
+
+// ---- keys and the first digit's histogram --------------------------------------
+
+// hist: [tile][256] counts of the lowest digit; zero[0 .. nzero): cleared for the
+// later passes' histograms and the primaries' counters.
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads) k_keys(IndexArgs a, const int64_t* cat_off, int ncat, unsigned* key,
+                                                       int* status, int* hist, int* zero, int64_t nzero) {
+    __shared__ int h[256];
+    h[threadIdx.x] = 0;
+    for (int64_t k = blockIdx.x * (int64_t)kSortThreads + threadIdx.x; k < nzero;
+         k += (int64_t)gridDim.x * kSortThreads)
+        zero[k] = 0;
+    __syncthreads();
+    const int64_t base = blockIdx.x * (int64_t)(kSortThreads * ITEMS) + threadIdx.x;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const int64_t i = base + it * kSortThreads;
+        if (i >= a.n) continue;
+        double x[3];
+        const bool ok = load_pos(a, i, x);
+        if (!ok || !isfinite(a.w[i])) atomicOr(status, kStatusRange);
+        int c[3];
+        for (int d = 0; d < 3; ++d) {
+            const float xf = (float)x[d];
+            const int n = d == 0 ? a.g.ncx : a.g.nc;
+            const int cc = (int)(xf * (d == 0 ? a.g.inv_cellx : a.g.inv_cell));
+            c[d] = cc < 0 ? 0 : (cc >= n ? n - 1 : cc);
         }
-        cat = lo;
+        long long cat = 0;
+        if (cat_off) {
+            int lo = 0, hi = ncat - 1;  // last catalog with cat_off[c] <= i
+            while (lo < hi) {
+                int mid = (lo + hi + 1) >> 1;
+                if (cat_off[mid] <= i) lo = mid; else hi = mid - 1;
+            }
+            cat = lo;
+        }
+        const unsigned k = (unsigned)(cat * a.g.cells_per_cat + (long long)morton2(c[1], c[2]) * a.g.ncx + c[0]);
+        key[i] = k;
+        atomicAdd(&h[k & 255u], 1);
     }
-    long long k = cat * a.g.cells_per_cat + (long long)morton2(c[1], c[2]) * a.g.ncx + c[0];
-    key[i] = (unsigned)k;
-    val[i] = (int)i;
+    __syncthreads();
+    hist[blockIdx.x * 256 + threadIdx.x] = h[threadIdx.x];
 }
 
 // ---- exclusive scan (int32) --------------------------------------------
@@ -97,12 +120,15 @@ __device__ int block_scan_excl(int v, int* sh, int& total) {
     return pre;
 }
 
-__global__ void k_scan_reduce(const int* in, int64_t n, int* bsum) {
+// The radix offsets: an exclusive scan of hist in (digit, tile) order, in place of
+// [tile][digit].  Element e = digit * ntiles + tile.
+__device__ __forceinline__ int64_t hist_at(int64_t e, int ntiles) { return (e % ntiles) * 256 + e / ntiles; }
+
+__global__ void k_scan_reduce(const int* in, int ntiles, int64_t n, int* bsum) {
     __shared__ int sh[32];
-    int64_t i = blockIdx.x * (int64_t)kScanBlock + threadIdx.x;
-    int v = i < n ? in[i] : 0;
+    const int64_t i = blockIdx.x * (int64_t)kScanBlock + threadIdx.x;
     int tot;
-    block_scan_excl(v, sh, tot);
+    block_scan_excl(i < n ? in[hist_at(i, ntiles)] : 0, sh, tot);
     if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
@@ -119,123 +145,136 @@ __global__ void k_scan_top(int* bsum, int nb) {
     }
 }
 
-__global__ void k_scan_final(const int* in, int64_t n, const int* bsum, int* out) {
+__global__ void k_scan_final(int* io, int ntiles, int64_t n, const int* bsum) {
     __shared__ int sh[32];
-    int64_t i = blockIdx.x * (int64_t)kScanBlock + threadIdx.x;
-    int v = i < n ? in[i] : 0;
+    const int64_t i = blockIdx.x * (int64_t)kScanBlock + threadIdx.x;
     int tot;
-    int pre = block_scan_excl(v, sh, tot);
-    if (i < n) out[i] = bsum[blockIdx.x] + pre;
+    const int v = i < n ? io[hist_at(i, ntiles)] : 0;
+    const int pre = block_scan_excl(v, sh, tot);
+    if (i < n) io[hist_at(i, ntiles)] = bsum[blockIdx.x] + pre;
 }
 
 // ---- radix sort -----------------------------------------------------------
 
-__global__ void k_radix_hist(const unsigned* key, int64_t n, int shift, int ntiles, int* hist) {
-    __shared__ int h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kTile;
-#pragma unroll 4
-    for (int it = 0; it < kSortItems; ++it) {
-        int64_t i = base + it * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(key[i] >> shift) & 255u], 1);
-    }
-    __syncthreads();
-    hist[threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
-}
+struct ScatterArgs {
+    const unsigned* key;
+    const int* val;        // null in the first pass: value i
+    int64_t n;
+    int shift, ntiles;
+    const int* hist;       // [tile][256]: counts (SCANNED = false) or offsets
+    unsigned* key_out;
+    int* val_out;          // not written by the last pass
+    int* hist_next;        // next digit's histogram (not the last pass)
+    // last pass: the sorted arrays
+    float4* pts;
+    double* pts64;
+    int* orig;
+    int* negw;
+    int64_t n_primary;     // < n: count the primaries per kPrimTile slots
+    int* prim_count;
+};
 
-// Stable scatter: warp w of a tile owns tile items [w*512, (w+1)*512) and
-// ranks them round by round (32 at a time) with per-warp digit counters; the
-// warps' counters are then prefix-summed per digit in warp order.
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
-    const unsigned* key, const int* val, int64_t n, int shift, int ntiles, const int* offs,
-    unsigned* key_out, int* val_out) {
+// Stable scatter: warp w of a tile owns 32 ITEMS consecutive items and ranks them
+// round by round (32 at a time) with per-warp digit counters; the warps' counters
+// are then prefix-summed per digit in warp order.  With few tiles every CTA forms
+// its own digit offsets from the tiles' counts (no scan launches); the pass counts
+// the next digit while it scatters, and the last one writes the sorted points.
+template <int ITEMS, bool SCANNED, bool LAST>
+__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(ScatterArgs s, IndexArgs a) {
     constexpr int kWarps = kSortThreads / 32;
-    constexpr int kPerWarp = kTile / kWarps;    // 512
-    constexpr int kRounds = kPerWarp / 32;      // 16
+    constexpr int kPerWarp = 32 * ITEMS;
+    constexpr int kTile = kSortThreads * ITEMS;
     __shared__ int wcnt[kWarps][257];
+    __shared__ int soff[256];
+    __shared__ int wsum[kWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int d = threadIdx.x; d < kWarps * 257; d += kSortThreads) (&wcnt[0][0])[d] = 0;
+    if constexpr (SCANNED) {
+        soff[threadIdx.x] = s.hist[(int64_t)blockIdx.x * 256 + threadIdx.x];
+    } else {
+        // digit d = thread: items of lower digits, plus those of d in earlier tiles
+        int before = 0, tot = 0;
+#pragma unroll 8
+        for (int t = 0; t < s.ntiles; ++t) {
+            const int v = __ldg(s.hist + t * 256 + threadIdx.x);
+            before += t < (int)blockIdx.x ? v : 0;
+            tot += v;
+        }
+        int x = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[wid] = x;
+        __syncthreads();
+        int pre = 0;
+        for (int w = 0; w < wid; ++w) pre += wsum[w];
+        soff[threadIdx.x] = pre + x - tot + before;
+    }
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * kTile + wid * kPerWarp;
-    unsigned kk[kRounds];
-    int vv[kRounds];
-    int loc[kRounds];
+    unsigned kk[ITEMS];
+    int vv[ITEMS], loc[ITEMS];
     const unsigned lt = lanemask_lt();
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        int64_t i = base + r * 32 + lane;
-        unsigned k = 0;
-        int v = 0;
-        int dg = 256;  // sentinel digit for items past the end
-        if (i < n) {
-            k = key[i];
-            v = val[i];
-            dg = (k >> shift) & 255u;
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t i = base + r * 32 + lane;
+        kk[r] = 0;
+        vv[r] = 0;
+        if (i < s.n) {
+            kk[r] = s.key[i];
+            vv[r] = s.val ? s.val[i] : (int)i;
         }
-        kk[r] = k;
-        vv[r] = v;
-        unsigned peers = __match_any_sync(0xffffffffu, dg);
-        int leader = __ffs(peers) - 1;
-        int b = 0;
-        if (lane == leader) {
-            b = wcnt[wid][dg];
-            wcnt[wid][dg] = b + __popc(peers);
-        }
-        b = __shfl_sync(0xffffffffu, b, leader);
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int dg = base + r * 32 + lane < s.n ? (kk[r] >> s.shift) & 255u : 256;  // 256: past the end
+        const unsigned peers = __match_any_sync(0xffffffffu, dg);
+        const int b = wcnt[wid][dg];
         loc[r] = b + __popc(peers & lt);
+        __syncwarp();
+        if ((peers & lt) == 0u) wcnt[wid][dg] = b + __popc(peers);
         __syncwarp();
     }
     __syncthreads();
     {
-        int d = threadIdx.x;  // 256 threads <-> 256 digits
-        int run = 0;
+        const int d = threadIdx.x;  // 256 threads <-> 256 digits
+        int run = soff[d];
         for (int w = 0; w < kWarps; ++w) {
-            int t = wcnt[w][d];
+            const int t = wcnt[w][d];
             wcnt[w][d] = run;
             run += t;
         }
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        int64_t i = base + r * 32 + lane;
-        if (i < n) {
-            int dg = (kk[r] >> shift) & 255u;
-            int pos = offs[dg * ntiles + blockIdx.x] + wcnt[wid][dg] + loc[r];
-            key_out[pos] = kk[r];
-            val_out[pos] = vv[r];
+    for (int r = 0; r < ITEMS; ++r) {
+        if (base + r * 32 + lane >= s.n) continue;
+        const int pos = wcnt[wid][(kk[r] >> s.shift) & 255u] + loc[r];
+        s.key_out[pos] = kk[r];
+        if constexpr (!LAST) {
+            s.val_out[pos] = vv[r];
+            atomicAdd(&s.hist_next[(int64_t)(pos / kTile) * 256 + ((kk[r] >> (s.shift + 8)) & 255u)], 1);
+        } else {
+            double x[3];
+            load_pos(a, vv[r], x);
+            float w = a.w[vv[r]];
+            if (!isfinite(w)) w = 0.f;
+            if (w < 0.f) *s.negw = 1;
+            s.pts[pos] = make_float4((float)x[0], (float)x[1], (float)x[2], w);
+            if (s.pts64) {
+                s.pts64[3 * (int64_t)pos + 0] = x[0];
+                s.pts64[3 * (int64_t)pos + 1] = x[1];
+                s.pts64[3 * (int64_t)pos + 2] = x[2];
+            }
+            s.orig[pos] = vv[r];
+            if (s.prim_count && vv[r] < s.n_primary) atomicAdd(&s.prim_count[pos / kPrimTile], 1);
         }
     }
 }
 
-// ---- sorted arrays, cell starts, primary list -------------------------------
-
-__global__ void k_gather(IndexArgs a, const int* val, float4* pts, double* pts64, int* orig, int* negw) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= a.n) return;
-    int i = val[p];
-    double x[3];
-    if (a.pos_f64) {
-        const double* q = static_cast<const double*>(a.pos) + 3 * (int64_t)i;
-        x[0] = q[0]; x[1] = q[1]; x[2] = q[2];
-    } else {
-        const float* q = static_cast<const float*>(a.pos) + 3 * (int64_t)i;
-        x[0] = q[0]; x[1] = q[1]; x[2] = q[2];
-    }
-    for (int d = 0; d < 3; ++d)
-        if (!(x[d] >= 0.0 && x[d] < a.g.boxd)) x[d] = 0.0;  // flagged in k_keys
-    float w = a.w[i];
-    if (!isfinite(w)) w = 0.f;
-    if (w < 0.f) *negw = 1;
-    pts[p] = make_float4((float)x[0], (float)x[1], (float)x[2], w);
-    if (pts64) {
-        pts64[3 * p + 0] = x[0];
-        pts64[3 * p + 1] = x[1];
-        pts64[3 * p + 2] = x[2];
-    }
-    orig[p] = i;
-}
+// ---- cell starts, primary list ------------------------------------------------
 
 __global__ void k_cell_start(const unsigned* key, int64_t n, long long ncells, int* cstart) {
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -248,40 +287,57 @@ __global__ void k_cell_start(const unsigned* key, int64_t n, long long ncells, i
     cstart[c] = (int)lo;
 }
 
-__global__ void k_prim_flag(const int* orig, int64_t n, int64_t n_primary, int* flag) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p < n) flag[p] = orig[p] < n_primary ? 1 : 0;
+// Sorted slots of the primaries (original index < n_primary), in slot order: block
+// t compacts the kPrimTile slots of counter t behind the counts before it.
+__global__ void __launch_bounds__(kPrimTile) k_prim_compact(const int* orig, int64_t n, int64_t n_primary,
+                                                            const int* count, int* plist) {
+    __shared__ int sh[32];
+    __shared__ int off;
+    int before = 0;
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += kPrimTile) before += count[t];
+    if (threadIdx.x == 0) off = 0;
+    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if ((threadIdx.x & 31) == 0 && before) atomicAdd(&off, before);
+    const int64_t p = blockIdx.x * (int64_t)kPrimTile + threadIdx.x;
+    const int flag = p < n && orig[p] < n_primary;
+    int tot;
+    const int pre = block_scan_excl(flag, sh, tot);
+    if (flag) plist[off + pre] = (int)p;
 }
 
-__global__ void k_prim_compact(const int* flag, const int* pos, int64_t n, int* plist) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p < n && flag[p]) plist[pos[p]] = (int)p;
-}
-
-__global__ void k_iota_ranges(const int* rstart, const int* rlen, const int* rout, int nr,
-                              int* plist) {
-    // one block per range
-    int r = blockIdx.x;
-    if (r >= nr) return;
-    for (int k = threadIdx.x; k < rlen[r]; k += blockDim.x) plist[rout[r] + k] = rstart[r] + k;
+// Batch: the slot ranges of the catalogs end to end (nr ranges, out ascending).
+__global__ void k_iota_ranges(const int* rstart, const int* rlen, const int* rout, int nr, int64_t n, int* plist) {
+    const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (o >= n) return;
+    int lo = 0, hi = nr - 1;  // last range with out <= o (empty ranges share their start)
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (rout[mid] <= o) lo = mid; else hi = mid - 1;
+    }
+    const int k = (int)o - rout[lo];
+    if (k < rlen[lo]) plist[o] = rstart[lo] + k;
 }
 
 inline int grid_of(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
 }  // namespace
 
-int scan_exclusive(const int* in, int* out, int64_t n, int* tmp, cudaStream_t st) {
-    if (n <= 0) return 0;
-    int nb = grid_of(n, kScanBlock);
-    k_scan_reduce<<<nb, kScanBlock, 0, st>>>(in, n, tmp);
-    k_scan_top<<<1, kScanBlock, 0, st>>>(tmp, nb);
-    k_scan_final<<<nb, kScanBlock, 0, st>>>(in, n, tmp, out);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+namespace {
+template <int ITEMS, bool SCANNED>
+void scatter_pass(const ScatterArgs& s, const IndexArgs& a, bool last, cudaStream_t st) {
+    if (last)
+        k_radix_scatter<ITEMS, SCANNED, true><<<s.ntiles, kSortThreads, 0, st>>>(s, a);
+    else
+        k_radix_scatter<ITEMS, SCANNED, false><<<s.ntiles, kSortThreads, 0, st>>>(s, a);
 }
+}  // namespace
 
-size_t scan_tmp_ints(int64_t n) { return (size_t)grid_of(n, kScanBlock) + 1; }
-
-size_t radix_hist_ints(int64_t n) { return (size_t)256 * grid_of(n, kTile) + 1; }
+// Histograms of up to 4 passes, the primaries' counters, and the scan's block sums.
+size_t index_scratch_ints(int64_t n) {
+    const int64_t tiles = n <= kSmallSort ? grid_of(n, 4 * kSortThreads) : grid_of(n, 16 * kSortThreads);
+    return (size_t)(4 * 256 * tiles + grid_of(n, kPrimTile) + grid_of(256 * tiles, kScanBlock) + 1);
+}
 
 int build_index(IndexBuffers& b, const IndexArgs& a, const int64_t* cat_off_dev, int ncat,
                 long long ncells, int64_t n_primary, const PrimRanges* ranges,
@@ -289,39 +345,71 @@ int build_index(IndexBuffers& b, const IndexArgs& a, const int64_t* cat_off_dev,
     const int64_t n = a.n;
     if (n <= 0) return 0;
     const int T = 256;
-    int launches = 0;
-    k_keys<<<grid_of(n, T), T, 0, st>>>(a, cat_off_dev, ncat, b.key_a, b.val_a, b.status);
+    int launches = 1;
+    const bool small = n <= kSmallSort;
+    const int ntiles = small ? grid_of(n, 4 * kSortThreads) : grid_of(n, 16 * kSortThreads);
+    const int nprim_tiles = grid_of(n, kPrimTile);
+    const int64_t hist = (int64_t)256 * ntiles;
+    int* prim_count = b.scratch + 4 * hist;
+    int* bsum = prim_count + nprim_tiles;
     // LSD radix sort on the bits in use
     int bits = 1;
     while (bits < 32 && ((unsigned long long)1 << bits) <= (unsigned long long)ncells) ++bits;
-    const int ntiles = grid_of(n, kTile);
-    unsigned* kin = b.key_a;
-    int* vin = b.val_a;
-    unsigned* kout = b.key_b;
-    int* vout = b.val_b;
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_radix_hist<<<ntiles, kSortThreads, 0, st>>>(kin, n, shift, ntiles, b.hist);
-        scan_exclusive(b.hist, b.hist_off, (int64_t)256 * ntiles, b.scan_tmp, st);
-        k_radix_scatter<<<ntiles, kSortThreads, 0, st>>>(kin, vin, n, shift, ntiles, b.hist_off,
-                                                         kout, vout);
-        launches += 5;
-        unsigned* tk = kin; kin = kout; kout = tk;
-        int* tv = vin; vin = vout; vout = tv;
+    const int passes = (bits + 7) / 8;
+    if (small)
+        k_keys<4><<<ntiles, kSortThreads, 0, st>>>(a, cat_off_dev, ncat, b.key_a, b.status, b.scratch,
+                                                   b.scratch + hist, 3 * hist + nprim_tiles);
+    else
+        k_keys<16><<<ntiles, kSortThreads, 0, st>>>(a, cat_off_dev, ncat, b.key_a, b.status, b.scratch,
+                                                    b.scratch + hist, 3 * hist + nprim_tiles);
+    const bool subset = !ranges && n_primary < n;
+    ScatterArgs s{};
+    s.key = b.key_a;
+    s.n = n;
+    s.ntiles = ntiles;
+    s.key_out = b.key_b;
+    s.val_out = b.val_a;
+    s.pts = b.pts;
+    s.pts64 = b.pts64;
+    s.orig = b.orig;
+    s.negw = b.status + kNegWeightSlot;
+    s.n_primary = n_primary;
+    s.prim_count = subset ? prim_count : nullptr;
+    for (int p = 0; p < passes; ++p) {
+        s.shift = 8 * p;
+        int* h = b.scratch + p * hist;
+        s.hist = h;
+        s.hist_next = h + hist;
+        const bool last = p + 1 == passes;
+        if (small) {
+            scatter_pass<4, false>(s, a, last, st);
+            launches += 1;
+        } else {
+            const int nb = grid_of(hist, kScanBlock);
+            k_scan_reduce<<<nb, kScanBlock, 0, st>>>(h, ntiles, hist, bsum);
+            k_scan_top<<<1, kScanBlock, 0, st>>>(bsum, nb);
+            k_scan_final<<<nb, kScanBlock, 0, st>>>(h, ntiles, hist, bsum);
+            scatter_pass<16, true>(s, a, last, st);
+            launches += 4;
+        }
+        // the other buffers for the next pass
+        unsigned* kin = const_cast<unsigned*>(s.key);
+        s.key = s.key_out;
+        s.key_out = kin;
+        int* vin = s.val ? const_cast<int*>(s.val) : b.val_b;
+        s.val = s.val_out;
+        s.val_out = vin;
     }
-    b.key_sorted = kin;
-    k_gather<<<grid_of(n, T), T, 0, st>>>(a, vin, b.pts, b.pts64, b.orig, b.status + kNegWeightSlot);
-    k_cell_start<<<(int)((ncells + 1 + T - 1) / T), T, 0, st>>>(kin, n, ncells, b.cstart);
-    launches += 3;
+    b.key_sorted = const_cast<unsigned*>(s.key);
+    k_cell_start<<<(int)((ncells + 1 + T - 1) / T), T, 0, st>>>(b.key_sorted, n, ncells, b.cstart);
+    launches += 1;
     // primary list
     if (ranges) {
-        k_iota_ranges<<<ranges->n, 256, 0, st>>>(ranges->start, ranges->len, ranges->out,
-                                                 ranges->n, b.plist);
+        k_iota_ranges<<<grid_of(n, T), T, 0, st>>>(ranges->start, ranges->len, ranges->out, ranges->n, n, b.plist);
         launches += 1;
-    } else if (n_primary < n) {
-        k_prim_flag<<<grid_of(n, T), T, 0, st>>>(b.orig, n, n_primary, vout);
-        scan_exclusive(vout, b.hist_off, n, b.scan_tmp, st);
-        k_prim_compact<<<grid_of(n, T), T, 0, st>>>(vout, b.hist_off, n, b.plist);
-        launches += 5;
+    } else if (subset) {
+        k_prim_compact<<<nprim_tiles, kPrimTile, 0, st>>>(b.orig, n, n_primary, prim_count, b.plist);
+        launches += 1;
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {

@@ -86,9 +86,7 @@ struct IndexArgs {
 struct IndexBuffers {
     unsigned *key_a, *key_b;
     int *val_a, *val_b;
-    int* hist;         // 256 * ntiles
-    int* hist_off;     // max(256 * ntiles, n) + 1
-    int* scan_tmp;
+    int* scratch;      // index_scratch_ints(n)
     float4* pts;
     double* pts64;     // null unless FP64 input
     int* orig;
@@ -105,9 +103,7 @@ struct PrimRanges {    // batch mode: plist = concatenated slot ranges
 };
 int build_index(IndexBuffers& b, const IndexArgs& a, const int64_t* cat_off_dev, int ncat,
                 long long ncells, int64_t n_primary, const PrimRanges* ranges, cudaStream_t st);
-int scan_exclusive(const int* in, int* out, int64_t n, int* tmp, cudaStream_t st);
-size_t scan_tmp_ints(int64_t n);
-size_t radix_hist_ints(int64_t n);
+size_t index_scratch_ints(int64_t n);
 
 // ---- pair.cu ---------------------------------------------------------------
 struct PairArgs {
