@@ -116,10 +116,11 @@ struct g3pcf_plan_s {
     int kflush = 16;
     // device buffers
     DevBuf key_a, key_b, val_a, val_b, idx_scratch, pts, pts64, orig, cstart, plist;
-    DevBuf small;       // status, queue
-    DevBuf counts, A, partials, d_tiles, d_segs, d_segfirst, d_colmap, d_colscale, d_catoff;
+    DevBuf small;       // status block (kStatusBytes), then the pair counts
+    DevBuf A, partials, d_tiles, d_colmap, d_colscale, d_catoff;
     DevBuf d_colconv, d_colcoef, d_slotconv, d_slotcoef, d_monoexp, d_monoconv, d_monoidx, d_monocoef;
-    DevBuf d_ranges, d_tiles_tc, d_cats, d_mreal, d_V, d_bintab, wrow, d_vblk, d_strips_tc, d_items;
+    DevBuf d_ranges, d_tiles_tc, d_mreal, d_V, d_bintab, wrow, d_vblk, d_strips_tc;
+    DevBuf d_tables;    // segments, catalogs and work items of a contraction, first segments
     DevBuf d_bop, d_bblk, d_bcat;
     DevBuf d_slotcoefdf, d_mrealdf, d_Vdf, d_colcoefdf, d_mnorm;
     int64_t opt_chunk = 0;   // G3PCF_OPT_CHUNK_ROWS
@@ -152,9 +153,12 @@ struct g3pcf_plan_s {
     bool exact_alm = false;  // this forward runs with G3PCF_F_KEEP_ALM
     int gl_events = 0;  // events the capture run will record
     DevBuf l_gbase, l_scantmp, l_passq;
-    // events around every k_scan / k_accum launch of the last forward (4 per pass)
-    std::vector<cudaEvent_t> lev;
+    // events around every k_scan / k_accum launch of the last forward: start, middle
+    // and end of each pass (levq: the handles in order; the last end of a forward that
+    // is not chunked is ev[2])
+    std::vector<cudaEvent_t> lev, levq;
     int lev_used = 0;
+    bool pair_end_recorded = false;
     // per chunk of primaries: pair stage done, contraction done (stats [1], [2])
     std::vector<cudaEvent_t> cev;
     int cev_used = 0;
@@ -236,7 +240,7 @@ int setup_device(g3pcf_plan_t P) {
     CK(cudaGetDeviceProperties(&prop, dev));
     P->device = dev;
     P->nsm = prop.multiProcessorCount;
-    CK(cudaHostAlloc(reinterpret_cast<void**>(&P->h_status), 64, cudaHostAllocDefault));
+    CK(cudaHostAlloc(reinterpret_cast<void**>(&P->h_status), 256, cudaHostAllocDefault));
     for (auto& e : P->ev) CK(cudaEventCreate(&e));
     return 0;
 }
@@ -589,6 +593,11 @@ int ensure(g3pcf_plan_t P, DevBuf& b, size_t bytes, const char* what) {
     return 0;
 }
 
+// pair counts of the last call (behind the status block, so that one memset clears both)
+unsigned long long* counts_of(g3pcf_plan_t P) {
+    return reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(P->small.p) + kStatusBytes);
+}
+
 int read_status(g3pcf_plan_t P) {
     int s = P->h_status[0];
     if (s & kStatusRange)
@@ -617,6 +626,47 @@ int ensure_events(g3pcf_plan_t P, int n) {
     return 0;
 }
 
+// One pass of the pair lists: scan, then accumulate (mode 0), the adjoint pair pass
+// (1) or, recomputing, accumulate, V = M A and the adjoint pair pass (2).  reset: the
+// work counters have been used since they were cleared; end2: the pass's end is ev[2].
+int run_list_pass(g3pcf_plan_t P, ListArgs& la, const PairArgs& pa, int mode, bool reset, bool end2,
+                  cudaStream_t st) {
+    if (reset) CK(cudaMemsetAsync(pa.status + kQueueSlot, 0, (kCursorSlot + 1 - kQueueSlot) * sizeof(int), st));
+    cudaEvent_t* ev = P->lev.data() + P->lev_used;
+    P->lev_used += 3;
+    P->launches += 2;
+    CK(cudaEventRecord(ev[0], st));
+    la.queue = pa.status + kQueueSlot;
+    if (launch_scan(la, P->nsm, st) != 0)
+        return fail(G3PCF_ERR_CUDA, "pair scan launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+    CK(cudaEventRecord(ev[1], st));
+    la.queue = pa.status + kQueueSlot + 1;
+    if (mode == 2) {
+        // recompute: the chunk-local multipole rows of this pass and their V = M A (in FP32
+        // also their primary-weight terms), then the adjoint pair pass over the same lists
+        P->launches += 2;
+        int vr = launch_accum(P->lmax, la, P->nsm, st);
+        if (vr == 0)
+            vr = la.precise
+                     ? launch_vgemm_rows_df(la.A, la.RLP, la.RL, la.qa - la.q0, la.qb - la.q0, P->d_mrealdf.as<float2>(),
+                                            P->d_mnorm.as<float>(), P->nbins, P->lmax, P->d_Vdf.as<float2>(), st)
+                     : launch_vgemm_rows(la.A, la.RLP, la.RL, la.qa - la.q0, la.qb - la.q0, P->d_mreal.as<float>(),
+                                         P->nbins, P->lmax, P->d_V.as<float>(), pa.dw, la.plist, la.orig, la.q0, st);
+        if (vr != 0)
+            return fail(G3PCF_ERR_CUDA, "adjoint recompute launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+        la.queue = pa.status + kQueueSlot + 2;
+    }
+    if ((mode >= 1 ? launch_adj(P->lmax, la, P->nsm, st)
+                   : (P->opt_basis == 1 ? launch_mono(P->lmax, la, P->nsm, st)
+                                        : launch_accum(P->lmax, la, P->nsm, st))) != 0)
+        return fail(G3PCF_ERR_CUDA, "pair accumulate launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+    const cudaEvent_t end = end2 ? P->ev[2] : ev[2];
+    CK(cudaEventRecord(end, st));
+    if (end2) P->pair_end_recorded = true;
+    P->levq.insert(P->levq.end(), {ev[0], ev[1], end});
+    return G3PCF_OK;
+}
+
 // Forward pair stage through pair lists for the primaries [pa.q0, pa.nprim):
 // count candidates, bring the per-primary chunk bounds to the host, split the
 // range into passes whose lists fit the pool, then scan + accumulate each pass.
@@ -628,17 +678,9 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         ensure(P, P->l_base, 4 * (size_t)qb, "pair-list bounds") ||
         ensure(P, P->l_nch, 4 * (size_t)qb, "pair-list bounds"))
         return G3PCF_ERR_ALLOC;
-    if ((size_t)nq > P->h_list_cap) {
-        if (P->h_need) cudaFreeHost(P->h_need);
-        if (P->h_base) cudaFreeHost(P->h_base);
-        P->h_need = P->h_base = nullptr;
-        P->h_list_cap = 0;
-        if (cudaHostAlloc(reinterpret_cast<void**>(&P->h_need), 4 * nq, cudaHostAllocDefault) != cudaSuccess ||
-            cudaHostAlloc(reinterpret_cast<void**>(&P->h_base), 4 * nq, cudaHostAllocDefault) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(G3PCF_ERR_ALLOC, "pinned host allocation of %lld bytes failed", (long long)(8 * nq));
-        }
-        P->h_list_cap = (size_t)nq;
+    if (qa > 0) {  // a later chunk of primaries: the work counters and the count's totals
+        CK(cudaMemsetAsync(pa.status + kQueueSlot, 0, (kCursorSlot + 1 - kQueueSlot) * sizeof(int), st));
+        CK(cudaMemsetAsync(pa.status + kTotalSlot, 0, (kMostSlot + 1 - kTotalSlot) * sizeof(int), st));
     }
     ListArgs la{};
     la.pts = pa.pts;
@@ -647,6 +689,7 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     la.cstart = pa.cstart;
     la.plist = pa.plist;
     la.key = pa.key;
+    la.ncat = P->last_ncat;
     la.q0 = pa.q0;
     la.chunked = pa.chunked;
     la.wrow = pa.wrow;
@@ -657,7 +700,6 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     la.colcoef = P->d_colcoef.as<float>();
     la.RL = pa.RL;
     la.counts = pa.counts;
-    la.queue = pa.queue;
     la.status = pa.status;
     la.g = pa.g;
     la.bins = pa.bins;
@@ -683,7 +725,6 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     la.nchunks = P->l_nch.as<int>();
     la.qa = qa;
     la.qb = qb;
-    la.ncand = reinterpret_cast<unsigned long long*>(pa.status + 24);  // zeroed with the status word
     // plain forwards: the scan writes each pair's direction and weight (16 bytes)
     // instead of its list entry (4 bytes), unless that leaves passes too small to
     // fill the chip (below)
@@ -705,12 +746,16 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         const ListWarm wm = P->gl_warm[P->gl_idx++];
         dirs = wm.dirs;
         const int64_t C = (int64_t)(P->l_pool.bytes / (dirs ? 512 : 128));
+        // one pass where the pool holds the lists with headroom, else passes planned
+        // on the device
+        const bool one = wm.total + wm.total / 4 <= C;
         int64_t slack = 0, stride = 0;
-        int npass = 0;
-        graph_plan_sizes(C, wm.total, wm.most, P->nbins, slack, stride, npass);
-        if (stride < 1 || (int64_t)P->l_tag.bytes / 4 < C || (int64_t)P->l_ord.bytes / 4 < C ||
-            P->l_gbase.bytes < 8 * (size_t)nq || P->l_passq.bytes < 4 * (size_t)(npass + 1) ||
-            P->l_scantmp.bytes < plan_scan_tmp_bytes(nq) || (int)P->lev.size() < P->lev_used + 4 * npass) {
+        int npass = 1;
+        if (!one) graph_plan_sizes(C, wm.total, wm.most, P->nbins, slack, stride, npass);
+        if (C < 1 || (int64_t)P->l_tag.bytes / 4 < C || (int64_t)P->l_ord.bytes / 4 < C ||
+            (!one && (stride < 1 || P->l_gbase.bytes < 8 * (size_t)nq ||
+                      P->l_passq.bytes < 4 * (size_t)(npass + 1) || P->l_scantmp.bytes < plan_scan_tmp_bytes(nq))) ||
+            (int)P->lev.size() < P->lev_used + 3 * npass) {
             ++P->launches;  // the warm-up did not size the plan (cannot happen): the fused kernel
             if (launch_pair(P->lmax, pa, P->nsm, st) != 0)
                 return fail(G3PCF_ERR_CUDA, "pair kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -723,25 +768,18 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         ++P->launches;
         if (launch_count(la, P->nsm, st) != 0)
             return fail(G3PCF_ERR_CUDA, "pair count launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-        P->launches += 5;
-        if (launch_plan(la.need, P->l_gbase.as<long long>(), P->l_scantmp.as<long long>(), qa, qb, stride,
-                        (int)slack, npass, P->l_base.as<int>(), P->l_passq.as<int>(), pa.status, st) != 0)
-            return fail(G3PCF_ERR_CUDA, "pair-list plan launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+        if (one) {
+            la.cursor = pa.status + kCursorSlot;
+            la.cap = (int)std::min<int64_t>(C, (int64_t)1 << 30);
+        } else {
+            P->launches += 5;
+            if (launch_plan(la.need, P->l_gbase.as<long long>(), P->l_scantmp.as<long long>(), qa, qb, stride,
+                            (int)slack, npass, P->l_base.as<int>(), P->l_passq.as<int>(), pa.status, st) != 0)
+                return fail(G3PCF_ERR_CUDA, "pair-list plan launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+        }
         for (int k = 0; k < npass; ++k) {
-            la.qrange = P->l_passq.as<int>() + k;
-            cudaEvent_t* ev = P->lev.data() + P->lev_used;
-            P->lev_used += 4;
-            CK(cudaMemsetAsync(la.queue, 0, sizeof(int), st));
-            P->launches += 2;
-            CK(cudaEventRecord(ev[0], st));
-            if (launch_scan(la, P->nsm, st) != 0)
-                return fail(G3PCF_ERR_CUDA, "pair scan launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-            CK(cudaEventRecord(ev[1], st));
-            CK(cudaMemsetAsync(la.queue, 0, sizeof(int), st));
-            CK(cudaEventRecord(ev[2], st));
-            if ((P->opt_basis == 1 ? launch_mono(P->lmax, la, P->nsm, st) : launch_accum(P->lmax, la, P->nsm, st)) != 0)
-                return fail(G3PCF_ERR_CUDA, "pair accumulate launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-            CK(cudaEventRecord(ev[3], st));
+            if (!one) la.qrange = P->l_passq.as<int>() + k;
+            if (int r = run_list_pass(P, la, pa, mode, k > 0, !pa.chunked && k + 1 == npass, st)) return r;
         }
         P->stats[10] += (double)npass;
         return G3PCF_OK;
@@ -749,28 +787,33 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     ++P->launches;
     if (launch_count(la, P->nsm, st) != 0)
         return fail(G3PCF_ERR_CUDA, "pair count launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-    CK(cudaMemcpyAsync(P->h_need, la.need + qa, 4 * nq, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(P->h_status + 8, la.ncand, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(P->h_status + 12, pa.status + kNegWeightSlot, sizeof(int), cudaMemcpyDeviceToHost, st));
+    // the totals of the count (and the negative-weight flag) come to the host: what the
+    // pool has to hold
+    CK(cudaMemcpyAsync(P->h_status + kQueueSlot, pa.status + kQueueSlot, 64, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    P->stats[9] = (double)*reinterpret_cast<unsigned long long*>(P->h_status + 8);
+    auto h64 = [&](int slot) {
+        unsigned long long v;
+        std::memcpy(&v, P->h_status + slot, sizeof v);
+        return v;
+    };
+    P->stats[9] = (double)h64(kCandSlot);
     // the bf16 operands are sqrt(w) A: with a negative weight the contraction
     // forms its operands from the FP32 rows instead
-    if (la.bop && P->h_status[12] != 0) la.bop = nullptr;
+    if (la.bop && P->h_status[kNegWeightSlot] != 0) la.bop = nullptr;
     la.skip_a = (la.bop && !P->exact_alm) ? 1 : 0;
     if (mode == 0) P->direct_used = la.bop != nullptr;
-    // pool capacity (per chunk: 128 bytes of entries, a tag and a list int)
-    int64_t total = 0, most = 0;
-    for (int64_t k = 0; k < nq; ++k) {
-        total += P->h_need[k];
-        most = std::max<int64_t>(most, P->h_need[k]);
-    }
+    // pool capacity (per chunk: 512 bytes of records or 128 of entries, a tag and a list int)
+    const int64_t total = (int64_t)h64(kTotalSlot), most = P->h_status[kMostSlot];
     double budget = (double)P->opt_list_bytes;
+    const size_t own = P->l_pool.bytes + P->l_tag.bytes + P->l_ord.bytes;
     if (budget <= 0) {
-        size_t fr = 0, tot = 0;
-        CK(cudaMemGetInfo(&fr, &tot));
-        budget = 0.4 * (double)(fr + P->l_pool.bytes + P->l_tag.bytes + P->l_ord.bytes);
-        if (budget > 32e9) budget = 32e9;
+        // what the plan already holds is enough, or a share of the free memory
+        budget = std::min(32e9, (double)own);
+        if ((dirs ? 520.0 : 136.0) * (double)total > budget || P->warm_for_graph) {
+            size_t fr = 0, tot = 0;
+            CK(cudaMemGetInfo(&fr, &tot));
+            budget = std::min(32e9, 0.4 * (double)(fr + own));
+        }
     }
     // Direction records (520 bytes per chunk against 136) make more and smaller
     // passes.  Below about 28 primaries per SM and pass, list entries are faster: on
@@ -809,9 +852,32 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
             ensure(P, P->l_scantmp, plan_scan_tmp_bytes(nq), "pair-list plan") ||
             ensure(P, P->l_passq, 4 * (size_t)(npass + 1), "pair-list plan"))
             return G3PCF_ERR_ALLOC;
-        P->gl_events += 4 * npass;
+        P->gl_events += 3 * npass;
         if (int r = ensure_events(P, P->gl_events)) return r;
     }
+    if (total <= cap) {  // one pass: k_scan takes its chunks from a counter
+        la.cursor = pa.status + kCursorSlot;
+        la.cap = (int)cap;
+        if (int r = ensure_events(P, P->lev_used + 3)) return r;
+        if (int r = run_list_pass(P, la, pa, mode, false, !pa.chunked && mode == 0, st)) return r;
+        P->stats[10] += 1.0;
+        return G3PCF_OK;
+    }
+    // several passes: the bounds come to the host, which places every primary's chunks
+    if ((size_t)nq > P->h_list_cap) {
+        if (P->h_need) cudaFreeHost(P->h_need);
+        if (P->h_base) cudaFreeHost(P->h_base);
+        P->h_need = P->h_base = nullptr;
+        P->h_list_cap = 0;
+        if (cudaHostAlloc(reinterpret_cast<void**>(&P->h_need), 4 * nq, cudaHostAllocDefault) != cudaSuccess ||
+            cudaHostAlloc(reinterpret_cast<void**>(&P->h_base), 4 * nq, cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(G3PCF_ERR_ALLOC, "pinned host allocation of %lld bytes failed", (long long)(8 * nq));
+        }
+        P->h_list_cap = (size_t)nq;
+    }
+    CK(cudaMemcpyAsync(P->h_need, la.need + qa, 4 * nq, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
     std::vector<int> cuts{qa};
     int64_t acc = 0;
     for (int64_t k = 0; k < nq; ++k) {
@@ -828,39 +894,9 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         la.qa = cuts[k];
         la.qb = cuts[k + 1];
         if (la.qb <= la.qa) continue;
-        if (int r = ensure_events(P, P->lev_used + 4)) return r;
-        cudaEvent_t* ev = P->lev.data() + P->lev_used;
-        P->lev_used += 4;
-        CK(cudaMemsetAsync(la.queue, 0, sizeof(int), st));
-        ++P->launches;
-        CK(cudaEventRecord(ev[0], st));
-        if (launch_scan(la, P->nsm, st) != 0)
-            return fail(G3PCF_ERR_CUDA, "pair scan launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-        CK(cudaEventRecord(ev[1], st));
-        CK(cudaMemsetAsync(la.queue, 0, sizeof(int), st));
-        ++P->launches;
-        CK(cudaEventRecord(ev[2], st));
-        if (mode == 2) {
-            // recompute: the chunk-local multipole rows of this pass, their V = M A and
-            // primary-weight terms, then the adjoint pair pass over the same lists
-            P->launches += 2;
-            int vr = launch_accum(P->lmax, la, P->nsm, st);
-            if (vr == 0)
-                vr = la.precise ? launch_vgemm_rows_df(la.A, la.RLP, la.RL, la.qa - la.q0, la.qb - la.q0,
-                                                      P->d_mrealdf.as<float2>(), P->d_mnorm.as<float>(), P->nbins, P->lmax,
-                                                      P->d_Vdf.as<float2>(), st)
-                                : launch_vgemm_rows(la.A, la.RLP, la.RL, la.qa - la.q0, la.qb - la.q0,
-                                                    P->d_mreal.as<float>(), P->nbins, P->lmax, P->d_V.as<float>(),
-                                                    pa.dw, la.plist, la.orig, la.q0, st);
-            if (vr != 0)
-                return fail(G3PCF_ERR_CUDA, "adjoint recompute launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-            CK(cudaMemsetAsync(la.queue, 0, sizeof(int), st));
-        }
-        if ((mode >= 1 ? launch_adj(P->lmax, la, P->nsm, st)
-                       : (P->opt_basis == 1 ? launch_mono(P->lmax, la, P->nsm, st)
-                                            : launch_accum(P->lmax, la, P->nsm, st))) != 0)
-            return fail(G3PCF_ERR_CUDA, "pair accumulate launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-        CK(cudaEventRecord(ev[3], st));
+        if (int r = ensure_events(P, P->lev_used + 3)) return r;
+        const bool last = !pa.chunked && mode == 0 && k + 2 == cuts.size();
+        if (int r = run_list_pass(P, la, pa, mode, k > 0, last, st)) return r;
     }
     P->stats[10] += (double)(cuts.size() - 1);
     return G3PCF_OK;
@@ -875,9 +911,12 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
     const int64_t zs = zsize_of(B, P->lmax);
     P->have_forward = false;
     P->have_alm = false;
+    P->last_ncat = c.ncat;
     P->launches = 0;
     P->stats[9] = P->stats[10] = 0.0;
     P->lev_used = 0;
+    P->levq.clear();
+    P->pair_end_recorded = false;
     P->exact_alm = (c.flags & G3PCF_F_KEEP_ALM) != 0;
     if (P->capturing) {
         P->gl_idx = 0;
@@ -889,13 +928,10 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
     P->cev_used = 0;
     CK(cudaEventRecord(P->ev[0], st));
     // zero outputs and counters
-    if (ensure(P, P->small, 256, "status")) return G3PCF_ERR_ALLOC;
+    const size_t count_bytes = sizeof(unsigned long long) * B * c.ncat;
+    if (ensure(P, P->small, kStatusBytes + count_bytes, "status")) return G3PCF_ERR_ALLOC;
     int* d_status = P->small.as<int>();
-    int* d_queue = d_status + 16;
-    CK(cudaMemsetAsync(P->small.p, 0, 256, st));
-    if (ensure(P, P->counts, sizeof(unsigned long long) * B * c.ncat + 8, "counts")) return G3PCF_ERR_ALLOC;
-    CK(cudaMemsetAsync(P->counts.p, 0, sizeof(unsigned long long) * B * c.ncat, st));
-    CK(cudaMemsetAsync(c.zeta, 0, sizeof(double) * 2 * zs * c.ncat, st));
+    CK(cudaMemsetAsync(P->small.p, 0, kStatusBytes + count_bytes, st));
     // density for the grid: pair-weighted over catalogs
     double num = 0, den = 0;
     for (int k = 0; k < c.ncat; ++k) {
@@ -911,6 +947,7 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
     P->stats[7] = (double)P->rmax / (P->box / g.nc);
 
     int64_t nprim = 0;
+    bool reduced = false;
     if (n > 0) {
         // ---- workspace
         if (ensure(P, P->key_a, 4 * n, "keys") || ensure(P, P->key_b, 4 * n, "keys") ||
@@ -991,7 +1028,9 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
         const bool fixed = P->capturing && P->fixed_chunk > 0;
         double budget = 0.0;
         const double per_row = 4.0 * P->RLP + 4.0;
-        if (ops || (c.ncat == 1 && P->opt_chunk <= 0 && !fixed)) {
+        // (rows that fit what the plan already holds need no query)
+        const bool held = !ops && (double)P->A.bytes >= per_row * (double)rows_all;
+        if (ops || (c.ncat == 1 && P->opt_chunk <= 0 && !fixed && !held)) {
             size_t fr = 0, tot = 0;
             CK(cudaMemGetInfo(&fr, &tot));
             budget = 0.4 * (double)fr;
@@ -1003,7 +1042,7 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
                 C = P->opt_chunk;
             } else if (fixed) {
                 C = P->fixed_chunk;
-            } else {
+            } else if (!held) {
                 C = (int64_t)(budget / per_row) / KB * KB;
                 if (C < KB) C = KB;
             }
@@ -1085,29 +1124,68 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
             total_segs += (int)csegs[ch].size();
         }
         segfirst[c.ncat] = total_segs;
+        // tables of every chunk's contraction behind the first-segment table, one copy per
+        // chunk: segments, catalogs {padded start, first A row, length, 0}, work items
+        // (every strip over every virtual segment of every catalog, step[s] consecutive
+        // segments at a time)
+        struct Tables {
+            size_t segs, cats, items, bytes;
+            int nitems;
+        };
+        auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
+        const size_t tab0 = align(4 * (size_t)(c.ncat + 1));
+        std::vector<Tables> ctab(nchunks);
+        std::vector<std::vector<unsigned char>> cblob(nchunks);
         if (total_segs > 0) {
-            size_t max_segs = 0, max_cats = 1;
+            size_t most = 0;
             for (int64_t ch = 0; ch < nchunks; ++ch) {
-                max_segs = std::max(max_segs, csegs[ch].size());
-                max_cats = std::max(max_cats, ccats[ch].size());
+                const std::vector<Segment>& segs = csegs[ch];
+                const int nsegs = (int)segs.size();
+                std::vector<TcItem> items;
+                if (use_tc) {
+                    int kc = 0;  // catalog index within this chunk
+                    for (int s0 = 0; s0 < nsegs; ++kc) {
+                        int s1 = s0;
+                        while (s1 < nsegs && segs[s1].cat == segs[s0].cat) ++s1;
+                        const int* stp = csteps[ch].data() + (size_t)kc * nstrips;
+                        for (int k = 0; k < nstrips; ++k) {
+                            const int step = stp[k];
+                            for (int v = s0; v < s1; v += step)
+                                items.push_back(TcItem{k, v, std::min(step, s1 - v), 0});
+                        }
+                        s0 = s1;
+                    }
+                }
+                Tables& t = ctab[ch];
+                t.segs = 0;
+                t.cats = align(sizeof(Segment) * nsegs);
+                t.items = t.cats + align(4 * ccats[ch].size());
+                t.bytes = t.items + align(sizeof(TcItem) * items.size());
+                t.nitems = (int)items.size();
+                cblob[ch].assign(t.bytes, 0);
+                if (nsegs) std::memcpy(cblob[ch].data(), segs.data(), sizeof(Segment) * nsegs);
+                if (!ccats[ch].empty()) std::memcpy(cblob[ch].data() + t.cats, ccats[ch].data(), 4 * ccats[ch].size());
+                if (!items.empty()) std::memcpy(cblob[ch].data() + t.items, items.data(), sizeof(TcItem) * items.size());
+                most = std::max(most, t.bytes);
             }
-            if (ensure(P, P->d_segs, sizeof(Segment) * max_segs, "segments") ||
-                ensure(P, P->d_segfirst, 4 * (c.ncat + 1), "segments") ||
+            if (ensure(P, P->d_tables, tab0 + most, "contraction tables") ||
                 ensure(P, P->partials, sizeof(double) * (size_t)part_stride * total_segs, "partials"))
                 return G3PCF_ERR_ALLOC;
-            if (use_tc && ensure(P, P->d_cats, 4 * max_cats, "catalog table")) return G3PCF_ERR_ALLOC;
-            UP(P->d_segfirst.p, segfirst.data(), 4 * (c.ncat + 1));
+            std::vector<unsigned char> first(tab0 + ctab[0].bytes, 0);
+            std::memcpy(first.data(), segfirst.data(), 4 * (size_t)(c.ncat + 1));
+            if (ctab[0].bytes) std::memcpy(first.data() + tab0, cblob[0].data(), ctab[0].bytes);
+            UP(P->d_tables.p, first.data(), first.size());
         }
         // per-chunk stage events (created outside a capture; a capture that finds
         // too few keeps the single-span timing)
         P->cev_used = 0;
-        if (!P->capturing)
+        if (!P->capturing && nchunks > 1)
             while ((int64_t)P->cev.size() < 2 * nchunks) {
                 cudaEvent_t e;
                 CK(cudaEventCreate(&e));
                 P->cev.push_back(e);
             }
-        const bool chunk_events = (int64_t)P->cev.size() >= 2 * nchunks;
+        const bool chunk_events = nchunks > 1 && (int64_t)P->cev.size() >= 2 * nchunks;
         // bf16 tensor-core operands written by the pair stage (one pass of the
         // multipoles, list path, Chebyshev basis, outside a capture): rows in the
         // padded catalog coordinates of the contraction, padding rows zeroed
@@ -1128,7 +1206,6 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
         int seg_base = 0;
         for (int64_t ch = 0; ch < nchunks; ++ch) {
             const int64_t q0 = ch * C, q1 = chunked ? std::min(rows_all, q0 + C) : nprim;
-            if (ch > 0) CK(cudaMemsetAsync(d_queue, 0, sizeof(int), st));
             if (nprim > 0 && q1 > q0) {
                 PairArgs pa{};
                 pa.pts = ib.pts;
@@ -1147,8 +1224,8 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
                 pa.colmap = P->d_colmap.as<int>();
                 pa.colscale = P->d_colscale.as<float>();
                 pa.RL = P->RL;
-                pa.counts = P->counts.as<unsigned long long>();
-                pa.queue = d_queue;
+                pa.counts = counts_of(P);
+                pa.queue = d_status + kQueueSlot;
                 pa.status = d_status;
                 pa.kflush = P->kflush;
                 pa.g = g;
@@ -1166,50 +1243,36 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
                     if (int r = run_pair_lists(P, pa, st)) return r;
                 } else {
                     ++P->launches;
+                    if (ch > 0) CK(cudaMemsetAsync(pa.queue, 0, sizeof(int), st));
                     if (launch_pair(P->lmax, pa, P->nsm, st) != 0)
                         return fail(G3PCF_ERR_CUDA, "pair kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
                 }
             }
-            if (ch == 0) CK(cudaEventRecord(P->ev[2], st));
+            if (ch == 0 && !P->pair_end_recorded) CK(cudaEventRecord(P->ev[2], st));
             if (chunk_events) CK(cudaEventRecord(P->cev[2 * ch], st));
             const std::vector<Segment>& segs = csegs[ch];
             const int nsegs = (int)segs.size();
             if (nsegs > 0) {
                 double* part = P->partials.as<double>() + (size_t)seg_base * part_stride;
-                UP(P->d_segs.p, segs.data(), sizeof(Segment) * nsegs);
+                const Tables& t = ctab[ch];
+                unsigned char* d_tab = static_cast<unsigned char*>(P->d_tables.p) + tab0;
+                if (ch > 0) UP(d_tab, cblob[ch].data(), t.bytes);
+                const Segment* d_segs = reinterpret_cast<const Segment*>(d_tab + t.segs);
+                const int4* d_cats = reinterpret_cast<const int4*>(d_tab + t.cats);
+                const TcItem* d_items = reinterpret_cast<const TcItem*>(d_tab + t.items);
                 if (use_tc) {
-                    UP(P->d_cats.p, ccats[ch].data(), 4 * ccats[ch].size());
                     P->launches += 1;
-                    // work items: every strip over every virtual segment of every
-                    // catalog, step[s] consecutive segments at a time (planned above)
-                    std::vector<TcItem> items;
-                    int kc = 0;  // catalog index within this chunk
-                    for (int s0 = 0; s0 < nsegs; ++kc) {
-                        int s1 = s0;
-                        while (s1 < nsegs && segs[s1].cat == segs[s0].cat) ++s1;
-                        const int* stp = csteps[ch].data() + (size_t)kc * nstrips;
-                        for (int k = 0; k < nstrips; ++k) {
-                            const int step = stp[k];
-                            for (int v = s0; v < s1; v += step)
-                                items.push_back(TcItem{k, v, std::min(step, s1 - v), 0});
-                        }
-                        s0 = s1;
-                    }
-                    if (ensure(P, P->d_items, sizeof(TcItem) * items.size(), "tensor-core work items"))
-                        return G3PCF_ERR_ALLOC;
-                    UP(P->d_items.p, items.data(), sizeof(TcItem) * items.size());
                     // the rows of A written by this pass: the map reads zeros past them, so
                     // the padding primaries of the last k-block never meet stale memory
                     const int64_t rows_written = chunked ? q1 - q0 : rows_all;
                     const int rc =
                         P->direct_used
                             ? launch_contract_tc_op(bop, P->RLPb, cpad[ch], d_tl,
-                                                    P->d_strips_tc.as<TcStrip>(), P->d_items.as<TcItem>(),
-                                                    (int)items.size(), P->d_segs.as<Segment>(), part, part_stride,
+                                                    P->d_strips_tc.as<TcStrip>(), d_items, t.nitems, d_segs, part,
+                                                    part_stride,
                                                     d_status, st, P->test_tc_timeout)
                             : launch_contract_tc(P->A.as<float>(), P->RLP, P->RL, rows_written, P->wrow.as<float>(),
-                                                 P->d_cats.as<int4>(), d_tl, P->d_strips_tc.as<TcStrip>(),
-                                                 P->d_items.as<TcItem>(), (int)items.size(), P->d_segs.as<Segment>(),
+                                                 d_cats, d_tl, P->d_strips_tc.as<TcStrip>(), d_items, t.nitems, d_segs,
                                                  part, part_stride, d_status + kNegWeightSlot, d_status, st,
                                                  P->test_tc_timeout);
                     if (rc == -2) return fail(G3PCF_ERR_CUDA, "cuTensorMapEncodeTiled unavailable or failed");
@@ -1218,7 +1281,7 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
                 } else {
                     P->launches += 1;
                     if (launch_contract_fp32(P->A.as<float>(), P->RLP, P->wrow.as<float>(), d_tl, ntiles,
-                                             P->d_segs.as<Segment>(), nsegs, part, part_stride, st) != 0)
+                                             d_segs, nsegs, part, part_stride, st) != 0)
                         return fail(G3PCF_ERR_CUDA, "contraction launch failed: %s", cudaGetErrorString(cudaGetLastError()));
                 }
             }
@@ -1229,9 +1292,11 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
         CK(cudaEventRecord(P->ev[3], st));
         if (total_segs > 0) {
             P->launches += 1;
-            if (launch_reduce(P->partials.as<double>(), part_stride, P->d_segfirst.as<int>(), c.ncat,
-                              B, P->lmax, d_tl, T, c.zeta, st, use_tc ? 1 : 0) != 0)
+            // (writes every entry of zeta, and the pair counts to the caller's array)
+            if (launch_reduce(P->partials.as<double>(), part_stride, P->d_tables.as<int>(), c.ncat,
+                              B, P->lmax, d_tl, T, c.zeta, st, use_tc ? 1 : 0, counts_of(P), c.counts) != 0)
                 return fail(G3PCF_ERR_CUDA, "reduction launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+            reduced = true;
         }
         P->last_chunked = chunked;
     } else {
@@ -1240,8 +1305,9 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
         CK(cudaEventRecord(P->ev[3], st));
     }
     CK(cudaEventRecord(P->ev[4], st));
-    if (c.counts) {
-        CK(cudaMemcpyAsync(c.counts, P->counts.p, sizeof(int64_t) * B * c.ncat, cudaMemcpyDeviceToDevice, st));
+    if (!reduced) {  // nothing to reduce: zeta is 0
+        CK(cudaMemsetAsync(c.zeta, 0, sizeof(double) * 2 * zs * c.ncat, st));
+        if (c.counts) CK(cudaMemcpyAsync(c.counts, counts_of(P), count_bytes, cudaMemcpyDeviceToDevice, st));
     }
     CK(cudaMemcpyAsync(P->h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
     P->have_forward = true;
@@ -1543,15 +1609,14 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
                        ensure(P, P->d_V, sizeof(float) * (size_t)P->RLP * C, "adjoint V")))
             return G3PCF_ERR_ALLOC;
         int* d_status = P->small.as<int>();
-        int* d_queue = d_status + 16;
-        CK(cudaMemsetAsync(P->small.p, 0, 256, st));
-        CK(cudaMemsetAsync(P->counts.p, 0, sizeof(unsigned long long) * P->nbins, st));
+        CK(cudaMemsetAsync(P->small.p, 0, kStatusBytes + sizeof(unsigned long long) * P->nbins, st));
         if ((precise ? launch_adjoint_m_df(dzeta, P->nbins, P->lmax, 1, zsize_of(P->nbins, P->lmax),
                                            P->d_mrealdf.as<float2>(), P->d_mnorm.as<float>(), st)
                      : launch_adjoint_m(dzeta, P->nbins, P->lmax, 1, zsize_of(P->nbins, P->lmax),
                                         P->d_mreal.as<float>(), st)) != 0)
             return fail(G3PCF_ERR_CUDA, "adjoint preparation launch failed: %s", cudaGetErrorString(cudaGetLastError()));
         P->lev_used = 0;
+        P->levq.clear();
         for (int64_t q0 = 0; q0 < rows; q0 += C) {
             PairArgs pa{};
             pa.pts = P->pts.as<float4>();
@@ -1569,8 +1634,8 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
             pa.colmap = P->d_colmap.as<int>();
             pa.colscale = P->d_colscale.as<float>();
             pa.RL = P->RL;
-            pa.counts = P->counts.as<unsigned long long>();
-            pa.queue = d_queue;
+            pa.counts = counts_of(P);
+            pa.queue = d_status + kQueueSlot;
             pa.status = d_status;
             pa.kflush = P->kflush;
             pa.V = P->d_V.as<float>();
@@ -1580,7 +1645,6 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
             pa.bins = P->bins;
             pa.bintab = P->d_bintab.as<unsigned char>();
             pa.bin_tscale = P->bin_tscale;
-            CK(cudaMemsetAsync(d_queue, 0, sizeof(int), st));
             if (int r = run_pair_lists(P, pa, st, 2)) return r;
         }
         CK(cudaMemcpyAsync(P->h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1609,9 +1673,7 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
     if (!blks.empty())
         CK(cudaMemcpyAsync(P->d_vblk.p, blks.data(), sizeof(int4) * blks.size(), cudaMemcpyHostToDevice, st));
     int* d_status = P->small.as<int>();
-    int* d_queue = d_status + 16;
-    CK(cudaMemsetAsync(P->small.p, 0, 256, st));
-    CK(cudaMemsetAsync(P->counts.p, 0, sizeof(unsigned long long) * P->nbins * ncat, st));
+    CK(cudaMemsetAsync(P->small.p, 0, kStatusBytes + sizeof(unsigned long long) * P->nbins * ncat, st));
     const int64_t zs = zsize_of(P->nbins, P->lmax);
     int prep = 0;
     if (precise) {
@@ -1645,8 +1707,8 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
     pa.colmap = P->d_colmap.as<int>();
     pa.colscale = P->d_colscale.as<float>();
     pa.RL = P->RL;
-    pa.counts = P->counts.as<unsigned long long>();
-    pa.queue = d_queue;
+    pa.counts = counts_of(P);
+    pa.queue = d_status + kQueueSlot;
     pa.status = d_status;
     pa.kflush = P->kflush;
     pa.V = P->d_V.as<float>();
@@ -1660,6 +1722,7 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
         pa.q0 = 0;
         pa.chunked = 0;
         P->lev_used = 0;
+        P->levq.clear();
         if (int r = run_pair_lists(P, pa, st, 1)) return r;
     } else if (launch_pair(P->lmax, pa, P->nsm, st, 1) != 0) {
         return fail(G3PCF_ERR_CUDA, "adjoint pair kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1974,23 +2037,23 @@ int g3pcf_stats(g3pcf_plan_t P, double* vals, int nvals) {
         CK(cudaEventElapsedTime(&ms, P->ev[0], P->ev[4]));
         P->stats[4] = ms;
         std::vector<unsigned long long> cnt((size_t)P->nbins * P->last_ncat);
-        CK(cudaMemcpy(cnt.data(), P->counts.p, sizeof(unsigned long long) * cnt.size(), cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(cnt.data(), counts_of(P), sizeof(unsigned long long) * cnt.size(), cudaMemcpyDeviceToHost));
         double tot = 0;
         for (auto v : cnt) tot += (double)v;
         P->stats[5] = tot;
     }
     P->stats[8] = (double)P->launches;
     double scan_ms = 0.0, accum_ms = 0.0;
-    for (int k = 0; k + 3 < P->lev_used; k += 4) {
+    for (size_t k = 0; k + 2 < P->levq.size(); k += 3) {
         float a = 0.f, b = 0.f;
-        CK(cudaEventElapsedTime(&a, P->lev[k], P->lev[k + 1]));
-        CK(cudaEventElapsedTime(&b, P->lev[k + 2], P->lev[k + 3]));
+        CK(cudaEventElapsedTime(&a, P->levq[k], P->levq[k + 1]));
+        CK(cudaEventElapsedTime(&b, P->levq[k + 1], P->levq[k + 2]));
         scan_ms += a;
         accum_ms += b;
     }
     P->stats[11] = scan_ms;
     P->stats[12] = accum_ms;
-    P->stats[13] = (double)(P->lev_used / 4);
+    P->stats[13] = (double)(P->levq.size() / 3);
     P->stats[14] = P->direct_used ? 1.0 : 0.0;
     for (int k = 0; k < nvals && k < 15; ++k) vals[k] = P->stats[k];
     return G3PCF_OK;
@@ -2029,10 +2092,10 @@ int g3pcf_destroy(g3pcf_plan_t P) {
     if (P->device >= 0) cudaStreamSynchronize(P->stream);
     DevBuf* bufs[] = {&P->key_a, &P->key_b, &P->val_a, &P->val_b, &P->idx_scratch,
                       &P->pts, &P->pts64, &P->orig, &P->cstart, &P->plist,
-                      &P->small, &P->counts, &P->A, &P->partials, &P->d_tiles, &P->d_segs,
-                      &P->d_segfirst, &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_colcoef, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
-                      &P->d_tiles_tc, &P->d_cats, &P->d_mreal, &P->d_V, &P->d_bintab, &P->d_vblk,
-                      &P->d_strips_tc, &P->d_items,
+                      &P->small, &P->A, &P->partials, &P->d_tiles, &P->d_tables,
+                      &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_colcoef, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
+                      &P->d_tiles_tc, &P->d_mreal, &P->d_V, &P->d_bintab, &P->d_vblk,
+                      &P->d_strips_tc,
                       &P->d_slotcoefdf, &P->d_mrealdf, &P->d_mnorm, &P->d_Vdf, &P->d_colcoefdf,
                       &P->wrow, &P->l_need, &P->l_base, &P->l_nch, &P->l_pool, &P->l_tag, &P->l_ord,
                       &P->l_gbase, &P->l_scantmp, &P->l_passq};

@@ -170,8 +170,10 @@ __device__ __forceinline__ double c_lookup(const double* part, const Tile* tiles
 
 __global__ void k_reduce(const double* partials, int part_stride, const int* seg_first, int ncat,
                          const Tile* tiles, BlockInfo bi, int nbins, int lmax, int T, int cm,
-                         int64_t zsize, double* zeta) {
+                         int64_t zsize, double* zeta, const unsigned long long* counts, int64_t* counts_out) {
     const int cat = blockIdx.y;
+    if (counts_out && blockIdx.x == 0 && threadIdx.x < nbins && cat < ncat)
+        counts_out[cat * nbins + threadIdx.x] = (int64_t)counts[cat * nbins + threadIdx.x];
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= zsize || cat >= ncat) return;
     int m = 0;
@@ -272,7 +274,7 @@ int launch_contract_fp32(const float* A, int RLP, const float* wrow, const Tile*
 
 int launch_reduce(const double* partials, int part_stride, const int* seg_first, int ncat,
                   int nbins, int lmax, const Tile* tiles, int T, double* zeta, cudaStream_t st,
-                  int colmajor) {
+                  int colmajor, const unsigned long long* counts, int64_t* counts_out) {
     BlockInfo bi;
     int base = 0;
     int64_t zo = 0;
@@ -290,7 +292,7 @@ int launch_reduce(const double* partials, int part_stride, const int* seg_first,
     const int64_t zsize = zo;
     dim3 grid((unsigned)((zsize + 255) / 256), ncat);
     k_reduce<<<grid, 256, 0, st>>>(partials, part_stride, seg_first, ncat, tiles, bi, nbins, lmax,
-                                   T, colmajor, zsize, zeta);
+                                   T, colmajor, zsize, zeta, counts, counts_out);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

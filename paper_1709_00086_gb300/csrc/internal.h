@@ -163,6 +163,7 @@ struct ListArgs {
     const int* cstart;
     const int* plist;
     const unsigned* key;
+    int ncat;
     int qa, qb;              // primaries of this launch (processing order)
     int q0;                  // first primary of the A chunk (row = q - q0 when chunked)
     int chunked;
@@ -176,8 +177,9 @@ struct ListArgs {
     int* queue;
     int* status;
     int* need;               // [q] (global processing-order index)
-    unsigned long long* ncand;  // candidates visited (k_count adds)
-    const int* base;         // [q] first chunk of q, relative to the pool arrays
+    int* base;               // [q] first chunk of q, relative to the pool arrays
+    int* cursor;             // if set: k_scan takes base[q] from this counter, below cap
+    int cap;
     int* nchunks;            // [q]
     const int* qrange;       // if set: qa = qrange[0], qb = qrange[1] (device-planned pass)
     int exact_img;           // k_accum: separations from the head + tail of the primary's images
@@ -291,10 +293,11 @@ int64_t contract_fp32_split(int64_t seg, int64_t nbase, int ntiles, int nsm);
 int launch_contract_fp32(const float* A, int RLP, const float* wrow, const Tile* tiles, int ntiles,
                          const Segment* segs, int nsegs, double* partials, int part_stride,
                          cudaStream_t st);
-// colmajor: partial tiles stored [c][r] (tensor-core path) instead of [r][c]
+// colmajor: partial tiles stored [c][r] (tensor-core path) instead of [r][c];
+// counts (ncat x nbins) are copied to counts_out where that is given
 int launch_reduce(const double* partials, int part_stride, const int* seg_first, int ncat,
                   int nbins, int lmax, const Tile* tiles, int T, double* zeta, cudaStream_t st,
-                  int colmajor = 0);
+                  int colmajor = 0, const unsigned long long* counts = nullptr, int64_t* counts_out = nullptr);
 int pair_nrp(int lmax);
 int launch_isotropic(const double* zeta, int nbins, int lmax, int ncat, double* out, cudaStream_t st);
 // out = sum_c coef[c] zeta_c (coef: host, passed by value; ncat <= kMaxCombine)
@@ -375,10 +378,12 @@ void set_last_error(const char* msg);
 int noalloc_zeta_from_alm(int nbins, int lmax, const float* alm, int64_t ld, const float* w,
                           int64_t np, double* zeta, cudaStream_t st, char* err, size_t errlen);
 
-// Status block of a call (256 bytes, zeroed per call): int [0] status word,
-// [16] work counter, [20] set by the index build when a weight is negative,
-// [24..25] candidate count (64-bit).
-constexpr int kNegWeightSlot = 20;
+// Status block of a call (zeroed per call; int slots): [0] status word, [16..18] work
+// counters, [20] set by the index build when a weight is negative, [19] list chunks
+// handed out, [24..25] candidates, [26..27] list chunks needed (64-bit), [28] most
+// chunks of one primary.  The pair counts follow it.
+constexpr size_t kStatusBytes = 256;
+constexpr int kQueueSlot = 16, kCursorSlot = 19, kNegWeightSlot = 20, kCandSlot = 24, kTotalSlot = 26, kMostSlot = 28;
 
 // status bits written by kernels
 enum : int {

@@ -86,31 +86,70 @@ __device__ __forceinline__ float4 image_head(int code, const float4& P0, const d
     return make_float4((float)(x - sx * boxd), (float)(y - sy * boxd), (float)(z - sz * boxd), 0.f);
 }
 
-__global__ void __launch_bounds__(kLThreads) k_count(ListArgs a) {
+// Catalog of sorted slot p (cell keys stay below 2^31).
+__device__ __forceinline__ long long catalog_of(const ListArgs& a, int p) {
+    return a.ncat == 1 ? 0 : (long long)(a.key[p] / (unsigned)a.g.cells_per_cat);
+}
+
+// lpp (a power of two) lanes per primary, so that a launch has enough threads
+// whatever the number of primaries and of rows: one warp per primary left 23 of 32
+// lanes idle at 9 rows (120,000 primaries: 83 us).
+constexpr int kCountThreads = 256;
+__global__ void __launch_bounds__(kCountThreads) k_count(ListArgs a, int lpp) {
+    __shared__ unsigned long long s_cand, s_total;
+    __shared__ int s_most;
+    if (threadIdx.x == 0) {
+        s_cand = s_total = 0;
+        s_most = 0;
+    }
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
+    const int per = 32 / lpp, sub = lane & (lpp - 1);
     const Grid& g = a.g;
     const int K = g.reach, W = 2 * K + 1, nrows = W * W;
-    for (int q = a.qa + gw; q < a.qb; q += nw) {
-        const int p = a.plist ? a.plist[q] : q;
-        const float4 P0 = a.pts[p];
-        const long long cat = (long long)(a.key[p] / (unsigned long long)g.cells_per_cat);
-        const long long kbase = cat * g.cells_per_cat;
-        const int cy = cell_of(P0.y, g), cz = cell_of(P0.z, g);
+    unsigned long long cand = 0, total = 0;
+    int most = 0;
+    for (int q0 = a.qa + gw * per; q0 < a.qb; q0 += nw * per) {
+        const int q = q0 + lane / lpp;
         long long sum = 0;
-        for (int r = lane; r < nrows; r += 32) {
-            int4 pm, p0, pp;
-            row_pieces(r, W, K, cy, cz, P0, g, a.bins.slack, a.bins.rmax2f, kbase, a.cstart, pm, p0,
-                       pp);
-            sum += max(pm.y - pm.x, 0) + max(p0.y - p0.x, 0) + max(pp.y - pp.x, 0);
+        if (q < a.qb) {
+            const int p = a.plist ? a.plist[q] : q;
+            const float4 P0 = a.pts[p];
+            const long long kbase = catalog_of(a, p) * g.cells_per_cat;
+            const int cy = cell_of(P0.y, g), cz = cell_of(P0.z, g);
+            for (int r = sub; r < nrows; r += lpp) {
+                int4 pm, p0, pp;
+                row_pieces(r, W, K, cy, cz, P0, g, a.bins.slack, a.bins.rmax2f, kbase, a.cstart, pm, p0, pp);
+                sum += max(pm.y - pm.x, 0) + max(p0.y - p0.x, 0) + max(pp.y - pp.x, 0);
+            }
         }
+        for (int o = lpp >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+        if (q < a.qb && sub == 0) {
+            const int need = (int)((sum + kChunk - 1) / kChunk) + a.bins.nbins;
+            a.need[q] = need;
+            cand += sum;
+            total += need;
+            most = max(most, need);
+        }
+    }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
-        if (lane == 0) {
-            a.need[q] = (int)((sum + kChunk - 1) / kChunk) + a.bins.nbins;
-            atomicAdd(a.ncand, (unsigned long long)sum);
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+        cand += __shfl_xor_sync(kFull, cand, o);
+        total += __shfl_xor_sync(kFull, total, o);
+    }
+    most = __reduce_max_sync(kFull, most);
+    if (lane == 0 && most > 0) {
+        atomicAdd(&s_cand, cand);
+        atomicAdd(&s_total, total);
+        atomicMax(&s_most, most);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_most > 0) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.status + kCandSlot), s_cand);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.status + kTotalSlot), s_total);
+        atomicMax(a.status + kMostSlot, s_most);
     }
 }
 
@@ -183,12 +222,27 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
         if (lane == 0) q = qa + atomicAdd(a.queue, 1);
         q = __shfl_sync(kFull, q, 0);
         if (q >= qb) break;
-        if (a.base[q] < 0) {  // no room in the planned passes (flagged by the planner)
+        const int cap_ch = a.need[q];  // chunks reserved for the primary
+        int cbase = 0;
+        if (a.cursor) {
+            if (lane == 0) {
+                cbase = atomicAdd(a.cursor, cap_ch);
+                if (cbase < 0 || cbase > a.cap - cap_ch) {  // more than the captured pool holds
+                    cbase = -1;
+                    atomicOr(a.status, kStatusOverflow);
+                }
+                a.base[q] = cbase;
+            }
+            cbase = __shfl_sync(kFull, cbase, 0);
+        } else {
+            cbase = a.base[q];
+        }
+        if (cbase < 0) {  // no room in the planned passes (flagged by the planner)
             if (lane == 0) a.nchunks[q] = 0;
             continue;
         }
         const int p = a.plist ? a.plist[q] : q;
-        const long long cat = (long long)(a.key[p] / (unsigned long long)g.cells_per_cat);
+        const long long cat = catalog_of(a, p);
         if (cat != cur_cat) {
             if (cur_cat >= 0 && lane < B && my_total) atomicAdd(&a.counts[cur_cat * B + lane], my_total);
             my_total = 0;
@@ -214,11 +268,10 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
         }
         const int cy = cell_of(P0.y, g), cz = cell_of(P0.z, g);
         // this primary's chunks: list entries, or (DIR) one direction per pair
-        int* const pool = a.chunks + (int64_t)a.base[q] * kChunk;
-        float4* const dpool = a.dirs + (int64_t)a.base[q] * kChunk;
-        int* const ptag = a.tag + a.base[q];
-        int* const pord = a.ord + a.base[q];
-        const int cap_ch = a.need[q];  // chunks reserved for it
+        int* const pool = a.chunks + (int64_t)cbase * kChunk;
+        float4* const dpool = a.dirs + (int64_t)cbase * kChunk;
+        int* const ptag = a.tag + cbase;
+        int* const pord = a.ord + cbase;
         int nch = 0;                   // chunks opened so far (warp-uniform)
         // per bin: the last written slot of the open chunk (chunk * 32 + position;
         // -1, like any full chunk, has position 31) and the chunks opened so far
@@ -1108,10 +1161,13 @@ int launch_scan_k(const ListArgs& a, int nsm, cudaStream_t st) {
 
 int launch_count(const ListArgs& a, int nsm, cudaStream_t st) {
     if (a.qb <= a.qa) return 0;
-    const int warps = a.qb - a.qa;
-    int blocks = (warps + kLWarps - 1) / kLWarps;
-    if (blocks > nsm * 16) blocks = nsm * 16;
-    k_count<<<blocks, kLThreads, 0, st>>>(a);
+    // lanes per primary: at least about 1,000 threads per SM
+    const int rows = (2 * a.g.reach + 1) * (2 * a.g.reach + 1);
+    int lpp = 1;
+    while (lpp < 32 && lpp < rows && (int64_t)(a.qb - a.qa) * lpp < (int64_t)nsm * 1024) lpp *= 2;
+    int64_t blocks = ((int64_t)(a.qb - a.qa) * lpp + kCountThreads - 1) / kCountThreads;
+    if (blocks > nsm * 4) blocks = nsm * 4;  // (three atomics per block)
+    k_count<<<(unsigned)blocks, kCountThreads, 0, st>>>(a, lpp);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
