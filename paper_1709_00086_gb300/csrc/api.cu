@@ -1151,10 +1151,11 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
                         for (int k = 0; k < nstrips; ++k) {
                             const int step = stp[k];
                             for (int v = s0; v < s1; v += step)
-                                items.push_back(TcItem{k, v, std::min(step, s1 - v), 0});
+                                items.push_back(TcItem{k, v, std::min(step, s1 - v), -1});
                         }
                         s0 = s1;
                     }
+                    schedule_tc_items(items, P->strips_tc.data(), segs.data(), P->nsm);
                 }
                 Tables& t = ctab[ch];
                 t.segs = 0;

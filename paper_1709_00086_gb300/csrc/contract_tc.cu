@@ -42,6 +42,8 @@
 // word, every warp stops at its next wait, the TMA thread lets its own copies
 // land, the TMEM is freed and the kernel returns.
 #include <algorithm>
+#include <functional>
+#include <queue>
 #include <vector>
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -226,6 +228,17 @@ __device__ __forceinline__ bool mbar_wait_or_abort(unsigned bar, unsigned parity
     return false;
 }
 
+// The k-blocks of a part of a work item: its accumulation runs (kSubKB k-blocks each,
+// counted from the item's first) are dealt to the nvseg parts in order, so that the
+// runs, and with them the FP32 sums, are the same as those of the whole item.
+__device__ __forceinline__ void part_blocks(const TcItem& it, int& kb0, int& nkb) {
+    if (it.part < 0) return;
+    const int nr = (nkb + kSubKB - 1) / kSubKB;
+    const int k0 = it.part * nr / it.nvseg * kSubKB, k1 = min(nkb, (it.part + 1) * nr / it.nvseg * kSubKB);
+    kb0 += k0;
+    nkb = k1 > k0 ? k1 - k0 : 0;
+}
+
 // Drain warps of a work item: TMEM lane (= output row) 32 (warp % 4) + lane;
 // column c of the accumulator is column c % 128 of the strip's tile c / 128;
 // warp w takes the 32-column groups g with g % 2 == w / 4.  Each finished run
@@ -238,7 +251,8 @@ __device__ __forceinline__ void drain_item(int warp, int lane, unsigned tmem, in
     const int quarter = warp & 3, half = warp >> 2;
     const int row = quarter * 32 + lane;
     const unsigned long long keep = l2_keep_policy();
-    double* outs = partials + (int64_t)it.vseg0 * part_stride;
+    const int slot = it.vseg0 + (it.part > 0 ? it.part : 0);
+    double* outs = partials + (int64_t)slot * part_stride;
     for (int sub = 0; sub < nsub; ++sub) {
         const int buf = sub & 1;
         const bool ok = mbar_wait(ready0 + 8 * buf, (sub >> 1) & 1);
@@ -283,12 +297,13 @@ __device__ __forceinline__ void drain_item(int warp, int lane, unsigned tmem, in
         __syncwarp();
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(drained0 + 8 * buf) : "memory");
     }
-    // an empty range writes zeros; the item's later virtual segments are zeroed
+    // an empty range writes zeros; a whole item's later virtual segments are zeroed
     // (their primaries are in the first slot's sum)
+    const int nslot = it.part < 0 ? it.nvseg : 1;
     for (int p = 0; p < nt; ++p) {
         const Tile t = tiles[sp.tile0 + p];
-        for (int v = (nsub == 0 ? 0 : 1); v < it.nvseg; ++v) {
-            double* out = partials + (int64_t)(it.vseg0 + v) * part_stride + t.out_off;
+        for (int v = (nsub == 0 ? 0 : 1); v < nslot; ++v) {
+            double* out = partials + (int64_t)(slot + v) * part_stride + t.out_off;
             for (int c = half; c < kTT; c += 2) out[(int64_t)c * kTT + row] = 0.0;
         }
     }
@@ -315,8 +330,9 @@ __global__ void __launch_bounds__(kTcWarps * 32, 1)
     const TcStrip sp = a.strips[it.strip];
     const Segment sg0 = a.segs[it.vseg0];
     const int row0 = sg0.row0, row1 = a.segs[it.vseg0 + it.nvseg - 1].row1;
-    const int kb0 = row0 / kKB;
-    const int nkb = (row1 - row0 + kKB - 1) / kKB;
+    int kb0 = row0 / kKB;
+    int nkb = (row1 - row0 + kKB - 1) / kKB;
+    part_blocks(it, kb0, nkb);
     const int nsub = (nkb + kSubKB - 1) / kSubKB;
     const int nt = sp.ntile;   // tiles side by side (column panels of 128)
     const int N = sp.n;        // MMA width: the strip's valid columns rounded up to 16
@@ -656,8 +672,9 @@ __global__ void __launch_bounds__(kOpWarps * 32, 1)
     const TcItem it = a.items[blockIdx.x];
     const TcStrip sp = a.strips[it.strip];
     const int row0 = a.segs[it.vseg0].row0, row1 = a.segs[it.vseg0 + it.nvseg - 1].row1;
-    const int kb0 = row0 / kKB;
-    const int nkb = (row1 - row0 + kKB - 1) / kKB;
+    int kb0 = row0 / kKB;
+    int nkb = (row1 - row0 + kKB - 1) / kKB;
+    part_blocks(it, kb0, nkb);
     const int nsub = (nkb + kSubKB - 1) / kSubKB;
     const int nt = sp.ntile, N = sp.n, Np = kTT * nt;
     const int rowsL = a.tiles[sp.tile0].rows;
@@ -904,6 +921,59 @@ int plan_tc_items(const TcStrip* strips, int nstrips, int vmax, double slots, in
     if (V > vmax) V = vmax;
     if (V < 2) V = 2;
     return V;
+}
+
+// The items that share one list: whole, or every two-segment item as two parts, whichever
+// finishes first when the SMs take them in order of size (one CTA per SM; a CTA costs
+// about 8 k-blocks besides its own, a two-panel k-block 1.8 of a one-panel one).
+// Parts pay where whole items leave SMs idle: one catalog of 17,389 primaries
+// (B = 7, lmax = 5) 84 -> 51 us, of 20,000 (B = lmax = 10) 107 -> 98 us; one that fills
+// the chip keeps its whole items.
+// (Integer costs: a comparison of FP expressions may round differently at its two
+// uses inside a sort.)
+static int64_t makespan(std::vector<int64_t> cost, int nsm) {
+    std::sort(cost.begin(), cost.end(), std::greater<int64_t>());
+    std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> sm;
+    for (int k = 0; k < nsm; ++k) sm.push(0);
+    int64_t end = 0;
+    for (int64_t c : cost) {
+        const int64_t t = sm.top() + c;
+        sm.pop();
+        sm.push(t);
+        end = std::max(end, t);
+    }
+    return end;
+}
+
+void schedule_tc_items(std::vector<TcItem>& items, const TcStrip* strips, const Segment* segs, int nsm) {
+    auto blocks = [&](const TcItem& it) {
+        int n = (segs[it.vseg0 + it.nvseg - 1].row1 - segs[it.vseg0].row0 + kKB - 1) / kKB;
+        if (it.part >= 0) {
+            const int nr = (n + kSubKB - 1) / kSubKB;
+            const int k0 = it.part * nr / it.nvseg * kSubKB, k1 = std::min(n, (it.part + 1) * nr / it.nvseg * kSubKB);
+            n = std::max(0, k1 - k0);
+        }
+        return n;
+    };
+    auto cost = [&](const TcItem& it) -> int64_t { return 80 + (int64_t)blocks(it) * (strips[it.strip].ntile == 2 ? 18 : 10); };
+    std::vector<TcItem> parts;
+    bool any = false;
+    for (const TcItem& it : items) {
+        if (it.nvseg == 2 && blocks(it) > kSubKB) {
+            any = true;
+            for (int p = 0; p < 2; ++p) parts.push_back(TcItem{it.strip, it.vseg0, 2, p});
+        } else {
+            parts.push_back(it);
+        }
+    }
+    auto costs = [&](const std::vector<TcItem>& v) {
+        std::vector<int64_t> c;
+        for (const TcItem& it : v) c.push_back(cost(it));
+        return c;
+    };
+    if (any && items.size() <= 4096 && makespan(costs(parts), nsm) < makespan(costs(items), nsm)) items.swap(parts);
+    // largest first
+    std::stable_sort(items.begin(), items.end(), [&](const TcItem& a, const TcItem& b) { return cost(a) > cost(b); });
 }
 
 int launch_contract_tc(const float* A, int RLP, int RL, int64_t arows, const float* wrow, const int4* cats,

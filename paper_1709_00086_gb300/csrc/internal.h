@@ -13,6 +13,7 @@
 #pragma once
 
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
@@ -320,13 +321,17 @@ int contract_tc_kblock();
 // multiples of 64).
 struct TcStrip { int tile0; int ntile; int xrow; int xcol; int n; int xb; };
 // A work item of the tensor-core contraction: a strip and nvseg (1 or 2)
-// consecutive virtual segments from vseg0 (partials go to slot vseg0).
-struct TcItem { int strip; int vseg0; int nvseg; int pad; };
+// consecutive virtual segments from vseg0 (partials go to slot vseg0), or part 0 or 1 of
+// a two-segment item (whole accumulation runs; partials go to slot vseg0 + part).
+struct TcItem { int strip; int vseg0; int nvseg; int part; };
 int make_strips(const Tile* tiles, int ntiles, TcStrip* out, int max_strips);
 // Work split of one catalog for the tensor-core contraction: returns V, the
 // number of equal virtual segments (even, >= 2, <= vmax unless vmax < 2), about
 // slots / (items per segment), and step[s], the segments per work item of strip s.
 int plan_tc_items(const TcStrip* strips, int nstrips, int vmax, double slots, int* step);
+// Splits two-segment items into parts where that ends sooner on nsm SMs and orders the
+// items by size; segs: the virtual segments the items index.
+void schedule_tc_items(std::vector<TcItem>& items, const TcStrip* strips, const Segment* segs, int nsm);
 // arows: rows of A in the buffer (the tensor map's extent; rows beyond read as 0)
 int launch_contract_tc(const float* A, int RLP, int RL, int64_t arows, const float* wrow, const int4* cats,
                        const Tile* tiles, const TcStrip* strips, const TcItem* items, int nitems,
