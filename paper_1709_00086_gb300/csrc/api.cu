@@ -466,9 +466,11 @@ void compute_columns(g3pcf_plan_t P) {
             double kl = std::exp(lnN + lnLead);
             if (m & 1) kl = -kl;
             coef_off[l * (L + 1) + m] = (int)P->colcoef.size();
-            for (double ck : cheb_coeffs(m, l - m)) {
-                P->colcoef.push_back((float)(ck * kl));
-                P->colcoef64.push_back(ck * kl);
+            // (k of the parity of l - m only: the other coefficients are exact zeros)
+            const std::vector<double> cc = cheb_coeffs(m, l - m);
+            for (int k = (l - m) & 1; k <= l - m; k += 2) {
+                P->colcoef.push_back((float)(cc[k] * kl));
+                P->colcoef64.push_back(cc[k] * kl);
             }
         }
     int col = 0;
@@ -486,13 +488,15 @@ void compute_columns(g3pcf_plan_t P) {
                 if (m & 1) kl = -kl;
                 P->colmap[col] = b * P->nrp + slot;
                 P->colscale[col] = (float)kl;
-                const int slot0 = (m == 0) ? 0 : acc_base(L, m) + part;
-                P->colconv[col] = int4{b * P->nrp + slot0, m == 0 ? 1 : 2, l - m + 1, coef_off[l * (L + 1) + m]};
+                const int step = m == 0 ? 1 : 2;
+                const int slot0 = (m == 0 ? 0 : acc_base(L, m) + part) + step * ((l - m) & 1);
+                P->colconv[col] =
+                    int4{b * res_stride(P->nrp) + slot0, 2 * step, (l - m) / 2 + 1, coef_off[l * (L + 1) + m]};
                 ++col;
             }
     }
-    // adjoint: per accumulator slot (m, k, part) the A columns (l = m + n, n = k..L-m,
-    // stride B from bin 0) and coefficients c^(m)_{n,k} K_lm of the transposed connection
+    // adjoint: per accumulator slot (m, k, part) the A columns (l = m + n, n = k, k + 2,
+    // .. <= L-m, stride 2B from bin 0) and coefficients c^(m)_{n,k} K_lm of the transposed connection
     const int NR = (L + 1) * (L + 1);
     P->slotconv.assign(NR, int4{0, 0, 0, 0});
     P->slotcoef.clear();
@@ -503,8 +507,8 @@ void compute_columns(g3pcf_plan_t P) {
         for (int part = 0; part < (m == 0 ? 1 : 2); ++part)
             for (int k = 0; k <= L - m; ++k) {
                 const int slot = (m == 0) ? k : acc_base(L, m) + 2 * k + part;
-                P->slotconv[slot] = int4{colm + part * K + k * B, B, L - m - k + 1, (int)P->slotcoef.size()};
-                for (int nn = k; nn <= L - m; ++nn) {
+                P->slotconv[slot] = int4{colm + part * K + k * B, 2 * B, (L - m - k) / 2 + 1, (int)P->slotcoef.size()};
+                for (int nn = k; nn <= L - m; nn += 2) {
                     const int l = m + nn;
                     const double lnN = 0.5 * (std::log((2.0 * l + 1.0) / (4.0 * M_PI)) + lfact(l - m) - lfact(l + m));
                     const double lnLead = lfact(2 * l) - l * std::log(2.0) - lfact(l) - lfact(l - m);

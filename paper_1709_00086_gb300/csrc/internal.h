@@ -300,6 +300,11 @@ int launch_reduce(const double* partials, int part_stride, const int* seg_first,
                   int nbins, int lmax, const Tile* tiles, int T, double* zeta, cudaStream_t st,
                   int colmajor = 0, const unsigned long long* counts = nullptr, int64_t* counts_out = nullptr);
 int pair_nrp(int lmax);
+// Words from one bin's sums to the next in the accumulate kernels: odd, so that the
+// lanes that write a row of A (neighbours differ by the bin) read different banks.
+// At a multiple of 32 they shared one: 20,000 primaries at B = lmax = 10, 394 us
+// (with every coefficient, the zero ones of the wrong parity included) against 320.
+__host__ __device__ constexpr int res_stride(int nrp) { return nrp + 1; }
 int launch_isotropic(const double* zeta, int nbins, int lmax, int ncat, double* out, cudaStream_t st);
 // out = sum_c coef[c] zeta_c (coef: host, passed by value; ncat <= kMaxCombine)
 constexpr int kMaxCombine = 256;

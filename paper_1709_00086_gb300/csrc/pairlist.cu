@@ -644,12 +644,12 @@ __device__ __forceinline__ void reduce_cheb(float (&acc0)[L + 1], float2 (&accc)
 
 // Per-warp shared memory of k_accum / k_adj: img[27] float4 and its low parts
 // imglo[27] float4 (below), R[16] float, point ring [kPtRing][32] float4, entry
-// ring [kEntRing][32] uint, res[B][NRP] float.
+// ring [kEntRing][32] uint, res[B][res_stride(NRP)] float.
 constexpr int kImgBytes = 2 * 27 * 16;
 constexpr int kEntRing = 8;
 constexpr int kPtRing = 4;
 __host__ __device__ constexpr size_t accum_smem_per_warp(int B, int NRP) {
-    return (size_t)B * NRP * 4 + kImgBytes + 64 + kEntRing * 32 * 4 + kPtRing * 32 * 16;
+    return (((size_t)B * res_stride(NRP) * 4 + 15) & ~(size_t)15) + kImgBytes + 64 + kEntRing * 32 * 4 + kPtRing * 32 * 16;
 }
 
 // Column col of a row of A from the per-bin Chebyshev sums res: the
@@ -712,7 +712,7 @@ __device__ __noinline__ void emit_row(const ListArgs& a, const float* res, int r
 
 template <int L, bool EXACT>
 __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
-    constexpr int NRP = Shape<L>::NRP;
+    constexpr int NRP = Shape<L>::NRP, RS = res_stride(NRP);
     extern __shared__ __align__(16) unsigned char la_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int B = a.bins.nbins;
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
         const int nch = a.nchunks[q];
         const int* chunks = a.chunks + (int64_t)cb * kChunk;
         const int* ordp = a.ord + cb;
-        for (int k = lane; k < B * NRP; k += 32) res[k] = 0.f;
+        for (int k = lane; k < B * RS; k += 32) res[k] = 0.f;
         __syncwarp();
         if (nch > 0) {
             // List slot i = chunk (low 26 bits) | bin << 26.  Copies in flight
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
                 const unsigned s7 = slot(i + 7);
                 const int bA = (int)(sA >> 26);
                 if (bA != curb) {  // the bin changes: reduce the partials of the last one
-                    reduce_cheb<L>(acc0, accc, lane, res + curb * NRP);
+                    reduce_cheb<L>(acc0, accc, lane, res + curb * RS);
                     clear();
                     curb = bA;
                 }
@@ -812,7 +812,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
                 s6 = s7;
             }
             cp_async_wait<0>();
-            reduce_cheb<L>(acc0, accc, lane, res + curb * NRP);
+            reduce_cheb<L>(acc0, accc, lane, res + curb * RS);
         }
         __syncwarp();
         const int row = a.chunked ? q - a.q0 : a.orig[p];
@@ -833,11 +833,11 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
 // shuffle (a load per chunk: 25.9 ms).
 constexpr int kDirRing = 8;
 __host__ __device__ constexpr size_t accum_dir_smem_per_warp(int B, int NRP) {
-    return (size_t)B * NRP * 4 + kDirRing * 32 * 16;
+    return (((size_t)B * res_stride(NRP) * 4 + 15) & ~(size_t)15) + kDirRing * 32 * 16;
 }
 template <int L>
 __global__ void __launch_bounds__(kLThreads, 3) k_accum_dir(ListArgs a) {
-    constexpr int NRP = Shape<L>::NRP;
+    constexpr int NRP = Shape<L>::NRP, RS = res_stride(NRP);
     extern __shared__ __align__(16) unsigned char la_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int B = a.bins.nbins;
@@ -857,7 +857,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum_dir(ListArgs a) {
         const int nbc = nch > 0 && lane < B ? a.tag[cb + lane] : 0;  // chunks of bin lane
         const float4* recs = a.dirs + (int64_t)cb * kChunk + lane;
         const int* ordp = a.ord + cb;
-        for (int k = lane; k < B * NRP; k += 32) res[k] = 0.f;
+        for (int k = lane; k < B * RS; k += 32) res[k] = 0.f;
         __syncwarp();
         if (nch > 0) {
             // every lane copies and reads its own record: the ring needs no barrier
@@ -894,7 +894,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum_dir(ListArgs a) {
                     cp_async_commit();
                     accum_pair_cheb<L>(acc0, accc, v.x, v.y, v.z, v.w);
                 }
-                reduce_cheb<L>(acc0, accc, lane, res + b * NRP);
+                reduce_cheb<L>(acc0, accc, lane, res + b * RS);
             }
             cp_async_wait<0>();
         }
