@@ -91,7 +91,8 @@ struct g3pcf_plan_s {
     std::vector<int> colmap;
     std::vector<float> colscale;
     std::vector<int4> colconv;     // Chebyshev-form columns (pair-list path)
-    std::vector<float> colcoef;
+    std::vector<int4> rowconv;     // per complex column (FP32 kernels)
+    std::vector<float> rowcoef;    // rows of 8 coefficients
     std::vector<double> colcoef64;  // the same coefficients in FP64 (double-float path)
     std::vector<float2> colcoefdf;  // ... as head + tail FP32 pairs (uploaded)
     std::vector<int4> slotconv;    // the transposed connection (pair-list adjoint)
@@ -118,10 +119,10 @@ struct g3pcf_plan_s {
     DevBuf key_a, key_b, val_a, val_b, idx_scratch, pts, pts64, orig, cstart, plist;
     DevBuf small;       // status block (kStatusBytes), then the pair counts
     DevBuf A, partials, d_tiles, d_colmap, d_colscale, d_catoff;
-    DevBuf d_colconv, d_colcoef, d_slotconv, d_slotcoef, d_monoexp, d_monoconv, d_monoidx, d_monocoef;
+    DevBuf d_colconv, d_rowconv, d_rowcoef, d_slotconv, d_slotcoef, d_monoexp, d_monoconv, d_monoidx, d_monocoef;
     DevBuf d_ranges, d_tiles_tc, d_mreal, d_V, d_bintab, wrow, d_vblk, d_strips_tc;
     DevBuf d_tables;    // segments, catalogs and work items of a contraction, first segments
-    DevBuf d_bop, d_bblk, d_bcat;
+    DevBuf d_bop, d_bcat;
     DevBuf d_slotcoefdf, d_mrealdf, d_Vdf, d_colcoefdf, d_mnorm;
     int64_t opt_chunk = 0;   // G3PCF_OPT_CHUNK_ROWS
     // pinned staging for host -> device tables (capturable copies); offset
@@ -253,11 +254,6 @@ int upload_consts(g3pcf_plan_t P) {
         return fail(G3PCF_ERR_ALLOC, "workspace allocation failed (constants)");
     CK(cudaMemcpy(P->d_tiles_tc.p, P->tiles_tc.data(), P->tiles_tc.size() * sizeof(Tile),
                   cudaMemcpyHostToDevice));
-    if (!P->bblk.empty()) {
-        if (P->d_bblk.ensure(P->bblk.size() * sizeof(int4)))
-            return fail(G3PCF_ERR_ALLOC, "workspace allocation failed (constants)");
-        CK(cudaMemcpy(P->d_bblk.p, P->bblk.data(), P->bblk.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    }
     if (P->d_strips_tc.ensure(P->strips_tc.size() * sizeof(TcStrip)))
         return fail(G3PCF_ERR_ALLOC, "workspace allocation failed (constants)");
     CK(cudaMemcpy(P->d_strips_tc.p, P->strips_tc.data(), P->strips_tc.size() * sizeof(TcStrip),
@@ -268,10 +264,12 @@ int upload_consts(g3pcf_plan_t P) {
     CK(cudaMemcpy(P->d_colmap.p, P->colmap.data(), P->RL * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(P->d_colscale.p, P->colscale.data(), P->RL * sizeof(float), cudaMemcpyHostToDevice));
     if (P->d_colconv.ensure(P->colconv.size() * sizeof(int4)) ||
-        P->d_colcoef.ensure(P->colcoef.size() * sizeof(float)))
+        P->d_rowconv.ensure(P->rowconv.size() * sizeof(int4)) ||
+        P->d_rowcoef.ensure(P->rowcoef.size() * sizeof(float)))
         return fail(G3PCF_ERR_ALLOC, "workspace allocation failed (constants)");
     CK(cudaMemcpy(P->d_colconv.p, P->colconv.data(), P->colconv.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(P->d_colcoef.p, P->colcoef.data(), P->colcoef.size() * sizeof(float), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(P->d_rowconv.p, P->rowconv.data(), P->rowconv.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(P->d_rowcoef.p, P->rowcoef.data(), P->rowcoef.size() * sizeof(float), cudaMemcpyHostToDevice));
     if (P->d_slotconv.ensure(P->slotconv.size() * sizeof(int4)) ||
         P->d_slotcoef.ensure(P->slotcoef.size() * sizeof(float)))
         return fail(G3PCF_ERR_ALLOC, "workspace allocation failed (constants)");
@@ -455,8 +453,9 @@ void compute_columns(g3pcf_plan_t P) {
     P->colmap.assign(P->RL, 0);
     P->colscale.assign(P->RL, 0.f);
     P->colconv.assign(P->RL, int4{0, 0, 0, 0});
-    P->colcoef.clear();
     P->colcoef64.clear();
+    P->rowcoef.assign(8 * (L + 1) * (L + 1), 0.f);
+    P->rowconv.clear();
     // coefficient rows (times K_lm) per (l, m), shared by the bins and parts
     std::vector<int> coef_off((L + 1) * (L + 1), 0);
     for (int m = 0; m <= L; ++m)
@@ -465,11 +464,11 @@ void compute_columns(g3pcf_plan_t P) {
             const double lnLead = lfact(2 * l) - l * std::log(2.0) - lfact(l) - lfact(l - m);
             double kl = std::exp(lnN + lnLead);
             if (m & 1) kl = -kl;
-            coef_off[l * (L + 1) + m] = (int)P->colcoef.size();
+            coef_off[l * (L + 1) + m] = (int)P->colcoef64.size();
             // (k of the parity of l - m only: the other coefficients are exact zeros)
             const std::vector<double> cc = cheb_coeffs(m, l - m);
             for (int k = (l - m) & 1; k <= l - m; k += 2) {
-                P->colcoef.push_back((float)(cc[k] * kl));
+                P->rowcoef[8 * (l * (L + 1) + m) + k / 2] = (float)(cc[k] * kl);
                 P->colcoef64.push_back(cc[k] * kl);
             }
         }
@@ -490,8 +489,15 @@ void compute_columns(g3pcf_plan_t P) {
                 P->colscale[col] = (float)kl;
                 const int step = m == 0 ? 1 : 2;
                 const int slot0 = (m == 0 ? 0 : acc_base(L, m) + part) + step * ((l - m) & 1);
-                P->colconv[col] =
-                    int4{b * res_stride(P->nrp) + slot0, 2 * step, (l - m) / 2 + 1, coef_off[l * (L + 1) + m]};
+                const int n = (l - m) / 2 + 1, odd = (l - m) & 1;
+                P->colconv[col] = int4{b * P->nrp + slot0, 2 * step, n, coef_off[l * (L + 1) + m]};
+                // sums of the FP32 kernels: (Re, Im) per (m, k), then T_k of m = 0 two by two
+                const int pair0 = m == 0 ? L * (L + 1) / 2 : (m - 1) * (L + 1) - (m - 1) * m / 2 + odd;
+                if (part == 0)
+                    P->rowconv.push_back(int4{(b * res_stride(P->nrp) + 2 * pair0) | n << 16 | step << 24,
+                                              l * (L + 1) + m,
+                                              col | (m == 0 ? -odd : K) * 65536,
+                                              P->bblk[m].z + (col - P->bblk[m].x)});
                 ++col;
             }
     }
@@ -701,7 +707,9 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
     la.RLP = pa.RLP;
     la.colconv = P->d_colconv.as<int4>();
     la.slotconv = P->d_slotconv.as<int4>();
-    la.colcoef = P->d_colcoef.as<float>();
+    la.rowconv = P->d_rowconv.as<int4>();
+    la.rowcoef = P->d_rowcoef.as<float>();
+    la.nrowconv = (int)P->rowconv.size();
     la.RL = pa.RL;
     la.counts = pa.counts;
     la.status = pa.status;
@@ -738,8 +746,6 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
         la.bop = pa.bop;
         la.nbcat = pa.nbcat;
         la.bop_pitch = pa.bop_pitch;
-        la.bblk = pa.bblk;
-        la.nblk = pa.nblk;
         la.bcat = pa.bcat;
     }
     if (P->capturing) {
@@ -1240,8 +1246,6 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
                 pa.bop = bop;
                 pa.nbcat = (int)(ccats.empty() ? 0 : ccats[0].size() / 4);
                 pa.bop_pitch = P->RLPb;
-                pa.bblk = P->d_bblk.as<int4>();
-                pa.nblk = (int)P->bblk.size();
                 pa.bcat = P->d_bcat.as<int4>();
                 const bool use_list = P->opt_pair != 1;
                 if (use_list) {
@@ -1449,7 +1453,6 @@ int g3pcf_plan(g3pcf_plan_t* out, int nbins, double rmin, double rmax, int lmax,
     P->rmax = rmax;
     P->box = box;
     compute_bins(P);
-    compute_columns(P);
     // pairs per lane per bucket flush: the largest k <= 16 for which two
     // 4-warp CTAs of the pair kernel fit in 227 KB of shared memory
     // (dynamic per warp x 4 warps + ~2.6 KB static + 1 KB reserved, per CTA)
@@ -1484,6 +1487,7 @@ int g3pcf_plan(g3pcf_plan_t* out, int nbins, double rmin, double rmax, int lmax,
         delete P;
         return fail(G3PCF_ERR_ARG, "operand blocks out of range");
     }
+    compute_columns(P);
     *out = P;
     return G3PCF_OK;
 }
@@ -2098,7 +2102,7 @@ int g3pcf_destroy(g3pcf_plan_t P) {
     DevBuf* bufs[] = {&P->key_a, &P->key_b, &P->val_a, &P->val_b, &P->idx_scratch,
                       &P->pts, &P->pts64, &P->orig, &P->cstart, &P->plist,
                       &P->small, &P->A, &P->partials, &P->d_tiles, &P->d_tables,
-                      &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_colcoef, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
+                      &P->d_colmap, &P->d_colscale, &P->d_colconv, &P->d_rowconv, &P->d_rowcoef, &P->d_slotconv, &P->d_slotcoef, &P->d_monoexp, &P->d_monoconv, &P->d_monoidx, &P->d_monocoef, &P->d_catoff, &P->d_ranges,
                       &P->d_tiles_tc, &P->d_mreal, &P->d_V, &P->d_bintab, &P->d_vblk,
                       &P->d_strips_tc,
                       &P->d_slotcoefdf, &P->d_mrealdf, &P->d_mnorm, &P->d_Vdf, &P->d_colcoefdf,

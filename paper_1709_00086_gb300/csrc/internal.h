@@ -141,8 +141,6 @@ struct PairArgs {
     __nv_bfloat16* bop;
     int nbcat;
     int bop_pitch;
-    const int4* bblk;
-    int nblk;
     const int4* bcat;
 };
 // mode 0: forward multipoles; mode 1: adjoint pair pass
@@ -171,8 +169,14 @@ struct ListArgs {
     float* wrow;
     float* A;
     int RLP;
-    const int4* colconv;     // RL entries: {first res slot, slot stride, terms, coefficient offset}
-    const float* colcoef;    // Chebyshev -> Legendre-form coefficients (times K_lm)
+    const int4* colconv;     // RL entries (double-float): {first slot, slot stride, terms, coefficient offset}
+    // the same per complex column (one entry for Re and Im), for the FP32 kernels'
+    // sums: {first sum | terms << 16 | pairs per term << 24, coefficient row, A column |
+    // columns from Re to Im << 16 (m = 0: 0, or -1 where the pairs' second half counts),
+    // operand column}; rows of 8 Chebyshev -> Legendre-form coefficients (times K_lm)
+    const int4* rowconv;
+    const float* rowcoef;
+    int nrowconv;
     int RL;
     unsigned long long* counts;
     int* queue;
@@ -198,22 +202,20 @@ struct ListArgs {
     double* dw;
     double* dpos;
     // double-float path (multipoles meant for differentiation): FP64 connection
-    // tables (same layout as colcoef / slotcoef) and the FP64 V rows
+    // tables (colconv's and slotconv's offsets) and the FP64 V rows
     int precise;
-    const float2* colcoefdf;     // colcoef as head + tail FP32 pairs (double-float path)
+    const float2* colcoefdf;     // Chebyshev -> Legendre-form coefficients (times K_lm), head + tail
     const float2* slotcoefdf;    // slotcoef likewise
     const float2* Vdf;           // V rows as head + tail pairs (double-float adjoint)
     // tensor-core operands written by k_accum (forward, no negative weight):
     // sqrt(w) A split into bf16 hi and lo: row r holds hi at bop + 2 r bop_pitch and
     // lo bop_pitch later (one contiguous stretch per row), m blocks from multiples
-    // of 64 (bblk[m] = {first A column, width, first operand column, 0}), rows in
+    // of 64 (operand columns in rowconv), rows in
     // padded coordinates (bcat per catalog: {first padded row, first A row, rows,
     // 0}; nbcat catalogs); skip_a: the FP32 rows of A are not written
     __nv_bfloat16* bop;
     int nbcat;
     int bop_pitch;
-    const int4* bblk;
-    int nblk;
     const int4* bcat;
     int skip_a;
     int* chunks;             // pool: 32 ints per chunk (list entries)
@@ -300,11 +302,12 @@ int launch_reduce(const double* partials, int part_stride, const int* seg_first,
                   int nbins, int lmax, const Tile* tiles, int T, double* zeta, cudaStream_t st,
                   int colmajor = 0, const unsigned long long* counts = nullptr, int64_t* counts_out = nullptr);
 int pair_nrp(int lmax);
-// Words from one bin's sums to the next in the accumulate kernels: odd, so that the
-// lanes that write a row of A (neighbours differ by the bin) read different banks.
-// At a multiple of 32 they shared one: 20,000 primaries at B = lmax = 10, 394 us
-// (with every coefficient, the zero ones of the wrong parity included) against 320.
-__host__ __device__ constexpr int res_stride(int nrp) { return nrp + 1; }
+// Words from one bin's sums to the next in the accumulate kernels: an odd number of
+// word pairs, so that the lanes that write a row of A (neighbours differ by the bin)
+// read different banks.  At a multiple of 32 they shared one: 20,000 primaries at
+// B = lmax = 10, 394 us (with every coefficient, the zero ones of the wrong parity
+// included) against 320.
+__host__ __device__ constexpr int res_stride(int nrp) { return nrp + 2; }
 int launch_isotropic(const double* zeta, int nbins, int lmax, int ncat, double* out, cudaStream_t st);
 // out = sum_c coef[c] zeta_c (coef: host, passed by value; ncat <= kMaxCombine)
 constexpr int kMaxCombine = 256;

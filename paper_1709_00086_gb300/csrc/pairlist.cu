@@ -632,12 +632,15 @@ template <int L>
 __device__ __forceinline__ void reduce_cheb(float (&acc0)[L + 1], float2 (&accc)[Cheb<L>::NC > 0 ? Cheb<L>::NC : 1],
                                             int lane, float* res_b) {
     constexpr int NR = Shape<L>::NR;
-    float acc[NR];
-    static_for<0, L + 1>([&](auto kc) { acc[decltype(kc)::value] = acc0[decltype(kc)::value]; });
+    float acc[NR];  // the (Re, Im) pairs first, then m = 0 (see emit_row)
     static_for<0, Cheb<L>::NC>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
-        acc[L + 1 + 2 * i] = accc[i].x;
-        acc[L + 2 + 2 * i] = accc[i].y;
+        acc[2 * i] = accc[i].x;
+        acc[2 * i + 1] = accc[i].y;
+    });
+    static_for<0, L + 1>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        acc[2 * Cheb<L>::NC + k] = acc0[k];
     });
     butterfly_add<L>(acc, lane, res_b);
 }
@@ -652,60 +655,70 @@ __host__ __device__ constexpr size_t accum_smem_per_warp(int B, int NRP) {
     return (((size_t)B * res_stride(NRP) * 4 + 15) & ~(size_t)15) + kImgBytes + 64 + kEntRing * 32 * 4 + kPtRing * 32 * 16;
 }
 
-// Column col of a row of A from the per-bin Chebyshev sums res: the
-// Legendre-form connection times K_lm.
-__device__ __forceinline__ float connect(const ListArgs& a, const float* res, int col) {
-    const int4 cv = __ldg(a.colconv + col);
-    const float* cf = a.colcoef + cv.w;
-    float v = 0.f;
-    for (int k = 0; k < cv.z; ++k) v = fmaf(__ldg(cf + k), res[cv.x + cv.y * k], v);
-    return v;
-}
-
-// The row of A of one primary, and, when asked for, the tensor-core operands:
-// sqrt(w) times the row split into bf16 hi and lo (the operations of the
-// contraction's converter warps) at the row's padded position inside its
-// catalog, m block by m block.  Out of line, so that the register allocation of
-// the pair loop does not see it.
+// The row of A of one primary from the per-bin Chebyshev sums res (Legendre-form
+// connection times K_lm), and, when asked for, the tensor-core operands: sqrt(w)
+// times the row split into bf16 hi and lo (the operations of the contraction's
+// converter warps) at the row's padded position inside its catalog.  One table
+// entry per complex column: Re and Im share the coefficients, their sums are one
+// 8-byte load.  Two entries per lane, chains unrolled: the warp runs this tail with
+// fewer FMA warps beside it, so its latency counts.  20,000 primaries at B = lmax =
+// 10: the kernel takes 298 us, 320 with a chain per real column.  Out of line, so
+// that the register allocation of the pair loop does not see it.
+template <int L>
 __device__ __noinline__ void emit_row(const ListArgs& a, const float* res, int row, int p, float w, int lane) {
+    constexpr int NT = L / 2 + 1, U = 2;
     float* Arow = a.A + (int64_t)row * a.RLP;
-    if (!a.bop) {
-        // two columns per lane, their coefficient chains interleaved: the warp runs
-        // this tail with fewer FMA warps beside it, so its latency is what counts
-        // (337 ms per forward against 341 ms one column at a time; four: 340 ms)
-        for (int c0 = lane; c0 < a.RL; c0 += 64) {
-            const int c1 = c0 + 32;
-            const int4 cv0 = __ldg(a.colconv + c0);
-            const int4 cv1 = c1 < a.RL ? __ldg(a.colconv + c1) : make_int4(0, 0, 0, 0);
-            const float* cf0 = a.colcoef + cv0.w;
-            const float* cf1 = a.colcoef + cv1.w;
-            float v0 = 0.f, v1 = 0.f;
-            const int n = cv0.z > cv1.z ? cv0.z : cv1.z;
-            for (int k = 0; k < n; ++k) {
-                if (k < cv0.z) v0 = fmaf(__ldg(cf0 + k), res[cv0.x + cv0.y * k], v0);
-                if (k < cv1.z) v1 = fmaf(__ldg(cf1 + k), res[cv1.x + cv1.y * k], v1);
-            }
-            Arow[c0] = v0;
-            if (c1 < a.RL) Arow[c1] = v1;
-        }
-        return;
+    __nv_bfloat16 *Bh = nullptr, *Bl = nullptr;
+    if (a.bop) {
+        const int4 bc = __ldg(a.bcat + (a.nbcat == 1 ? 0 : (int)(a.key[p] / (unsigned long long)a.g.cells_per_cat)));
+        Bh = a.bop + ((int64_t)bc.x + (row - bc.y)) * 2 * a.bop_pitch;
+        Bl = Bh + a.bop_pitch;
     }
-    const int4 bc = __ldg(a.bcat + (a.nbcat == 1 ? 0 : (int)(a.key[p] / (unsigned long long)a.g.cells_per_cat)));
-    __nv_bfloat16* Bh = a.bop + ((int64_t)bc.x + (row - bc.y)) * 2 * a.bop_pitch;
-    __nv_bfloat16* Bl = Bh + a.bop_pitch;
+    const bool fp32 = !a.bop || !a.skip_a;
     const float sw = sqrtf(w);
-    // one column per lane, as the FP32 rows (consecutive lanes read the bins of
-    // one (l, m) in turn from res), the operand columns of an m block contiguous
-    for (int m = 0; m < a.nblk; ++m) {
-        const int4 bb = __ldg(a.bblk + m);  // {first A column, width, first operand column, 0}
-        for (int j = lane; j < bb.y; j += 32) {
-            const int col = bb.x + j;
-            const float v = connect(a, res, col);
-            if (!a.skip_a) Arow[col] = v;
+    auto put = [&](int col, int opcol, float v) {
+        if (fp32) Arow[col] = v;
+        if (Bh) {
             const float y = __fmul_rn(v, sw);
             const __nv_bfloat16 h = __float2bfloat16_rn(y);
-            Bh[bb.z + j] = h;
-            Bl[bb.z + j] = __float2bfloat16_rn(__fsub_rn(y, __bfloat162float(h)));
+            Bh[opcol] = h;
+            Bl[opcol] = __float2bfloat16_rn(__fsub_rn(y, __bfloat162float(h)));
+        }
+    };
+    const int ne = a.nrowconv;
+    for (int e0 = lane; e0 < ne; e0 += 32 * U) {
+        int4 t[U];
+        float2 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            t[u] = e0 + 32 * u < ne ? __ldg(a.rowconv + e0 + 32 * u) : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float4* cf = reinterpret_cast<const float4*>(a.rowcoef + 8 * t[u].y);
+            const float4 c0 = __ldg(cf);
+            float4 c1 = c0;
+            if constexpr (NT > 4) c1 = __ldg(cf + 1);
+            const float2* r = reinterpret_cast<const float2*>(res + (t[u].x & 0xffff));
+            const int n = (t[u].x >> 16) & 0xff, step = t[u].x >> 24;
+            v[u] = make_float2(0.f, 0.f);
+            static_for<0, NT>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                const float4& c4 = k < 4 ? c0 : c1;
+                const float c = (k & 3) == 0 ? c4.x : (k & 3) == 1 ? c4.y : (k & 3) == 2 ? c4.z : c4.w;
+                if (k < n) v[u] = __ffma2_rn(make_float2(c, c), r[k * step], v[u]);
+            });
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int K = t[u].z >> 16, col = t[u].z & 0xffff, oc = t[u].w;
+            if (e0 + 32 * u < ne) {
+                if (K > 0) {  // m >= 1: Re, and Im K columns behind it
+                    put(col, oc, v[u].x);
+                    put(col + K, oc + K, v[u].y);
+                } else {  // m = 0: the sums of an even and an odd T_k share a word pair
+                    put(col, oc, K < 0 ? v[u].y : v[u].x);
+                }
+            }
         }
     }
 }
@@ -816,7 +829,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
         }
         __syncwarp();
         const int row = a.chunked ? q - a.q0 : a.orig[p];
-        emit_row(a, res, row, p, P0.w, lane);
+        emit_row<L>(a, res, row, p, P0.w, lane);
         if (lane == 0) a.wrow[row] = P0.w;
         __syncwarp();
     }
@@ -900,7 +913,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum_dir(ListArgs a) {
         }
         __syncwarp();
         const int row = a.chunked ? q - a.q0 : a.orig[p];
-        emit_row(a, res, row, p, w0, lane);
+        emit_row<L>(a, res, row, p, w0, lane);
         if (lane == 0) a.wrow[row] = w0;
         __syncwarp();
     }

@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 8 ? 4 : 3) k_accum_df(ListArgs
                     const int col = __ldg(&a.slotconv[sl].x) + b;
                     const int4 cv = __ldg(a.colconv + col);
                     const float2* cf = a.colcoefdf + cv.w;
-                    const float2* rs = res + (cv.x - b * res_stride(NRP));
+                    const float2* rs = res + (cv.x - b * NRP);
                     df v2 = {0.f, 0.f};
                     for (int k = 0; k < cv.z; ++k) {
                         const float2 c = __ldg(cf + k), r = rs[cv.y * k];
