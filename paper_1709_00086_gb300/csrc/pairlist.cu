@@ -41,8 +41,9 @@ namespace {
 constexpr int kLWarps = 4;
 constexpr int kLThreads = kLWarps * 32;
 constexpr int kChunk = 32;      // pairs per list chunk
-constexpr int kTrip = 4;        // candidate sub-iterations per trip in k_scan
-constexpr int kStage = (kTrip + 1) * kChunk;  // compaction stage of k_scan (pairs)
+// Candidate sub-iterations per trip in k_scan, staged or not, and its stage (pairs)
+constexpr int kTripStaged = 4, kTripDirect = 3;
+constexpr int kStage = (kTripStaged + 1) * kChunk;
 constexpr int kScanWarps = 8;  // warps per CTA of k_scan, kScanCtas CTAs per SM
 constexpr int kScanThreads = kScanWarps * 32;
 constexpr int kScanCtas = 4;
@@ -50,15 +51,16 @@ constexpr unsigned kNoPair = 0xffffffffu;  // padding entry of a list chunk (ima
 
 // Per-warp shared memory of k_scan: img[27] float4, pd[4] double, pcs[kMaxPieces]
 // int2 (the slot ranges of a row batch: first | image code << 27, end), the compaction
-// stage (kStage accepted pairs: separation and weight, or list entry, and bin),
+// stage if staged (kStage accepted pairs: separation and weight, or list entry, and bin),
 // per bin the last written list slot and the chunk count, R[9] float.
-template <bool DIR>
+template <bool DIR, bool STAGED>
 struct ScanSmem {
+    static constexpr int N = STAGED ? kStage : 1;
     using Item = typename std::conditional<DIR, float4, int>::type;
     float4 img[27];
     int2 pcs[kMaxPieces];
-    Item stage[kStage];
-    int sbin[kStage];
+    Item stage[N];
+    int sbin[N];
     int bst[32];
     int bnbc[32];
     double pd[4];
@@ -162,10 +164,11 @@ __global__ void __launch_bounds__(kCountThreads) k_count(ListArgs a, int lpp) {
 // bin comes from r = r^2 rsqrt(r^2) by one rounding instead of a table look-up
 // (whose bank conflicts cost 3.5 wavefronts per 32 candidates); the 1e-4 of
 // the candidates near an edge take the exact rule.  32 warps per SM at 64
-// registers: 28 warps are 3% slower, 24 are 9%, two or three loads per trip
-// instead of four 10% and 3%.  200,000 clustered points (L = 696, 4.0e9 pairs):
-// 19.8 ms writing 16 bytes per pair, as long as the form that wrote 4 bytes and
-// left the direction to the accumulate kernel.
+// registers: 40 and 48 are 6% and 24% slower.  Staged, two or three loads per trip
+// instead of four are 10% and 3% slower; direct (no stage), three and two are the same,
+// four spill (3%).  200,000 clustered points (L = 696, 4.0e9 pairs): 16.8 ms writing
+// 16 bytes per pair (staged 19.7, which is what the form took that wrote 4 bytes
+// and left the direction to the accumulate kernel).
 //
 // What k_scan writes per pair: a list entry, or for k_accum_dir its direction (in
 // radial mode rotated to the primary's line of sight).
@@ -191,9 +194,11 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-template <int MODE>
+template <int MODE, bool STAGED>
 __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
     constexpr bool DIR = MODE != kEntries;
+    constexpr int kTrip = STAGED ? kTripStaged : kTripDirect;
+    using Smem = ScanSmem<DIR, STAGED>;
     extern __shared__ __align__(16) unsigned char ls_raw[];
     __shared__ double s_e2[kMaxBins + 1];
     __shared__ float2 s_dec[kMaxBins];
@@ -205,7 +210,7 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
             s_dec[k] = make_float2(a.bins.e2f[k] + a.bins.guard[k], a.bins.e2f[k + 1] - a.bins.guard[k + 1]);
     }
     __syncthreads();
-    ScanSmem<DIR>& S = reinterpret_cast<ScanSmem<DIR>*>(ls_raw)[wid];
+    Smem& S = reinterpret_cast<Smem*>(ls_raw)[wid];
     const unsigned lt = lanemask_lt(), gt = ~lt & ~(1u << lane);
     const Grid& g = a.g;
     const bool exact_inputs = (a.pts64 == nullptr);
@@ -281,11 +286,10 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
 
         // Place one accepted pair per lane (bin 63: none) into the open chunk of
         // its bin, opening a new chunk where a bin's chunk fills (at most one per
-        // bin and call).  Lanes of one bin form a group (match.any: its 72 cycles run
-        // beside the other warps' instructions); the group's highest lane opens
-        // the chunk and leaves the bin's last slot.
-        auto place = [&](typename ScanSmem<DIR>::Item it, int bin, bool v) {
-            const unsigned mine = __match_any_sync(kFull, bin);
+        // bin and call).  Lanes of one bin form a group (mine, from match.any: its 72
+        // cycles run beside the other warps' instructions); the group's highest
+        // lane opens the chunk and leaves the bin's last slot.
+        auto place = [&](typename Smem::Item it, int bin, bool v, unsigned mine) {
             const int rank = __popc(mine & lt);
             const int st = S.bst[bin & 31];
             const int f = (st & 31) + 1 + rank;
@@ -388,6 +392,24 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
                                                  j0 + u * kChunk, S.pd, g.boxd, g.periodic, s_e2);
                             }
                     }
+                    if constexpr (!STAGED) {  // place the candidates' lanes as they are
+                        unsigned mine[kTrip];
+#pragma unroll
+                        for (int u = 0; u < kTrip; ++u) {
+                            if constexpr (MODE == kDirs)
+                                d[u] = make_float4(d[u].z * rinv[u], d[u].x * rinv[u], d[u].y * rinv[u], d[u].w);
+                            if ((unsigned)bn[u] >= (unsigned)B) bn[u] = 63;
+                            mine[u] = __match_any_sync(kFull, bn[u]);
+                        }
+#pragma unroll
+                        for (int u = 0; u < kTrip; ++u) {
+                            if constexpr (DIR)
+                                place(d[u], bn[u], bn[u] != 63, mine[u]);
+                            else
+                                place((unsigned)(j0 + u * kChunk) | (code << kIdxBits), bn[u], bn[u] != 63, mine[u]);
+                        }
+                        continue;
+                    }
 #pragma unroll
                     for (int u = 0; u < kTrip; ++u) {
                         // accepted lanes append in lane order
@@ -407,7 +429,10 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
                     if (scnt >= kChunk) {
                         __syncwarp();
                         int at = lane;
-                        for (; scnt >= kChunk; scnt -= kChunk, at += kChunk) place(S.stage[at], S.sbin[at], true);
+                        for (; scnt >= kChunk; scnt -= kChunk, at += kChunk) {
+                            const int bin = S.sbin[at];
+                            place(S.stage[at], bin, true, __match_any_sync(kFull, bin));
+                        }
                         // the rest (fewer than 32) to the stage's front
                         const auto it = S.stage[at];
                         const int bin = S.sbin[at];
@@ -420,9 +445,10 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
             }
             __syncwarp();
         }
-        if (scnt > 0) {  // the last accepted pairs (fewer than 32)
+        if (STAGED && scnt > 0) {  // the last accepted pairs (fewer than 32)
             __syncwarp();
-            place(S.stage[lane], lane < scnt ? S.sbin[lane] : 63, lane < scnt);
+            const int bin = lane < scnt ? S.sbin[lane] : 63;
+            place(S.stage[lane], bin, lane < scnt, __match_any_sync(kFull, bin));
         }
         // the bin state back in lane b
         int cfill = kChunk, ccur = 0, nbc = 0;
@@ -1154,20 +1180,28 @@ int launch_accum_t(const ListArgs& a, int nsm, cudaStream_t st) {
     return a.exact_img ? launch_accum_e<L, true>(a, nsm, st) : launch_accum_e<L, false>(a, nsm, st);
 }
 
-template <int MODE>
-int launch_scan_k(const ListArgs& a, int nsm, cudaStream_t st) {
-    const size_t smem = sizeof(ScanSmem<MODE != kEntries>) * kScanWarps;
-    if (cudaFuncSetAttribute(k_scan<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return -1;
+template <int MODE, bool STAGED>
+int launch_scan_s(const ListArgs& a, int nsm, cudaStream_t st) {
+    const size_t smem = sizeof(ScanSmem<MODE != kEntries, STAGED>) * kScanWarps;
+    auto* k = k_scan<MODE, STAGED>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scan<MODE>, kScanThreads, smem) != cudaSuccess ||
-        per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kScanThreads, smem) != cudaSuccess || per_sm < 1)
         return -1;
     int blocks = per_sm * nsm;
     const int need = (a.qb - a.qa + kScanWarps - 1) / kScanWarps;
     if (!a.qrange && blocks > need) blocks = need;
-    k_scan<MODE><<<blocks, kScanThreads, smem, st>>>(a);
+    k<<<blocks, kScanThreads, smem, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+// Above 1.5 cells per rmax about half of the candidates or more are pairs, and they
+// are placed from the candidates' lanes; below, the accepted ones are gathered in
+// groups of 32 first.  200,000 clustered points, scan direct / staged: 34.1 / 32.1 ms
+// at 0.86 cells (27% pairs), 21.0 / 22.5 at 1.72 (47%), 16.8 / 19.7 at 3.74 (68%).
+template <int MODE>
+int launch_scan_k(const ListArgs& a, int nsm, cudaStream_t st) {
+    return a.bins.rmaxf * a.g.inv_cell < 1.5f ? launch_scan_s<MODE, true>(a, nsm, st)
+                                              : launch_scan_s<MODE, false>(a, nsm, st);
 }
 
 }  // namespace

@@ -67,3 +67,34 @@ def test_partly_filled_chunks(n):
     np.testing.assert_array_equal(c.cpu().numpy(), co)
     # a_lm: FP32 sums of at most 256 terms, each within 2^-24 per operation of ~40
     assert np.abs(z.cpu().numpy() - zo).max() <= 1e-5 * max(np.abs(zo).max(), 1e-300)
+
+
+@pytest.mark.parametrize("cells", [1, 2, 4])
+@pytest.mark.parametrize("los,f64,nbins,lmax,n", [
+    (0, False, 10, 4, 2000), (1, True, 32, 3, 1999), (2, False, 7, 5, 2017), (1, False, 1, 2, 33), (2, True, 5, 1, 1),
+])
+def test_cell_resolutions(cells, los, f64, nbins, lmax, n):
+    # about 0.9, 1.9 and 3.9 cells per rmax: the scan places accepted pairs in groups of
+    # 32 in the first, from the candidates' lanes in the others
+    cat = _case(los, f64, nbins, lmax, 400.0, 0.0, 61.0, n=n, near=n > 240)
+    pos, w = to_dev(cat, torch)
+    zo, co = oracle_zeta(cat)
+    out = []
+    for budget in (0, 1 << 20):
+        plan = g3.Plan(**cat.params())
+        plan.set_option(g3.OPT_CELLS_PER_RMAX, cells)
+        plan.set_option(g3.OPT_LIST_BYTES, budget)
+        z, c = plan.compute(pos, w, fp32_contraction=True)
+        np.testing.assert_array_equal(c.cpu().numpy(), co)
+        out.append(z.cpu().numpy())
+    np.testing.assert_array_equal(out[0], out[1])
+    # FP64 points that FP32 cannot tell apart have no FP32 direction: their bins are NaN
+    # here as in the fused kernel, which shares none of this path
+    plan = g3.Plan(**cat.params())
+    plan.set_option(g3.OPT_PAIR_KERNELS, 1)
+    bad = np.isnan(plan.compute(pos, w, fp32_contraction=True)[0].cpu().numpy())
+    assert f64 or not bad.any()
+    np.testing.assert_array_equal(np.isnan(out[0]), bad)
+    # a_lm: at most 2000 / 32 partial sums per lane, ~45 more operations: (63 + 45) 2^-24
+    # of sum |w| K_lm; a product of two, K_lm^2 <= (2 lmax + 1) K_00^2
+    assert np.abs(np.where(bad, 0, out[0] - zo)).max() <= 1.3e-5 * (2 * lmax + 1) * max(np.abs(zo).max(), 1e-300)
