@@ -29,7 +29,7 @@
 //                 pipe runs at 1/58 of the FP32 rate.  Bound by issue, with
 //                 shared memory (records in and out) close behind: 1,250 cycles
 //                 per chunk and SM quarter at lmax = 6.  100,000 clustered
-//                 points, lmax = 6 (7.1e8 pairs): 24 ms, against 40 ms with
+//                 points, lmax = 6 (7.1e8 pairs): 23.5 ms, against 40 ms with
 //                 12 instead of 6 operations per term and one sum pair per lane
 //                 (twice the shared-memory bytes per term).  Sums in the
 //                 registers of the pair's lane alone (no records, a
@@ -37,12 +37,24 @@
 //                 times this kernel's time at 55 pairs per bin and lmax = 10.
 //   k_adj_df   -- per primary (one warp), one pair per lane: the adjoint
 //                 coefficients G_{m,k} = w_i sum_l c^(m)_{l-m,k} K_lm V_lm of
-//                 the primary (FP64 from the FP64 V = M A, held as head + tail
-//                 in shared memory), and per pair F = sum Re(conj(G) T_k
-//                 (x + iy)^m) with its gradient in double-float (F with dF/dz,
-//                 and the per-m sums against T_k and T_k', as packed f32x2
-//                 pairs), rounded once to FP32 per pair; FP64 atomics for the
-//                 secondary, a double-float sum for the primary.
+//                 the primary (double-float, from the double-float V = M A,
+//                 in shared memory with a bound of each bin's sums), the
+//                 primary's weight term Re(A^H V), and per pair
+//                 F = sum Re(conj(G) T_k (x + iy)^m) with its gradient in
+//                 double-float: per m the sums against T_k and T_k' on (Re, Im)
+//                 pairs with biased heads, then their products with
+//                 (x + iy)^(m-1), whose partial sums as m descends are the x
+//                 and y derivatives.  Rounded once to FP32 per pair; FP64
+//                 atomics for the secondary, a double-float sum for the
+//                 primary.  Bound by issue: about 1,450 cycles of arithmetic
+//                 per chunk and SM quarter at lmax = 6, of 1,880.  100,000
+//                 clustered points, lmax = 6: 36 ms against 57 with error-free
+//                 additions and an FP32 pair per derivative.  Resident CTAs (registers):
+//                 at lmax = 10 four take 2.08 ms on 1.1e7 pairs, three 2.14, two,
+//                 without any limit on the registers, 2.44; at lmax = 4 five
+//                 take 0.83 and four 0.86; at lmax = 6 three and five are 3% slower
+//                 than four.  k_accum_df likewise: at lmax = 6 six CTAs 23.5 ms, five
+//                 24.2, four 25.0; at lmax = 8 four are the best.
 #include "pair_common.cuh"
 
 namespace g3 {
@@ -255,7 +267,7 @@ __host__ __device__ constexpr size_t accum_df_smem_per_warp(int RL, int RS, int 
 }
 
 template <int L>
-__global__ void __launch_bounds__(kDThreads, L <= 8 ? 4 : 3) k_accum_df(ListArgs a) {
+__global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_accum_df(ListArgs a) {
     using R_ = DfRec<L>;
     constexpr int RS = R_::RS, G = R_::G, M0 = R_::M0, KE = R_::KE;
     constexpr int NR = Shape<L>::NR, NRP = Shape<L>::NRP;
@@ -568,7 +580,7 @@ __host__ __device__ constexpr size_t adj_df_smem_per_warp(int B, int N) {
 __device__ __forceinline__ float2 unbias(float2 H, float b) { return __fadd2_rn(H, dup(-b)); }
 
 template <int L>
-__global__ void __launch_bounds__(kDThreads, L <= 6 ? 4 : (L <= 8 ? 3 : 2)) k_adj_df(ListArgs a) {
+__global__ void __launch_bounds__(kDThreads, L <= 5 ? 5 : 4) k_adj_df(ListArgs a) {
     constexpr int NR = Shape<L>::NR;
     using G_ = AdjG<L>;
     extern __shared__ __align__(16) unsigned char draw[];
@@ -696,7 +708,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 4 : (L <= 8 ? 3 : 2)) k_ad
                         T[k] = df_add(df_mul(z2, T[k - 1]), df_neg(T[k - 2]));
                         D[k] = df_mulf(u1, (float)k);
                         if constexpr (k < L) {
-                            const df u2 = df_add(df_mul(z2, u1), df_neg(u0));
+                            const df u2 = df_add({2.f * T[k].h, 2.f * T[k].l}, u0);  // U_k = 2 T_k + U_{k-2}
                             u0 = u1;
                             u1 = u2;
                         }
