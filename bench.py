@@ -52,17 +52,21 @@ def zeta_flops_per_primary(nbins: int, L: int) -> int:
 
 # Executed FP32 flops per pair of the accumulate kernel (Chebyshev form, FMA = 2):
 # T_k recurrence 2(L-1), m = 0 sums 2L + 1, m >= 1 terms 2 L + 4 L (L - 1) / 2 x 2,
-# (x + iy)^m 6 (L - 1) + 2, separation and unit vector 12.
+# (x + iy)^m 6 (L - 1) + 2.  The scan forms the separation and unit vector: 12 more
+# for the pair stage.
+UNIT_VECTOR_FLOPS = 12
+
+
 def accum_exec_flops(L: int) -> int:
     if L == 0:
-        return 13
-    return 2 * (L - 1) + (2 * L + 1) + 2 * L + 4 * (L * (L + 1) // 2 - L) + 6 * (L - 1) + 2 + 12
+        return 1
+    return 2 * (L - 1) + (2 * L + 1) + 2 * L + 4 * (L * (L + 1) // 2 - L) + 6 * (L - 1) + 2
 
 
-# DRAM bytes of one k_accum launch per primary, from the ncu capture summarised
-# in profiles/k_accum_clustered_200k_L696.md (17.60 GB for 200,000 primaries,
+# DRAM bytes of one k_accum_dir launch per primary, from the ncu capture summarised
+# in profiles/k_accum_clustered_200k_L696.md (1.629 GB for about 4,970 primaries,
 # Lambda = 10); a full-size launch is scaled by its primaries.
-ACCUM_DRAM_BYTES_PER_PRIMARY = 17.60e9 / 200000
+ACCUM_DRAM_BYTES_PER_PRIMARY = 1.629e9 / 4970
 
 
 def peaks():
@@ -547,7 +551,7 @@ def run_ours(args):
         "roofline": {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                      "frac": achieved / fp32_peak,
                      "traffic": ACCUM_DRAM_BYTES_PER_PRIMARY * nprim / n_acc if L == 10 else None,
-                     "kernel": "k_accum<%d> (FP32 FMA pipe), %d launches per step, %.2f ms per launch"
+                     "kernel": "k_accum_dir<%d> (FP32 FMA pipe), %d launches per step, %.2f ms per launch"
                                % (L, n_acc, accum_ms / n_acc),
                      "peak_source": "measured: g3pcf_fp32_peak FMA-chain probe on this GPU "
                                     "(nominal 2 x 128 lanes x %d SMs x %.0f MHz = %.1f)" % (n_sm, clk_max, nominal),
@@ -559,7 +563,7 @@ def run_ours(args):
                      "pair_stage": {"ms": pair_ms,
                                     "achieved": pairs * pair_flops(L) / (pair_ms / 1e3) / 1e12,
                                     "frac": pairs * pair_flops(L) / (pair_ms / 1e3) / 1e12 / fp32_peak,
-                                    "frac_executed": pairs * accum_exec_flops(L) / (pair_ms / 1e3) / 1e12
+                                    "frac_executed": pairs * (accum_exec_flops(L) + UNIT_VECTOR_FLOPS) / (pair_ms / 1e3) / 1e12
                                                      / fp32_peak}},
         "e2e": {"value": e2e_val, "unit": "pairs/s",
                 "h2d_bytes_per_step": int(hpos.numel() * 4 + hw.numel() * 4),
