@@ -7,7 +7,8 @@
 //      V_i = M_m A_i                    (k_vgemm, per m block, FP32; k_vgemm_df
 //                                        in double-float for the double-float
 //                                        pair pass)
-//      dL/dw_i (as a primary) = Re(A_i^H V_i)   (fused into k_vgemm)
+//      dL/dw_i (as a primary) = Re(A_i^H V_i)   (FP32: fused into k_vgemm;
+//                                        double-float: in k_adj_df)
 //      H_i = w_i V_i                    (applied by the adjoint pair pass)
 // (per catalog c of a batched forward, M is built from that catalog's dL/dzeta_c)
 // and the pair pass (k_adj over the pair lists, or the fused k_pair mode 1)

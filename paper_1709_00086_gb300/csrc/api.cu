@@ -154,7 +154,7 @@ struct g3pcf_plan_s {
     bool exact_alm = false;  // this forward runs with G3PCF_F_KEEP_ALM
     int gl_events = 0;  // events the capture run will record
     DevBuf l_gbase, l_scantmp, l_passq;
-    // events around every k_scan / k_accum launch of the last forward: start, middle
+    // events around every k_scan and accumulate launch of the last forward: start, middle
     // and end of each pass (levq: the handles in order; the last end of a forward that
     // is not chunked is ev[2])
     std::vector<cudaEvent_t> lev, levq;
@@ -677,9 +677,10 @@ int run_list_pass(g3pcf_plan_t P, ListArgs& la, const PairArgs& pa, int mode, bo
     return G3PCF_OK;
 }
 
-// Forward pair stage through pair lists for the primaries [pa.q0, pa.nprim):
-// count candidates, bring the per-primary chunk bounds to the host, split the
-// range into passes whose lists fit the pool, then scan + accumulate each pass.
+// Pair stage through pair lists for the primaries [pa.q0, pa.nprim): count the
+// candidates, bring the totals to the host, and scan + accumulate (mode 0) in one
+// pass if the pool holds the lists, else in passes placed by the host from the
+// per-primary bounds.
 int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode = 0) {
     const int qa = pa.q0, qb = pa.nprim;
     const int64_t nq = (int64_t)qb - qa;

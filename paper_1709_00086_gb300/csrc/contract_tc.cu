@@ -21,7 +21,9 @@
 // panel is the first column panel.  The primaries of every catalog are cut
 // into an even number of equal "virtual segments"; a two-tile strip takes one
 // per CTA and a one-tile strip two, so that every CTA does the same MMA work
-// (its partial goes to the first slot and the second is zeroed).
+// (its partial goes to the first slot and the second is zeroed), or one of its two
+// parts, cut at an accumulation run, where whole items would leave SMs idle (each
+// part then has its own slot; schedule_tc_items).
 //   warp 9 (TMA): per k-block of 64 primaries and panel, one 2-D bulk copy of
 //     the FP32 rows of A (the columns the panel's MMAs use, from the panel's
 //     first column rounded down to a 16-byte boundary) into a staging slot,
@@ -616,8 +618,8 @@ __global__ void __launch_bounds__(kTcWarps * 32, 1)
                      : "memory");
 }
 
-// ---- the same contraction from bf16 operand rows written by k_accum ----------
-// On request (G3PCF_OPT_TC_OPERANDS = 1) and when no weight is negative, k_accum
+// ---- the same contraction from bf16 operand rows of the accumulate kernel ----
+// On request (G3PCF_OPT_TC_OPERANDS = 1) and when no weight is negative, emit_row
 // writes sqrt(w) A split into bf16 hi and lo rows (the same operations as the
 // converter warps, so the operands and the result are bit-identical), each m
 // block from a multiple of 64 columns, a row's hi and lo side by side.  The

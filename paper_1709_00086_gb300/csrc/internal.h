@@ -150,11 +150,12 @@ size_t pair_smem_per_warp(int lmax, int nbins, int kflush);
 // ---- pairlist.cu -----------------------------------------------------------
 // Forward pair stage as three kernels over the primaries [qa, qb) (processing
 // order): k_count writes need[q] = ceil(candidates / 32) + nbins (an upper
-// bound of the list chunks of q); the host sets base[q] (first chunk of q in
-// the pool, relative to the pass) so that a pass fits the pool; k_scan writes
-// the chunks (32 entries j | code << 27, padding 0xffffffff), the list of them
-// ordered by bin (ord: chunk | bin << 26) and nchunks[q]; k_accum walks that
-// list and writes A rows.
+// bound of the list chunks of q); base[q] (first chunk of q in the pool, relative
+// to the pass) comes from a counter in k_scan or, in several passes, from the host
+// or the device planner, so that a pass fits the pool; k_scan writes the chunks (32
+// direction records, padding of weight 0, or 32 entries j | code << 27, padding
+// 0xffffffff), the list of them ordered by bin (ord: chunk | bin << 26) and
+// nchunks[q]; k_accum_dir or k_accum walks that list and writes A rows.
 struct ListArgs {
     const float4* pts;
     const double* pts64;
@@ -207,7 +208,7 @@ struct ListArgs {
     const float2* colcoefdf;     // Chebyshev -> Legendre-form coefficients (times K_lm), head + tail
     const float2* slotcoefdf;    // slotcoef likewise
     const float2* Vdf;           // V rows as head + tail pairs (double-float adjoint)
-    // tensor-core operands written by k_accum (forward, no negative weight):
+    // tensor-core operands written with the rows of A (forward, no negative weight):
     // sqrt(w) A split into bf16 hi and lo: row r holds hi at bop + 2 r bop_pitch and
     // lo bop_pitch later (one contiguous stretch per row), m blocks from multiples
     // of 64 (operand columns in rowconv), rows in
@@ -345,7 +346,7 @@ int launch_contract_tc(const float* A, int RLP, int RL, int64_t arows, const flo
                        const Tile* tiles, const TcStrip* strips, const TcItem* items, int nitems,
                        const Segment* segs, double* partials, int part_stride, const int* negw, int* status,
                        cudaStream_t st, int test_timeout = 0);
-// Operand columns of the bf16 rows written by k_accum: every m block starts on a
+// Operand columns of the bf16 rows written by emit_row: every m block starts on a
 // multiple of 64; blk[m] = {first A column, width, first operand column, 0}
 // (m <= lmax < max_blk); returns the row pitch, or -1
 int tc_operand_blocks(const Tile* tiles, int ntiles, int4* blk, int max_blk);

@@ -7,14 +7,16 @@
 // primary and bin instead of one per pair group).
 //
 //   k_count  -- per primary, the number of candidate secondaries in the
-//               sphere's cell rows; the host turns ceil(candidates/32) + B
-//               into exact, non-overlapping list offsets and into passes that
-//               fit the list pool.
+//               sphere's cell rows: at most ceil(candidates/32) + B chunks.
+//               One pass over the list pool if it holds the total (k_scan
+//               takes its chunks from a counter), else the host places every
+//               primary's chunks and cuts the range into passes.
 //   k_scan   -- per primary (one warp), streams the candidates of 32 cell rows
 //               at a time, slot range by slot range, decides each pair's bin
-//               exactly and compacts the accepted pairs into a stage in shared
-//               memory; every 32 staged pairs are placed into per-bin chunks of
-//               32 (tagged with the bin) of this primary.  For a plain forward
+//               exactly and places the accepted pairs into per-bin chunks of
+//               32 (tagged with the bin) of this primary, straight from the
+//               candidates' lanes or, where fewer than half of them are
+//               pairs, gathered in groups of 32 first.  For a plain forward
 //               a chunk holds 32 direction records (unit vector and weight, 512
 //               bytes), for the calls that differentiate 32 list entries (slot
 //               and image, 128 bytes).
@@ -155,10 +157,10 @@ __global__ void __launch_bounds__(kCountThreads) k_count(ListArgs a, int lpp) {
     }
 }
 
-// k_scan: about 180 warp instructions per 32 accepted pairs, and every
-// instruction slot counts: a packed FMA takes two issue cycles, logic and selects
-// two on their pipe, so the kernel is bound by issue and by the shared-memory
-// pipe (70% busy), not by DRAM.  The unit vector is formed here because the
+// k_scan: 125 warp instructions per 32 accepted pairs at 3.7 cells per rmax, and
+// every instruction slot counts: logic and selects take two cycles on their pipe,
+// match.any 72 beside the other warps' work, so the kernel is bound by issue
+// (staged also by the shared-memory pipe, 70% busy), not by DRAM.  The unit vector is formed here because the
 // distance test has the separation and 1/r at hand: gathering the point again and
 // forming it in the accumulate kernel cost about 100 cycles per chunk there.  The
 // bin comes from r = r^2 rsqrt(r^2) by one rounding instead of a table look-up
@@ -866,10 +868,11 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
 // and the harmonics.  Bound by issue: at lmax = 10 a chunk's 55 packed FMAs take
 // two issue cycles each, the recurrences of T_k and (x + iy)^m about 65 more, the
 // list walk about 30; the loop body without any load measures 208 cycles per chunk
-// and SM quarter, the kernel 232 (the form that gathers points from list entries:
-// 310).  200,000 clustered points (L = 696, 4.0e9 pairs, lmax = 10): 25.2 ms
+// and SM quarter, the kernel 226 (the form that gathers points from list entries:
+// 310).  200,000 clustered points (L = 696, 4.0e9 pairs, lmax = 10): 24.5 ms
 // against 33.8.  The list words of 32 chunks are held one per lane and read by
-// shuffle (a load per chunk: 25.9 ms).
+// shuffle (a load per chunk: 0.7 ms more).  20,000 uniform points (67 pairs per
+// bin): 298 us, of which the butterflies are 86 and the rows of A 70.
 constexpr int kDirRing = 8;
 __host__ __device__ constexpr size_t accum_dir_smem_per_warp(int B, int NRP) {
     return (((size_t)B * res_stride(NRP) * 4 + 15) & ~(size_t)15) + kDirRing * 32 * 16;
