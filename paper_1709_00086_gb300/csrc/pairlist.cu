@@ -63,7 +63,7 @@ struct ScanSmem {
     int2 pcs[kMaxPieces];
     Item stage[N];
     int sbin[N];
-    int bst[32];
+    int bst[64];  // (63: lanes without a bin)
     int bnbc[32];
     double pd[4];
     float R[12];
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count(ListArgs a, int lpp) {
 // the candidates near an edge take the exact rule.  32 warps per SM at 64
 // registers: 40 and 48 are 6% and 24% slower.  Staged, two or three loads per trip
 // instead of four are 10% and 3% slower; direct (no stage), three and two are the same,
-// four spill (3%).  200,000 clustered points (L = 696, 4.0e9 pairs): 16.8 ms writing
+// four spill (3%).  200,000 clustered points (L = 696, 4.0e9 pairs): 16.0 ms writing
 // 16 bytes per pair (staged 19.7, which is what the form took that wrote 4 bytes
 // and left the direction to the accumulate kernel).
 //
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
         int nch = 0;                   // chunks opened so far (warp-uniform)
         // per bin: the last written slot of the open chunk (chunk * 32 + position;
         // -1, like any full chunk, has position 31) and the chunks opened so far
-        S.bst[lane] = -1;
+        S.bst[lane] = S.bst[32 + lane] = -1;
         S.bnbc[lane] = 0;
         __syncwarp();
 
@@ -293,17 +293,17 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
         // lane opens the chunk and leaves the bin's last slot.
         auto place = [&](typename Smem::Item it, int bin, bool v, unsigned mine) {
             const int rank = __popc(mine & lt);
-            const int st = S.bst[bin & 31];
-            const int f = (st & 31) + 1 + rank;
+            const int st = S.bst[bin];
             int sl = st + 1 + rank;
+            const bool cross = (unsigned)(sl ^ st) >= (unsigned)kChunk;  // past the open chunk
             const bool last = v && (mine & gt) == 0u;
-            const bool opens = last && f >= kChunk;
+            const bool opens = last && cross;
             const unsigned gm = __ballot_sync(kFull, opens);
             if (gm) {
                 // the new chunk of this lane's group: numbered by the groups' highest lanes
-                const int hl = 31 - __clz((int)mine);
-                const int nnew = nch + __popc(gm & ((1u << hl) - 1u));
-                if (f >= kChunk) sl = nnew * kChunk + (f - kChunk);
+                // (mine & gm: the highest lane's bit)
+                const int nnew = nch + __popc(gm & ((mine & gm) - 1u));
+                if (cross) sl = nnew * kChunk + (sl & (kChunk - 1));
                 nch += __popc(gm);
                 if (opens) {
                     const int nb = S.bnbc[bin];
