@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count(ListArgs a, int lpp) {
     }
 }
 
-// k_scan: 125 warp instructions per 32 accepted pairs at 3.7 cells per rmax, and
+// k_scan: 116 warp instructions per 32 accepted pairs at 3.7 cells per rmax, and
 // every instruction slot counts: logic and selects take two cycles on their pipe,
 // match.any 72 beside the other warps' work, so the kernel is bound by issue
 // (staged also by the shared-memory pipe, 70% busy), not by DRAM.  The unit vector is formed here because the
