@@ -756,18 +756,24 @@ int run_pair_lists(g3pcf_plan_t P, const PairArgs& pa, cudaStream_t st, int mode
             return fail(G3PCF_ERR_STATE, "graph capture without a matching warm-up forward");
         const ListWarm wm = P->gl_warm[P->gl_idx++];
         dirs = wm.dirs;
-        const int64_t C = (int64_t)(P->l_pool.bytes / (dirs ? 512 : 128));
+        // (the pool may have been sized for the other chunk size: the tags bound it too)
+        const int64_t C = (int64_t)std::min({P->l_pool.bytes / (dirs ? 512 : 128), P->l_tag.bytes / 4,
+                                             P->l_ord.bytes / 4});
         // one pass where the pool holds the lists with headroom, else passes planned
         // on the device
         const bool one = wm.total + wm.total / 4 <= C;
         int64_t slack = 0, stride = 0;
         int npass = 1;
         if (!one) graph_plan_sizes(C, wm.total, wm.most, P->nbins, slack, stride, npass);
-        if (C < 1 || (int64_t)P->l_tag.bytes / 4 < C || (int64_t)P->l_ord.bytes / 4 < C ||
+        if (C < 1 ||
             (!one && (stride < 1 || P->l_gbase.bytes < 8 * (size_t)nq ||
                       P->l_passq.bytes < 4 * (size_t)(npass + 1) || P->l_scantmp.bytes < plan_scan_tmp_bytes(nq))) ||
             (int)P->lev.size() < P->lev_used + 3 * npass) {
-            ++P->launches;  // the warm-up did not size the plan (cannot happen): the fused kernel
+            // the warm-up did not size the plan: the fused kernel, which has neither the
+            // double-float multipoles nor the monomial basis
+            if (la.exact_img || P->opt_basis != 0)
+                return fail(G3PCF_ERR_STATE, "graph capture: the warm-up forward did not size the pair lists");
+            ++P->launches;
             if (launch_pair(P->lmax, pa, P->nsm, st) != 0)
                 return fail(G3PCF_ERR_CUDA, "pair kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
             return G3PCF_OK;
