@@ -218,6 +218,15 @@ __device__ __forceinline__ void bias_fma(float2& H, float2& Lo, float2 Th, float
     Lo = __ffma2_rn(Tl, Ch, __fadd2_rn(Lo, e));
     H = s;
 }
+// (H, Lo) += T c for a head without a bias (an error-free addition, 11 operations)
+__device__ __forceinline__ void df_fma2(float2& H, float2& Lo, float2 Th, float2 Tl, float2 c) {
+    const float2 p = __fmul2_rn(Th, c);
+    const float2 pe = __ffma2_rn(Th, c, neg2(p));
+    const float2 s = __fadd2_rn(H, p), bb = __fadd2_rn(s, neg2(H));
+    const float2 er = __fadd2_rn(__fadd2_rn(H, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
+    Lo = __ffma2_rn(Tl, c, __fadd2_rn(Lo, __fadd2_rn(er, pe)));
+    H = s;
+}
 // (H, Lo) += C
 __device__ __forceinline__ void bias_add(float2& H, float2& Lo, float2 Ch, float2 Cl) {
     const float2 s = __fadd2_rn(H, Ch);
@@ -255,12 +264,7 @@ struct DfRec {
     // record stride (floats), an odd number of 16-byte units: conflict-free stores
     static constexpr int RS = ((4 * L + 2 * KE) / 4 % 2) ? 4 * L + 2 * KE : 4 * L + 2 * KE + 4;
     static constexpr int M0 = (L + 2) / 2;  // packed pairs of m = 0
-    // bias of a chunk's sums (32 / G terms of size <= 1)
-    static constexpr float kBias = 32.f / G + 8.f;
 };
-// Bias of the m = 0 sums: one term of size <= 1 per chunk and lane, flushed after 32.
-constexpr int kBiasChunks = 32;
-constexpr float kBias0 = 40.f;
 
 __host__ __device__ constexpr size_t accum_df_smem_per_warp(int RL, int RS, int NRP) {
     return (size_t)32 * RS * 4 + 54 * 16 + 9 * 8 + 8 + (size_t)NRP * 8 + (size_t)((RL + 3) & ~3) * 4;
@@ -327,32 +331,34 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
         const int* chunks = a.chunks + (int64_t)cb * 32;
         const int* ordp = a.ord + cb;
         __syncwarp();
-        // m = 0: packed (k, k + 1); m >= 1: this lane's sums k0 and k0 + 1 as (Re, Im)
-        // (biased: Ha .. Lb; added to SaH .. SbL after every chunk, so that the bias, which
-        // sets the rounding, stays near the sums)
-        float2 H0[M0], L0[M0], Ha, La, Hb, Lb, SaH, SaL, SbH, SbL;
+        // m = 0: packed (k, k + 1), error-free additions (one per chunk and lane); m >= 1: this
+        // lane's sums k0 and k0 + 1 as (Re, Im), biased by 2 + the chunk's terms (each of size
+        // <= 1) in Ha .. Lb, and added to SaH .. SbL after every chunk.  The residues that the
+        // tail gathers are half an ulp of a head near the bias, so that the bias sets the
+        // rounding: emulated with random terms, 2^-45 of the largest |w| (rms) after 4 terms,
+        // 2^-42 after 16, 2^-40 after 32, 2^-38 after 200 (error-free heads: 2^-49, 2^-45,
+        // 2^-44, 2^-42), where the stored row is rounded to 2^-25 of the entry.
+        float2 H0[M0], L0[M0], SaH, SaL, SbH, SbL;
         auto clear = [&]() {
             static_for<0, M0>([&](auto ic) {
-                H0[decltype(ic)::value] = dup(kBias0);
-                L0[decltype(ic)::value] = dup(0.f);
+                H0[decltype(ic)::value] = L0[decltype(ic)::value] = dup(0.f);
             });
-            Ha = Hb = dup(R_::kBias);
-            La = Lb = SaH = SaL = SbH = SbL = dup(0.f);
+            SaH = SaL = SbH = SbL = dup(0.f);
         };
         clear();
-        auto fold1 = [&](float2& SH, float2& SL, float2& H, float2& Lo) {
-            const float2 x = __fadd2_rn(H, dup(-R_::kBias));  // exact
+        auto fold1 = [&](float2& SH, float2& SL, float2 H, float2 Lo, float bias) {
+            // H = bias + x + xe (a head near 2 has a finer grid than x near -bias)
+            const float2 x = __fadd2_rn(H, dup(-bias));
+            const float2 xe = __fadd2_rn(H, neg2(__fadd2_rn(x, dup(bias))));
             const float2 s = __fadd2_rn(SH, x), bb = __fadd2_rn(s, neg2(SH));
             const float2 er = __fadd2_rn(__fadd2_rn(SH, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(x, neg2(bb)));
-            SL = __fadd2_rn(SL, __fadd2_rn(er, Lo));
+            SL = __fadd2_rn(SL, __fadd2_rn(__fadd2_rn(er, xe), Lo));
             SH = s;
-            H = dup(R_::kBias);
-            Lo = dup(0.f);
         };
         // |w| <= cap (a power of two fixed by the first weights of a bin; a larger one
         // flushes the sums): the sums take w / cap
         unsigned cap = 0u;
-        int cnt = 0;
+        bool held = false;  // the sums hold a chunk of this cap
         float inv = 1.f, scale = 1.f;
         // the sums, times cap, into res
         auto flush = [&]() {
@@ -383,7 +389,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
             float h[L + 1], l[L + 1];
             static_for<0, L + 1>([&](auto kc) {
                 constexpr int k = decltype(kc)::value;
-                h[k] = ((k & 1) ? H0[k / 2].y : H0[k / 2].x) - kBias0;
+                h[k] = (k & 1) ? H0[k / 2].y : H0[k / 2].x;
                 l[k] = (k & 1) ? L0[k / 2].y : L0[k / 2].x;
             });
             int b0 = 0, size = L + 1;
@@ -420,7 +426,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
                 res[b0] = make_float2(v.h, v.l);
             }
             clear();
-            cnt = 0;
+            held = false;
         };
         // list words three chunks ahead, entries two, points one
         auto word = [&](int i) { return (unsigned)__ldg(ordp + (i < nch ? i : nch - 1)); };
@@ -444,16 +450,14 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
             const bool v = e != kNoPairD;
             const unsigned wm = __reduce_max_sync(kFull, v ? __float_as_uint(fabsf(qv.w)) : 0u);
             const int nv = __popc(__ballot_sync(kFull, v));  // the chunk's pairs, its first lanes
-            if (wm > cap || cnt == kBiasChunks) {
-                if (cnt > 0) flush();
-                if (wm > cap) {
-                    const unsigned ex = min((wm >> 23) + 1u, 253u);
-                    cap = ex << 23;
-                    scale = __uint_as_float(cap);
-                    inv = __uint_as_float((254u - ex) << 23);
-                }
+            if (wm > cap) {
+                if (held) flush();
+                const unsigned ex = min((wm >> 23) + 1u, 253u);
+                cap = ex << 23;
+                scale = __uint_as_float(cap);
+                inv = __uint_as_float((254u - ex) << 23);
             }
-            ++cnt;
+            held = true;
             {
                 // this lane's pair -> its record; a padding lane takes a unit separation
                 // and weight 0
@@ -482,8 +486,8 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
                 });
                 static_for<0, M0>([&](auto ic) {
                     constexpr int k = 2 * decltype(ic)::value;
-                    bias_fma(H0[k / 2], L0[k / 2], make_float2(T[k].h, T[k + 1].h), make_float2(T[k].l, T[k + 1].l),
-                             dup(w));
+                    df_fma2(H0[k / 2], L0[k / 2], make_float2(T[k].h, T[k + 1].h), make_float2(T[k].l, T[k + 1].l),
+                            dup(w));
                     if constexpr (k < KE) my[(R_::TB + 2 * k) / 4] = make_float4(T[k].h, T[k].l, T[k + 1].h, T[k + 1].l);
                 });
                 if constexpr (L >= 1) {
@@ -506,6 +510,8 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
                 // records past the last pair hold weight 0)
                 const float* rt = rec + grp * RS;
                 const int steps = (nv + G - 1) / G;
+                const float bias = (float)(steps + 2);
+                float2 Ha = dup(bias), Hb = Ha, La = dup(0.f), Lb = La;
                 for (int t = 0; t < steps; t += U, rt += U * G * RS) {
                     float4 T4[U], C4[U];
 #pragma unroll
@@ -520,8 +526,8 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
                         bias_fma(Hb, Lb, dup(T4[u].z), dup(T4[u].w), Ch, Cl);
                     }
                 }
-                fold1(SaH, SaL, Ha, La);
-                fold1(SbH, SbL, Hb, Lb);
+                fold1(SaH, SaL, Ha, La, bias);
+                fold1(SbH, SbL, Hb, Lb, bias);
                 __syncwarp();
             }
             if (i + 1 == nch || (o0 ^ o1) >> 26) {  // the bin's last chunk: its columns of the row
