@@ -139,54 +139,70 @@ __global__ void __launch_bounds__(kVThreads) k_vgemm(const float* __restrict__ A
     }
 }
 
-// M of one catalog for the double-float path, one warp per row c: entries as head +
-// tail, and the row's sum of |M|, which bounds the sums of k_vgemm_df.  The real
-// form is symmetric, so that row c is also column c.
-constexpr int kBWarps = 8;
-__global__ void __launch_bounds__(kBWarps * 32) k_build_m_df(const double* dz, MInfo mi, int lmax, int RL,
-                                                            int64_t zsize, size_t mfloats, float2* Mr, float* norm) {
-    const int lane = threadIdx.x & 31, cat = blockIdx.y;
-    const int col = blockIdx.x * kBWarps + (threadIdx.x >> 5);
-    if (col >= RL) return;
-    int m = 0;
-    while (m < lmax && col >= mi.col0[m + 1]) ++m;
-    const int K = mi.K[m], W = mi.W[m], rr = col - mi.col0[m], r = rr % K;
+// M of one catalog for the double-float path, one CTA per order m and bin b1, one warp per
+// row c of that bin: entries as head + tail, and for every bin b2 the largest row sum of |M|
+// over the columns of b2 (norm[m][b1][b2]), which bounds the sums of k_vgemm_df.  The real
+// form is symmetric, so that row c is also column c.  Lane = b2 + nbins x share: 32 / nbins
+// lanes share a bin's columns.
+constexpr int kBWarps = 16;
+__global__ void __launch_bounds__(kBWarps * 32) k_build_m_df(const double* dz, MInfo mi, int nbins, int64_t zsize,
+                                                            size_t mfloats, size_t nfloats, float2* Mr, float* norm) {
+    __shared__ float s_max[kBWarps][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, cat = blockIdx.y;
+    const int m = blockIdx.x / nbins, b1 = blockIdx.x - m * nbins;
+    const int K = mi.K[m], W = mi.W[m], shares = 32 / nbins;
     const double* Z = dz + 2 * ((int64_t)cat * zsize + mi.zoff[m]);
-    float2* out = Mr + (size_t)cat * mfloats + mi.moff[m] + (int64_t)rr * W;
-    float sum = 0.f;
-    for (int cc = lane; cc < W; cc += 32) {
-        const int c = cc % K;
-        // M = G + G^H, G = dz / 2
-        const double re = 0.5 * (Z[2 * ((int64_t)r * K + c)] + Z[2 * ((int64_t)c * K + r)]);
-        const double im = 0.5 * (Z[2 * ((int64_t)r * K + c) + 1] - Z[2 * ((int64_t)c * K + r) + 1]);
-        const bool rlo = rr < K, clo = cc < K;
-        const float2 v = m_entry(m == 0 || rlo == clo ? re : (rlo ? -im : im));
-        out[cc] = v;
-        sum += fabsf(v.x);
+    float most = 0.f;
+    for (int rr = b1 + wid * nbins; rr < W; rr += kBWarps * nbins) {
+        const int r = rr % K;
+        float2* out = Mr + (size_t)cat * mfloats + mi.moff[m] + (int64_t)rr * W;
+        float sum = 0.f;
+        for (int cc = lane; lane < shares * nbins && cc < W; cc += shares * nbins) {
+            const int c = cc % K;
+            // M = G + G^H, G = dz / 2
+            const double re = 0.5 * (Z[2 * ((int64_t)r * K + c)] + Z[2 * ((int64_t)c * K + r)]);
+            const double im = 0.5 * (Z[2 * ((int64_t)r * K + c) + 1] - Z[2 * ((int64_t)c * K + r) + 1]);
+            const bool rlo = rr < K, clo = cc < K;
+            const float2 v = m_entry(m == 0 || rlo == clo ? re : (rlo ? -im : im));
+            out[cc] = v;
+            sum += fabsf(v.x);
+        }
+        float tot = sum;
+        for (int sh = 1; sh < shares; ++sh) tot += __shfl_sync(0xffffffffu, sum, (lane + sh * nbins) & 31);
+        most = fmaxf(most, tot);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) norm[(size_t)cat * RL + col] = sum;
+    s_max[wid][lane] = most;
+    __syncthreads();
+    if (wid == 0 && lane < nbins) {
+        for (int w = 1; w < kBWarps; ++w) most = fmaxf(most, s_max[w][lane]);
+        norm[cat * nfloats + blockIdx.x * nbins + lane] = most;
+    }
 }
 
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 // V = M A in double-float (M head + tail, A exact), 8 rows of one catalog per CTA,
 // one column per thread at a time, two rows per packed operation.  The head of
-// every sum carries a bias of three times its bound (the row sum of |M| times the
-// largest |A| of the block), so that the difference to the next head is exact and
-// one FMA returns the rounding error: 5 operations per multiply-add (10 with an
-// error-free addition).  Bound by issue; M (from L2) is read once per 8 rows,
+// every sum carries a bias of three times its bound, so that the difference to the next
+// head is exact and one FMA returns the rounding error: 5 operations per multiply-add (10
+// with an error-free addition).  The tail gathers half an ulp of the bias per term, about
+// 2^-44 of the bound (rms, 140 terms), so the bound keeps apart what the gradient keeps
+// apart: it is formed per row (neighbours of any size share a CTA), and per bin of the
+// column as the sum over the bins b of M's largest row sum in b times the row's largest
+// |A| there (bins that dL/dzeta leaves out count nothing).  Bound by issue; M (from L2) is read once per 8 rows,
 // coalesced by its symmetry (16 rows per CTA: the same time).  20,000 rows at B =
-// lmax = 10: 0.65 ms against 1.73.
+// lmax = 10: 0.68 ms against 1.73 with error-free additions (0.65 with one bias per CTA
+// and order); 85 registers and three CTAs per SM, as 64 and four take 0.82.
 // The primary-weight term Re(A^H V) is the pair pass's (k_adj_df).
-__global__ void __launch_bounds__(kVThreads, 4) k_vgemm_df(
+__global__ void __launch_bounds__(kVThreads, 3) k_vgemm_df(
     const float* __restrict__ A, int RLP, int RL, const int4* __restrict__ blks, int64_t row_lo, int64_t row_hi,
-    const float2* __restrict__ Mall, const float* __restrict__ norm, size_t mfloats, MInfo mi, int lmax,
+    const float2* __restrict__ Mall, const float* __restrict__ norm, size_t mfloats, MInfo mi, int nbins, int lmax,
     float2* V) {
     constexpr int R = kRows, RS = R + 4;  // rows, column stride in shared memory
     extern __shared__ __align__(16) float sA[];  // RL x RS
-    __shared__ int amax[kMaxL + 1];
+    const int nmb = (lmax + 1) * nbins;
+    float* amax = sA + (size_t)RL * RS;  // [m][bin][row]: largest |A|
+    float* bias = amax + nmb * R;        // [m][bin][row]
     int4 blk;
     if (blks) {
         blk = blks[blockIdx.x];
@@ -195,22 +211,27 @@ __global__ void __launch_bounds__(kVThreads, 4) k_vgemm_df(
         blk = make_int4(0, (int)b0, (int)(row_hi - b0 < R ? row_hi - b0 : R), 0);
     }
     const float2* __restrict__ Mr = Mall + (size_t)blk.x * mfloats;
-    const float* __restrict__ nr = norm + (size_t)blk.x * RL;
+    const float* __restrict__ nr = norm + (size_t)blk.x * (lmax + 1) * nbins * nbins;
     const int64_t r0 = blk.y;
     const int nrow = blk.z;
-    if (threadIdx.x <= lmax) amax[threadIdx.x] = 0;
-    __syncthreads();
     for (int c = threadIdx.x; c < RL; c += kVThreads) {
-        int m = 0;
-        while (m < lmax && c >= mi.col0[m + 1]) ++m;
-        float mx = 0.f;
 #pragma unroll
-        for (int rr = 0; rr < R; ++rr) {
-            const float v = rr < nrow ? __ldg(A + (r0 + rr) * RLP + c) : 0.f;
-            sA[c * RS + rr] = v;
-            mx = fmaxf(mx, fabsf(v));
-        }
-        atomicMax(&amax[m], __float_as_int(mx));
+        for (int rr = 0; rr < R; ++rr) sA[c * RS + rr] = rr < nrow ? __ldg(A + (r0 + rr) * RLP + c) : 0.f;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < nmb * R; k += kVThreads) {
+        // (a block's columns: the bin varies fastest)
+        const int rr = k % R, m = k / R / nbins, b = k / R - m * nbins, W = mi.W[m];
+        float mx = 0.f;
+        for (int c = b; c < W; c += nbins) mx = fmaxf(mx, fabsf(sA[(mi.col0[m] + c) * RS + rr]));
+        amax[k] = mx;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < nmb * R; k += kVThreads) {
+        const int rr = k % R, mb = k / R, m = mb / nbins;
+        float s = 0.f;
+        for (int b = 0; b < nbins; ++b) s = fmaf(__ldg(nr + mb * nbins + b), amax[(m * nbins + b) * R + rr], s);
+        bias[k] = 3.f * s;
     }
     __syncthreads();
     for (int col = threadIdx.x; col < RL; col += kVThreads) {
@@ -219,14 +240,16 @@ __global__ void __launch_bounds__(kVThreads, 4) k_vgemm_df(
         const int W = mi.W[m], c = col - mi.col0[m];
         const float2* Mc = Mr + mi.moff[m] + c;
         const float4* As = reinterpret_cast<const float4*>(sA + mi.col0[m] * RS);
-        const float bias = 3.f * __ldg(nr + col) * __int_as_float(amax[m]);
+        const float4* bs = reinterpret_cast<const float4*>(bias + (m * nbins + c % nbins) * R);
         float2 H[R / 2], Lo[R / 2];
 #pragma unroll
-        for (int r = 0; r < R / 2; ++r) {
-            H[r] = dup(bias);
-            Lo[r] = dup(0.f);
+        for (int r = 0; r < R / 4; ++r) {
+            const float4 b4 = bs[r];
+            H[2 * r] = make_float2(b4.x, b4.y);
+            H[2 * r + 1] = make_float2(b4.z, b4.w);
+            Lo[2 * r] = Lo[2 * r + 1] = dup(0.f);
         }
-#pragma unroll 4
+#pragma unroll 8
         for (int k = 0; k < W; ++k) {
             const float2 mv = __ldg(Mc + (int64_t)k * W);
             const float2 Mh = dup(mv.x), Ml = dup(mv.y);
@@ -247,7 +270,7 @@ __global__ void __launch_bounds__(kVThreads, 4) k_vgemm_df(
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const float hb = __fsub_rn(r & 1 ? H[r / 2].y : H[r / 2].x, bias);  // exact
+            const float hb = __fsub_rn(r & 1 ? H[r / 2].y : H[r / 2].x, reinterpret_cast<const float*>(bs)[r]);  // exact
             const float lb = r & 1 ? Lo[r / 2].y : Lo[r / 2].x;
             // renormalised
             const float h = __fadd_rn(hb, lb), bb = __fsub_rn(h, hb);
@@ -288,6 +311,8 @@ size_t adjoint_m_floats(int nbins, int lmax) {
     return s;
 }
 
+size_t adjoint_norm_floats(int nbins, int lmax) { return (size_t)(lmax + 1) * nbins * nbins; }
+
 int adjoint_rows_per_block() { return kRows; }
 
 int launch_adjoint_m(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float* Mr,
@@ -301,9 +326,9 @@ int launch_adjoint_m(const double* dzeta, int nbins, int lmax, int ncat, int64_t
 int launch_adjoint_m_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float2* Mr, float* norm,
                         cudaStream_t st) {
     const MInfo mi = make_info(nbins, lmax);
-    const int RL = nbins * (lmax + 1) * (lmax + 1);
-    dim3 grid((RL + kBWarps - 1) / kBWarps, ncat);
-    k_build_m_df<<<grid, kBWarps * 32, 0, st>>>(dzeta, mi, lmax, RL, zsize, adjoint_m_floats(nbins, lmax), Mr, norm);
+    dim3 grid((lmax + 1) * nbins, ncat);
+    k_build_m_df<<<grid, kBWarps * 32, 0, st>>>(dzeta, mi, nbins, zsize, adjoint_m_floats(nbins, lmax),
+                                                adjoint_norm_floats(nbins, lmax), Mr, norm);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -343,11 +368,11 @@ namespace {
 int vgemm_df(const float* A, int RLP, int RL, const int4* blks, int64_t nb, int64_t row_lo, int64_t row_hi,
              const float2* Mr, const float* norm, int nbins, int lmax, float2* V, cudaStream_t st) {
     const MInfo mi = make_info(nbins, lmax);
-    const size_t smem = sizeof(float) * (kRows + 4) * RL;
+    const size_t smem = sizeof(float) * ((kRows + 4) * (size_t)RL + 2 * (size_t)(lmax + 1) * nbins * kRows);
     if (cudaFuncSetAttribute(k_vgemm_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return -1;
     k_vgemm_df<<<(unsigned)nb, kVThreads, smem, st>>>(A, RLP, RL, blks, row_lo, row_hi, Mr, norm,
-                                                      adjoint_m_floats(nbins, lmax), mi, lmax, V);
+                                                      adjoint_m_floats(nbins, lmax), mi, nbins, lmax, V);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 }  // namespace

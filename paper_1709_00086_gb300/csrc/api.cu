@@ -1619,7 +1619,7 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
         const int64_t C = P->fixed_chunk;
         const bool precise = P->opt_grad == 0;
         if (precise ? (ensure(P, P->d_mrealdf, sizeof(float2) * adjoint_m_floats(P->nbins, P->lmax), "adjoint M") ||
-                       ensure(P, P->d_mnorm, sizeof(float) * P->RL, "adjoint M") ||
+                       ensure(P, P->d_mnorm, sizeof(float) * adjoint_norm_floats(P->nbins, P->lmax), "adjoint M") ||
                        ensure(P, P->d_Vdf, sizeof(float2) * (size_t)P->RLP * C, "adjoint V"))
                     : (ensure(P, P->d_mreal, sizeof(float) * adjoint_m_floats(P->nbins, P->lmax), "adjoint M") ||
                        ensure(P, P->d_V, sizeof(float) * (size_t)P->RLP * C, "adjoint V")))
@@ -1680,7 +1680,7 @@ int g3pcf_backward(g3pcf_plan_t P, const double* dzeta, double* dpos, double* dw
             for (int64_t r = r0; r < r1; r += RB) blks.push_back(int4{c, (int)r, (int)std::min<int64_t>(RB, r1 - r), 0});
         }
     if ((precise ? (ensure(P, P->d_mrealdf, sizeof(float2) * adjoint_m_floats(P->nbins, P->lmax) * ncat, "adjoint M") ||
-                    ensure(P, P->d_mnorm, sizeof(float) * (size_t)P->RL * ncat, "adjoint M") ||
+                    ensure(P, P->d_mnorm, sizeof(float) * adjoint_norm_floats(P->nbins, P->lmax) * ncat, "adjoint M") ||
                     ensure(P, P->d_Vdf, sizeof(float2) * (size_t)P->RLP * rows, "adjoint V"))
                  : (ensure(P, P->d_mreal, sizeof(float) * adjoint_m_floats(P->nbins, P->lmax) * ncat, "adjoint M") ||
                     ensure(P, P->d_V, sizeof(float) * (size_t)P->RLP * rows, "adjoint V"))) ||

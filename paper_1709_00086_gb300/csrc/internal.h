@@ -378,7 +378,9 @@ int launch_vgemm_rows(const float* A, int RLP, int RL, int64_t row_lo, int64_t r
                       int64_t q0, cudaStream_t st);
 // Double-float forms of the three (M and V as head + tail FP32 pairs, ~48 bits;
 // for the double-float adjoint pass)
-// norm: per catalog and A column the row sum of |M| (filled with M, ncat x RL)
+// norm: per catalog, order and two bins the largest row sum of |M| (filled with M;
+// adjoint_norm_floats per catalog)
+size_t adjoint_norm_floats(int nbins, int lmax);
 int launch_adjoint_m_df(const double* dzeta, int nbins, int lmax, int ncat, int64_t zsize, float2* Mr, float* norm,
                         cudaStream_t st);
 // V of the row blocks blks (adjoint_rows_per_block rows at most, one catalog each)
