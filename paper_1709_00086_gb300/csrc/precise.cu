@@ -585,6 +585,14 @@ __host__ __device__ constexpr size_t adj_df_smem_per_warp(int B, int N) {
 // the value of a biased sum as head (exact) and tail
 __device__ __forceinline__ float2 unbias(float2 H, float b) { return __fadd2_rn(H, dup(-b)); }
 
+// f2d_exact without a branch: subnormal inputs give zero (V has no tail there).
+__device__ __forceinline__ double f2d_sel(float x) {
+    const unsigned u = __float_as_uint(x), e = u & 0x7f800000u;
+    unsigned hi = ((u >> 3) & 0x0fffffffu) + ((1023u - 127u) << 20);
+    hi = e == 0x7f800000u ? hi | 0x7ff00000u : (e == 0u ? 0u : hi);
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), e == 0u ? 0 : (int)(u << 29));
+}
+
 template <int L>
 __global__ void __launch_bounds__(kDThreads, L <= 5 ? 5 : 4) k_adj_df(ListArgs a) {
     constexpr int NR = Shape<L>::NR;
@@ -651,15 +659,28 @@ __global__ void __launch_bounds__(kDThreads, L <= 5 ? 5 : 4) k_adj_df(ListArgs a
             // biases: three times the bound keeps every head above twice any term
             if (lane == 0) bias[b] = make_float2(3.f * s1, 3.f * s2);
         }
-        // the primary's own weight term of dL/dw: Re(A^H V)
+        // the primary's own weight term of dL/dw: Re(A^H V), the heads of V in FP64 and their
+        // tails (2^-25 of them, themselves good to half their bits) in FP32
         {
             const float* Arow = a.A + (int64_t)(a.chunked ? q - a.q0 : row) * a.RLP;
-            df wt = {0.f, 0.f};
-            for (int c = lane; c < a.RL; c += 32) {
-                const float2 v = Vrow[c];
-                df_acc(wt, df_mulf({v.x, v.y}, __ldg(Arow + c)));
+            double t = 0.0;
+            float tail = 0.f;
+            for (int c0 = lane; c0 < a.RL; c0 += 32 * 4) {
+                float2 v[4];
+                float x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {  // (loads of four columns in flight)
+                    const bool in = c0 + 32 * u < a.RL;
+                    v[u] = in ? Vrow[c0 + 32 * u] : make_float2(0.f, 0.f);
+                    x[u] = in ? __ldg(Arow + c0 + 32 * u) : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    t = fma(f2d_sel(x[u]), f2d_sel(v[u].x), t);
+                    tail = fmaf(v[u].y, x[u], tail);
+                }
             }
-            double t = df_to(wt);
+            t += (double)tail;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
             if (lane == 0) atomicAdd(a.dw + row, t);

@@ -10,6 +10,8 @@ tail gathers W residues of at most 2^-22 S_c (sqrt(W) 2^-24 as a random walk), a
 its 2 W roundings is 2^-24 of that: below 2^-38 S_c for W <= 220; the row's sum of A_c V_c
 adds nothing of that size.  2^-36 of sum |A_c| S_c.
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -74,3 +76,20 @@ def test_rows_and_bins_of_very_different_size(kind, nbins, lmax, chunk):
             big = np.tile((np.abs(v.real) + np.abs(v.imag)).reshape(-1, nbins).max(axis=0), lmax + 1 - m)
             tol += np.sum((np.abs(v.real) + np.abs(v.imag)) * ((np.abs(M.real) + np.abs(M.imag)) @ big))
         assert abs(dw[i] - ref) <= 2.0 ** -36 * tol, i
+
+
+def test_primary_weight_term_sums_in_fp64():
+    # M = 1: V = A exactly, and the term is sum |A|^2 with one rounding of 2^-53 per column and
+    # lane (38 of them) and per level of the reduction, as a random walk below 2^-51 of the sum
+    rng = np.random.default_rng(3)
+    cat = _catalog("bins", 10, 10, rng)
+    cat.w[:] = 1.0
+    pos, w = to_dev(cat, torch)
+    plan = g3.Plan(**cat.params())
+    plan.compute(pos, w, n_primary=64, keep_alm=True)
+    a = plan.alm(np.arange(64))
+    one = np.concatenate([0.5 * np.eye(cat.nbins * (cat.lmax + 1 - m)).ravel() for m in range(cat.lmax + 1)])
+    _, dw = plan.backward(torch.from_numpy(np.stack([2 * one, 0 * one], axis=1)).cuda())
+    for i, got in enumerate(dw.cpu().numpy()[:64]):
+        ref = math.fsum(np.concatenate([a[i].real.ravel() ** 2, a[i].imag.ravel() ** 2]))
+        assert abs(got - ref) <= 2.0 ** -51 * ref, i
