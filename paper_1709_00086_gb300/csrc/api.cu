@@ -1046,7 +1046,8 @@ int run_forward(g3pcf_plan_t P, CallSpec& c) {
         double budget = 0.0;
         const double per_row = 4.0 * P->RLP + 4.0;
         // (rows that fit what the plan already holds need no query)
-        const bool held = !ops && (double)P->A.bytes >= per_row * (double)rows_all;
+        const bool held = !ops && (double)P->A.bytes >= 4.0 * P->RLP * (double)rows_all &&
+                          (double)P->wrow.bytes >= 4.0 * (double)rows_all;
         if (ops || (c.ncat == 1 && P->opt_chunk <= 0 && !fixed && !held)) {
             size_t fr = 0, tot = 0;
             CK(cudaMemGetInfo(&fr, &tot));
