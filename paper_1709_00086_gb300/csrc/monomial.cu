@@ -27,7 +27,8 @@ constexpr unsigned kIdxMaskM = kIdxMask;
 __host__ __device__ constexpr int n_mono(int L) { return (L + 1) * (L + 2) * (L + 3) / 6; }
 
 // per-warp shared memory: powers [32][3][L+1] double, weights [32] double,
-// sums [NM] double, images [27] double3 (padded to 4), LOS rotation [12]
+// sums [NM] double, image shifts [27] double3 (padded to 4: the primary's
+// position), LOS rotation [12]
 // double, row res [RL] float
 __host__ __device__ constexpr size_t mono_smem_per_warp(int L, int RL) {
     return (size_t)32 * 3 * (L + 1) * 8 + 32 * 8 + (size_t)n_mono(L) * 8 + 27 * 32 + 12 * 8 + (size_t)RL * 4;
@@ -60,17 +61,17 @@ __global__ void __launch_bounds__(kMThreads) k_mono(ListArgs a) {
         if (q >= qb) break;
         const int p = a.plist ? a.plist[q] : q;
         const float4 P0 = a.pts[p];
-        if (lane < 27) {  // the primary's images in FP64
+        if (lane < 27) {  // the primary's position and the shifts of its images
             double x = P0.x, y = P0.y, z = P0.z;
             if (a.pts64) {
                 x = a.pts64[3 * (int64_t)p];
                 y = a.pts64[3 * (int64_t)p + 1];
                 z = a.pts64[3 * (int64_t)p + 2];
             }
-            const int sx = lane % 3 - 1, sy = (lane / 3) % 3 - 1, sz = lane / 9 - 1;
-            im[4 * lane] = x - sx * g.boxd;
-            im[4 * lane + 1] = y - sy * g.boxd;
-            im[4 * lane + 2] = z - sz * g.boxd;
+            im[4 * lane] = (lane % 3 - 1) * g.boxd;
+            im[4 * lane + 1] = ((lane / 3) % 3 - 1) * g.boxd;
+            im[4 * lane + 2] = (lane / 9 - 1) * g.boxd;
+            if (lane < 3) im[4 * lane + 3] = lane == 0 ? x : (lane == 1 ? y : z);
             if (lane < 9) Rm[lane] = g.radial ? los_rotation_entry_d(lane, x, y, z, g.boxd) : ((lane % 4 == 0) ? 1.0 : 0.0);
         }
         for (int k = lane; k < a.RL; k += 32) res[k] = 0.f;
@@ -117,7 +118,8 @@ __global__ void __launch_bounds__(kMThreads) k_mono(ListArgs a) {
                     qy = a.pts64[3 * j + 1];
                     qz = a.pts64[3 * j + 2];
                 }
-                double dx = qx - oi[0], dy = qy - oi[1], dz = qz - oi[2];
+                // (the difference first: an image rounds away what a close pair differs in)
+                double dx = (qx - im[3]) + oi[0], dy = (qy - im[7]) + oi[1], dz = (qz - im[11]) + oi[2];
                 if (g.radial) {  // into the primary's line-of-sight frame
                     const double rx = Rm[0] * dx + Rm[1] * dy + Rm[2] * dz;
                     const double ry = Rm[3] * dx + Rm[4] * dy + Rm[5] * dz;

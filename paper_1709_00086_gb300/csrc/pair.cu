@@ -18,7 +18,8 @@
 // evaluates Y_lm with an FP32 recurrence and accumulates into (lmax+1)^2
 // register partials; a 5-round butterfly then reduces the partials across
 // the 32 lanes into the warp's shared-memory a_lm(b).  The arithmetic is
-// FP32 on the FMA pipe; only the guard-band re-check of a bin edge is FP64.
+// FP32 on the FMA pipe; only the guard-band re-check of a bin edge and the
+// separation of pairs within a few FP32 ulps of one another are FP64.
 //
 // Harmonics.  Y_lm(rhat) = K_lm Dt_lm(z) (x + i y)^m with rhat = (x, y, z),
 // Dt_lm the monic polynomial of degree l-m proportional to the m-th
@@ -82,7 +83,8 @@ constexpr int kScanDepth = kStashDepth;
 template <int L>
 __device__ __forceinline__ void flush_bin(const float4* __restrict__ pts, const int* bucket_b,
                                           int cap, int navail, int kflush, int head, float* res_b,
-                                          const float4* img, const float* R, int radial, int lane) {
+                                          const float4* img, const float* R, int radial, int lane,
+                                          const PairArgs& a, int p, bool close) {
     constexpr int NR = Shape<L>::NR;
     float acc[NR];
     static_for<0, NR>([&](auto ic) { acc[decltype(ic)::value] = 0.f; });
@@ -118,6 +120,13 @@ __device__ __forceinline__ void flush_bin(const float4* __restrict__ pts, const 
             dy = q.y - o.y;
             dz = q.z - o.z;
             w = q.w;
+            if (close && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= close_r2(a.bins, a.pts64)) {
+                double s[4];
+                close_sep(pts, a.pts64, p, e, a.g.boxd, s);
+                dx = (float)s[0];
+                dy = (float)s[1];
+                dz = (float)s[2];
+            }
             if (radial) {
                 const float rx = fmaf(R[0], dx, fmaf(R[1], dy, R[2] * dz));
                 const float ry = fmaf(R[3], dx, fmaf(R[4], dy, R[5] * dz));
@@ -148,7 +157,8 @@ template <int L>
 __device__ __forceinline__ void flush_grad(const float4* __restrict__ pts, const int* __restrict__ orig,
                                            const int* bucket_b, int cap, int navail, int kflush,
                                            int head, const float* Hb, const float4* img, int lane,
-                                           double* dw, double* dpos, double (&dpi)[3]) {
+                                           double* dw, double* dpos, double (&dpi)[3], const PairArgs& a, int p,
+                                           bool close) {
     float pix = 0.f, piy = 0.f, piz = 0.f;
 #define G3_FETCH(t_, q_, e_)                              \
     do {                                                  \
@@ -174,10 +184,19 @@ __device__ __forceinline__ void flush_grad(const float4* __restrict__ pts, const
         G3_FETCH(t + 2, q1, e1);
         if (t * 32 + lane < navail) {
             const float4 o = img[e >> kIdxBits];
-            const float dx = q.x - o.x, dy = q.y - o.y, dz = q.z - o.z, wj = q.w;
+            float dx = q.x - o.x, dy = q.y - o.y, dz = q.z - o.z, sep = 1.f;
+            const float wj = q.w;
             const int jj = __ldg(orig + (e & kIdxMask));
+            if (close && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= close_r2(a.bins, a.pts64)) {
+                double s[4];
+                close_sep(pts, a.pts64, p, e, a.g.boxd, s);
+                dx = (float)s[0];
+                dy = (float)s[1];
+                dz = (float)s[2];
+                sep = (float)s[3];
+            }
             const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float rinv = rsqrtf(r2);
+            const float rinv = rsqrtf(r2);  // sep / r
             const float z = dz * rinv, ux = dx * rinv, uy = dy * rinv;
             float F, Fz, Fx = 0.f, Fy = 0.f;
             {  // m = 0 (real)
@@ -238,7 +257,7 @@ __device__ __forceinline__ void flush_grad(const float4* __restrict__ pts, const
                 ui = ni;
             });
             const float gdr = fmaf(Fx, ux, fmaf(Fy, uy, Fz * z));
-            const float sc = 2.f * wj * rinv;
+            const float sc = 2.f * wj * (sep * rinv);
             const float gx = sc * fmaf(-gdr, ux, Fx), gy = sc * fmaf(-gdr, uy, Fy),
                         gz = sc * fmaf(-gdr, z, Fz);
             atomicAdd(dw + jj, f2d_exact(2.f * F));
@@ -297,6 +316,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) k_pair(PairArgs a) {
     const bool exact_inputs = (a.pts64 == nullptr);
     const float hi_rej = a.bins.hi_rej, lo_rej = a.bins.lo_rej;
     const float rminf = a.bins.rmin, invw = a.bins.invw;
+    const int close_end = close_bins(a.bins, a.pts64);
 
     unsigned long long my_total = 0;  // lane b < B: pairs accepted into bin b
     long long cur_cat = -1;
@@ -529,10 +549,10 @@ __global__ void __launch_bounds__(kPairThreads, 2) k_pair(PairArgs a) {
             __syncwarp();
             if constexpr (MODE == 0)
                 flush_bin<L>(a.pts, bucket + fb * bstride, cap, fn, kk, head[fb], res + fb * NRP, img,
-                             Rs, g.radial, lane);
+                             Rs, g.radial, lane, a, p, fb < close_end);
             else
                 flush_grad<L>(a.pts, a.orig, bucket + fb * bstride, cap, fn, kk, head[fb],
-                              res + fb * NRP, img, lane, a.dw, a.dpos, dpi);
+                              res + fb * NRP, img, lane, a.dw, a.dpos, dpi, a, p, fb < close_end);
             __syncwarp();
 #pragma unroll
             for (int s = 0; s < kScanDepth; ++s) {

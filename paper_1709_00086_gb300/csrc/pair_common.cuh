@@ -232,6 +232,58 @@ __device__ __forceinline__ int exact_bin(const float4* __restrict__ pts, const d
 }
 
 
+// Close pairs.  FP32 positions leave nothing of a separation of a few of their ulps: no
+// direction at all (0 * rsqrt(0)) where two FP64 points round to one FP32 point.  Accepted
+// pairs up to close_r2 (every one of them has its bin from exact_bin) take their separation
+// from the input positions in FP64; FP32 input is exact without it, except where the
+// squared separation leaves FP32's range.
+__device__ __forceinline__ float close_r2(const Bins& b, const double* pts64) {
+    return pts64 ? b.guard[0] : fminf(b.guard[0], 0x1p-100f);
+}
+// The first bin without such pairs: a test per chunk of one bin instead of one per pair
+// (which cost the double-float kernels 2%).
+__device__ __forceinline__ int close_bins(const Bins& b, const double* pts64) {
+    int k = 0;
+    while (k < b.nbins && b.e2f[k] - b.guard[k] <= close_r2(b, pts64)) ++k;
+    return k;
+}
+// d[0..2]: separation of secondary j from image `code` of the point pd, times d[3], a power
+// of two that takes the largest component to [1, 2).
+__device__ __forceinline__ void close_sep_inline(const float4* __restrict__ pts, const double* pts64, const double* pd,
+                                                 int j, int code, double boxd, double* d) {
+    const float4 pj = pts[j];
+    const double xj[3] = {pts64 ? pts64[3 * (int64_t)j] : (double)pj.x, pts64 ? pts64[3 * (int64_t)j + 1] : (double)pj.y,
+                          pts64 ? pts64[3 * (int64_t)j + 2] : (double)pj.z};
+    const int want[3] = {code % 3 - 1, (code / 3) % 3 - 1, code / 9 - 1};
+    double s[3], most = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        s[k] = __dadd_rn(__dsub_rn(xj[k], pd[k]), want[k] * boxd);
+        most = fmax(most, fabs(s[k]));
+    }
+    // 2^-e of the largest component's exponent e (the squared separation is not 0 in FP64)
+    const double scale = __hiloint2double((int)(2046u - ((unsigned)__double2hiint(most) >> 20)) << 20, 0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) d[k] = s[k] * scale;
+    d[3] = scale;
+}
+__device__ __noinline__ void close_sep(const float4* __restrict__ pts, const double* pts64, const double* pd, int j,
+                                       int code, double boxd, double* d) {
+    close_sep_inline(pts, pts64, pd, j, code, boxd, d);
+}
+// the same from the list entry e of primary p
+template <bool INLINE = false>
+__device__ __forceinline__ void close_sep(const float4* __restrict__ pts, const double* pts64, int p, unsigned e,
+                                          double boxd, double* d) {
+    const float4 pi = pts[p];
+    const double pd[3] = {pts64 ? pts64[3 * (int64_t)p] : (double)pi.x, pts64 ? pts64[3 * (int64_t)p + 1] : (double)pi.y,
+                          pts64 ? pts64[3 * (int64_t)p + 2] : (double)pi.z};
+    if constexpr (INLINE)
+        close_sep_inline(pts, pts64, pd, (int)(e & kIdxMask), (int)(e >> kIdxBits), boxd, d);
+    else
+        close_sep(pts, pts64, pd, (int)(e & kIdxMask), (int)(e >> kIdxBits), boxd, d);
+}
+
 // Slot ranges of row r of the (2K+1)^2 rows of cells around a primary at P0
 // whose cell is (cy, cz): the x-range of cells that the sphere of radius
 // rmax (+ slack) can reach in that row, split by x image (-L, 0, +L) into at

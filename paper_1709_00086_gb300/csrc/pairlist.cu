@@ -196,7 +196,10 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-template <int MODE, bool STAGED>
+// F64: directions of close pairs from FP64 positions (FP32 ones need only a scale, and the
+// call behind the FP64 form costs the kernel 5%: 200,000 clustered points 16.9 against
+// 16.1 ms; inlined 17.4).
+template <int MODE, bool STAGED, bool F64>
 __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
     constexpr bool DIR = MODE != kEntries;
     constexpr int kTrip = STAGED ? kTripStaged : kTripDirect;
@@ -388,10 +391,23 @@ __global__ void __launch_bounds__(kScanThreads, kScanCtas) k_scan(ListArgs a) {
                         for (int u = 0; u < kTrip; ++u)
                             if (near[u]) {
                                 const float r2 = fmaf(d[u].x, d[u].x, fmaf(d[u].y, d[u].y, d[u].z * d[u].z));
-                                rinv[u] = rsqrtf(r2);
+                                float rr = r2;
                                 bn[u] = bin_slow(r2, a.bins.lo_rej, a.bins.hi_rej, a.bins.guard[0], s_dec,
                                                  a.bins.rmin, invw, B, exact_inputs, (int)code, a.pts, a.pts64,
                                                  j0 + u * kChunk, S.pd, g.boxd, g.periodic, s_e2);
+                                if (DIR && (unsigned)bn[u] < (unsigned)B && r2 <= close_r2(a.bins, a.pts64)) {
+                                    if constexpr (F64) {
+                                        double s[4];
+                                        close_sep(a.pts, a.pts64, S.pd, j0 + u * kChunk, (int)code, g.boxd, s);
+                                        d[u] = make_float4((float)s[0], (float)s[1], (float)s[2], d[u].w);
+                                    } else {  // exact already
+                                        d[u].x *= 0x1p100f;
+                                        d[u].y *= 0x1p100f;
+                                        d[u].z *= 0x1p100f;
+                                    }
+                                    rr = fmaf(d[u].x, d[u].x, fmaf(d[u].y, d[u].y, d[u].z * d[u].z));
+                                }
+                                rinv[u] = rsqrtf(rr);
                             }
                     }
                     if constexpr (!STAGED) {  // place the candidates' lanes as they are
@@ -623,8 +639,9 @@ __device__ __forceinline__ void set_image(float4* img, int code, const float4& P
 // Separation of one list entry from the primary (image img[code]), rotated
 // to the primary's line of sight in radial mode, as a unit vector and weight.
 template <bool EXACT>
-__device__ __forceinline__ void pair_dir(const float4& q, unsigned e, const float4* img, const float* R,
-                                         int radial, float& z, float& ux, float& uy, float& w) {
+__device__ __forceinline__ void pair_dir(const ListArgs& a, int p, bool close, const float4& q, unsigned e,
+                                         const float4* img, const float* R, int radial, float& z, float& ux,
+                                         float& uy, float& w) {
     float dx = 1.f, dy = 0.f, dz = 0.f;
     w = 0.f;
     if (e != kNoPair) {
@@ -637,6 +654,13 @@ __device__ __forceinline__ void pair_dir(const float4& q, unsigned e, const floa
             dx -= ol.x;
             dy -= ol.y;
             dz -= ol.z;
+        }
+        if (close && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= close_r2(a.bins, a.pts64)) {
+            double s[4];
+            close_sep(a.pts, a.pts64, p, e, a.g.boxd, s);
+            dx = (float)s[0];
+            dy = (float)s[1];
+            dz = (float)s[2];
         }
         w = q.w;
         if (radial) {
@@ -764,6 +788,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
     unsigned* ering = reinterpret_cast<unsigned*>(base + kImgBytes + 64 + kPtRing * 32 * 16);
     float* res = reinterpret_cast<float*>(base + kImgBytes + 64 + kPtRing * 32 * 16 + kEntRing * 32 * 4);
     const Grid& g = a.g;
+    const int close_end = close_bins(a.bins, a.pts64);
     const int qa = a.qrange ? a.qrange[0] : a.qa, qb = a.qrange ? a.qrange[1] : a.qb;
     for (;;) {
         int q = 0;
@@ -841,7 +866,7 @@ __global__ void __launch_bounds__(kLThreads, 3) k_accum(ListArgs a) {
                     const unsigned e = ering[(i & (kEntRing - 1)) * 32 + lane];
                     const float4 qv = pring[(i & (kPtRing - 1)) * 32 + lane];
                     float z, ux, uy, w;
-                    pair_dir<EXACT>(qv, e, img, Rs, g.radial, z, ux, uy, w);
+                    pair_dir<EXACT>(a, p, bA < close_end, qv, e, img, Rs, g.radial, z, ux, uy, w);
                     accum_pair_cheb<L>(acc0, accc, z, ux, uy, w);
                 }
                 sA = sB;
@@ -970,6 +995,7 @@ __global__ void __launch_bounds__(kLThreads) k_adj(ListArgs a) {
     unsigned* ering = reinterpret_cast<unsigned*>(base + kImgBytes + 64 + kPtRing * 32 * 16);
     float* G = reinterpret_cast<float*>(base + kImgBytes + 64 + kPtRing * 32 * 16 + kEntRing * 32 * 4);
     const Grid& g = a.g;
+    const int close_end = close_bins(a.bins, a.pts64);
     const int qa = a.qrange ? a.qrange[0] : a.qa, qb = a.qrange ? a.qrange[1] : a.qb;
     for (;;) {
         int q = 0;
@@ -1039,8 +1065,16 @@ __global__ void __launch_bounds__(kLThreads) k_adj(ListArgs a) {
                     const float4 qv = pring[(i & (kPtRing - 1)) * 32 + lane];
                     const float4 o = img[e >> kIdxBits], ol = img[27 + (e >> kIdxBits)];
                     const int jj = __ldg(a.orig + (e & kIdxMask));
-                    const float dx = (qv.x - o.x) - ol.x, dy = (qv.y - o.y) - ol.y, dz = (qv.z - o.z) - ol.z;
-                    const float rinv = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+                    float dx = (qv.x - o.x) - ol.x, dy = (qv.y - o.y) - ol.y, dz = (qv.z - o.z) - ol.z, sep = 1.f;
+                    if (bA < close_end && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= close_r2(a.bins, a.pts64)) {
+                        double s[4];
+                        close_sep(a.pts, a.pts64, p, e, g.boxd, s);
+                        dx = (float)s[0];
+                        dy = (float)s[1];
+                        dz = (float)s[2];
+                        sep = (float)s[3];
+                    }
+                    const float rinv = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));  // sep / r
                     const float z = dz * rinv, ux = dx * rinv, uy = dy * rinv;
                     const float* Gb = G + bA * NRP;
                     // T_k(z) and T_k'(z) = k U_{k-1}(z)
@@ -1088,7 +1122,7 @@ __global__ void __launch_bounds__(kLThreads) k_adj(ListArgs a) {
                         pim = ui;
                     });
                     const float gdr = fmaf(Fx, ux, fmaf(Fy, uy, Fz * z));
-                    const float sc = 2.f * qv.w * rinv;
+                    const float sc = 2.f * qv.w * (sep * rinv);
                     const float gx = sc * fmaf(-gdr, ux, Fx), gy = sc * fmaf(-gdr, uy, Fy),
                                 gz3 = sc * fmaf(-gdr, z, Fz);
                     atomicAdd(a.dw + jj, f2d_exact(2.f * F));
@@ -1183,10 +1217,10 @@ int launch_accum_t(const ListArgs& a, int nsm, cudaStream_t st) {
     return a.exact_img ? launch_accum_e<L, true>(a, nsm, st) : launch_accum_e<L, false>(a, nsm, st);
 }
 
-template <int MODE, bool STAGED>
+template <int MODE, bool STAGED, bool F64>
 int launch_scan_s(const ListArgs& a, int nsm, cudaStream_t st) {
     const size_t smem = sizeof(ScanSmem<MODE != kEntries, STAGED>) * kScanWarps;
-    auto* k = k_scan<MODE, STAGED>;
+    auto* k = k_scan<MODE, STAGED, F64>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kScanThreads, smem) != cudaSuccess || per_sm < 1)
@@ -1201,10 +1235,14 @@ int launch_scan_s(const ListArgs& a, int nsm, cudaStream_t st) {
 // are placed from the candidates' lanes; below, the accepted ones are gathered in
 // groups of 32 first.  200,000 clustered points, scan direct / staged: 34.1 / 32.1 ms
 // at 0.86 cells (27% pairs), 21.0 / 22.5 at 1.72 (47%), 16.8 / 19.7 at 3.74 (68%).
-template <int MODE>
+template <int MODE, bool F64>
 int launch_scan_k(const ListArgs& a, int nsm, cudaStream_t st) {
-    return a.bins.rmaxf * a.g.inv_cell < 1.5f ? launch_scan_s<MODE, true>(a, nsm, st)
-                                              : launch_scan_s<MODE, false>(a, nsm, st);
+    return a.bins.rmaxf * a.g.inv_cell < 1.5f ? launch_scan_s<MODE, true, F64>(a, nsm, st)
+                                              : launch_scan_s<MODE, false, F64>(a, nsm, st);
+}
+template <bool F64>
+int launch_scan_d(const ListArgs& a, int nsm, cudaStream_t st) {
+    return a.g.radial ? launch_scan_k<kDirsRadial, F64>(a, nsm, st) : launch_scan_k<kDirs, F64>(a, nsm, st);
 }
 
 }  // namespace
@@ -1223,8 +1261,8 @@ int launch_count(const ListArgs& a, int nsm, cudaStream_t st) {
 
 int launch_scan(const ListArgs& a, int nsm, cudaStream_t st) {
     if (!a.qrange && a.qb <= a.qa) return 0;
-    if (!a.dirs) return launch_scan_k<kEntries>(a, nsm, st);
-    return a.g.radial ? launch_scan_k<kDirsRadial>(a, nsm, st) : launch_scan_k<kDirs>(a, nsm, st);
+    if (!a.dirs) return launch_scan_k<kEntries, false>(a, nsm, st);
+    return a.pts64 ? launch_scan_d<true>(a, nsm, st) : launch_scan_d<false>(a, nsm, st);
 }
 
 size_t plan_scan_tmp_bytes(int64_t n) { return 8 * (size_t)((n + kScan64 - 1) / kScan64 + 1); }

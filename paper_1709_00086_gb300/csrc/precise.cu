@@ -196,6 +196,24 @@ __device__ __forceinline__ void load_sec(const ListArgs& a, unsigned e, float4& 
     }
 }
 
+// The separation of a close pair (close_r2) from the input positions, times the power of
+// two `scale`: head and tail leave out the last five bits of FP64 positions, which is all
+// of a separation of a few of their ulps.  INLINE: not by a call (k_accum_df, 80 registers
+// at lmax = 6: 24.9 ms against 25.2; k_adj_df: 36.5 against 36.4).
+template <bool INLINE>
+__device__ __forceinline__ void close_df(const ListArgs& a, int p, unsigned e, bool close, df& dx, df& dy, df& dz,
+                                         float& scale) {
+    scale = 1.f;
+    if (close && __fmaf_rn(dx.h, dx.h, __fmaf_rn(dy.h, dy.h, __fmul_rn(dz.h, dz.h))) <= close_r2(a.bins, a.pts64)) {
+        double s[4];
+        close_sep<INLINE>(a.pts, a.pts64, p, e, a.g.boxd, s);
+        dx = df_from(s[0]);
+        dy = df_from(s[1]);
+        dz = df_from(s[2]);
+        scale = (float)s[3];
+    }
+}
+
 // ---- forward ----------------------------------------------------------------
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
@@ -209,13 +227,6 @@ __device__ __forceinline__ void bias_fma(float2& H, float2& Lo, float2 Th, float
     const float2 s = __ffma2_rn(Th, Ch, H);
     const float2 e = __ffma2_rn(Th, Ch, __fadd2_rn(H, neg2(s)));
     Lo = __ffma2_rn(Th, Cl, __ffma2_rn(Tl, Ch, __fadd2_rn(Lo, e)));
-    H = s;
-}
-// the same with Cl = 0
-__device__ __forceinline__ void bias_fma(float2& H, float2& Lo, float2 Th, float2 Tl, float2 Ch) {
-    const float2 s = __ffma2_rn(Th, Ch, H);
-    const float2 e = __ffma2_rn(Th, Ch, __fadd2_rn(H, neg2(s)));
-    Lo = __ffma2_rn(Tl, Ch, __fadd2_rn(Lo, e));
     H = s;
 }
 // (H, Lo) += T c for a head without a bias (an error-free addition, 11 operations)
@@ -301,6 +312,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
     const int offC = m > 0 ? 4 * (m - 1) : 0, offT = R_::TB + 2 * k0;
     const Grid& g = a.g;
     const df boxdf = df_from(g.boxd);  // the box side as head + tail
+    const int close_end = close_bins(a.bins, a.pts64);
     const bool radial = g.radial != 0;
     const int qa = a.qrange ? a.qrange[0] : a.qa, qb = a.qrange ? a.qrange[1] : a.qb;
     for (;;) {
@@ -465,7 +477,10 @@ __global__ void __launch_bounds__(kDThreads, L <= 6 ? 6 : (L == 7 ? 5 : 4)) k_ac
                 const float4 hh = img[code], tt = img[27 + code];
                 df dx = sep(qv.x, ql.x, hh.x, tt.x), dy = sep(qv.y, ql.y, hh.y, tt.y),
                    dz = sep(qv.z, ql.z, hh.z, tt.z);
-                if (!v) {
+                float scale1;
+                if (v) {
+                    close_df<true>(a, p, e, (int)(o0 >> 26) < close_end, dx, dy, dz, scale1);
+                } else {
                     dx = {1.f, 0.f};
                     dy = dz = {0.f, 0.f};
                 }
@@ -606,6 +621,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 5 ? 5 : 4) k_adj_df(ListArgs a
     float2* bias = reinterpret_cast<float2*>(base + (size_t)B * G_::N * 4 + 54 * 16);  // [B]
     const Grid& g = a.g;
     const df boxdf = df_from(g.boxd);  // the box side as head + tail
+    const int close_end = close_bins(a.bins, a.pts64);
     const int qa = a.qrange ? a.qrange[0] : a.qa, qb = a.qrange ? a.qrange[1] : a.qb;
     for (;;) {
         int q = 0;
@@ -717,9 +733,11 @@ __global__ void __launch_bounds__(kDThreads, L <= 5 ? 5 : 4) k_adj_df(ListArgs a
                 const int jj = __ldg(a.orig + (e & kIdxMask));
                 const int code = (int)(e >> kIdxBits);
                 const float4 hh = img[code], tt = img[27 + code];
-                const df dx = sep(qv.x, ql.x, hh.x, tt.x), dy = sep(qv.y, ql.y, hh.y, tt.y),
-                         dz = sep(qv.z, ql.z, hh.z, tt.z);
-                df ux, uy, z, rinv;
+                df dx = sep(qv.x, ql.x, hh.x, tt.x), dy = sep(qv.y, ql.y, hh.y, tt.y),
+                   dz = sep(qv.z, ql.z, hh.z, tt.z);
+                float scale;
+                close_df<false>(a, p, e, b < close_end, dx, dy, dz, scale);
+                df ux, uy, z, rinv;  // (rinv: 1 / (scale r))
                 unit_df(dx, dy, dz, nullptr, false, ux, uy, z, rinv);
                 // T_k(z) and T_k'(z) = k U_{k-1}(z), heads and tails
                 df T[L + 1], D[L + 1];
@@ -811,7 +829,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 5 ? 5 : 4) k_adj_df(ListArgs a
                 const float tx = df_add(Fx, df_neg(df_mul(gdr, ux))).h;
                 const float ty = df_add(Fy, df_neg(df_mul(gdr, uy))).h;
                 const float tz = df_add(Fz, df_neg(df_mul(gdr, z))).h;
-                const float sc = __fmul_rn(2.f * qv.w, __fadd_rn(rinv.h, rinv.l));
+                const float sc = __fmul_rn(2.f * qv.w, scale * __fadd_rn(rinv.h, rinv.l));
                 const float gx = __fmul_rn(sc, tx), gy = __fmul_rn(sc, ty), gz3 = __fmul_rn(sc, tz);
                 atomicAdd(a.dw + jj, f2d_exact(__fmul_rn(2.f, __fadd_rn(F.h, F.l))));
                 atomicAdd(a.dpos + 3 * (int64_t)jj, f2d_exact(gx));
