@@ -93,3 +93,44 @@ def test_primary_weight_term_sums_in_fp64():
     for i, got in enumerate(dw.cpu().numpy()[:64]):
         ref = math.fsum(np.concatenate([a[i].real.ravel() ** 2, a[i].imag.ravel() ** 2]))
         assert abs(got - ref) <= 2.0 ** -51 * ref, i
+
+
+@pytest.mark.parametrize("lmax", [4, 10])
+@pytest.mark.parametrize("kind", ["weights", "inner bin", "light"])
+def test_gradients_point_by_point(kind, lmax):
+    # weights over twelve decades; a dense clump beside isolated points with dL/dzeta on the
+    # innermost bin alone; light points whose rows share blocks with those of a heavy clump.
+    # Every point against its own size: the rows of A are FP32 (2^-25 of an entry, amplified by
+    # up to 2^7 to a pair's gradient), pairs are rounded to FP32, and one component in a few
+    # hundred may cancel tenfold: 1e-4 of the point's own, and 1e-6 of the median's
+    n, nbins = 300, 5
+    rng = np.random.default_rng(lmax)
+    pos = rng.uniform(60.0, 140.0, (n, 3))
+    w = rng.uniform(0.5, 1.5, n)
+    bins, pick = np.arange(nbins), np.ones(n, bool)
+    if kind == "weights":
+        w *= 10.0 ** rng.uniform(-6.0, 6.0, n)
+    elif kind == "inner bin":
+        pos[:200] = 100.0 + 1.5 * rng.normal(size=(200, 3))
+        bins = np.arange(1)
+    else:
+        pick = np.arange(n) % 2 == 0
+        pos = np.where(pick[:, None], 60.0, 200.0) + rng.uniform(-9.0, 9.0, (n, 3))
+        w *= np.where(pick, 1e-6, 1e6)
+    cat = catalogs.Catalog(pos.astype(np.float32), w.astype(np.float32), 300.0, nbins, 0.0, 30.0, lmax, 1)
+    G = []
+    for m in range(lmax + 1):
+        K = nbins * (lmax + 1 - m)
+        keep = np.isin(np.arange(K) % nbins, bins)
+        b = rng.normal(size=(K, K)) + 1j * rng.normal(size=(K, K))
+        G.append(((b + b.conj().T) * np.outer(keep, keep)).ravel())
+    G = np.concatenate(G)
+    p, wt = to_dev(cat, torch)
+    plan = g3.Plan(**cat.params())
+    plan.compute(p, wt, keep_alm=True)
+    dpos, dw = plan.backward(torch.from_numpy(np.stack([2 * G.real, 2 * G.imag], axis=1)).cuda())
+    rpos, rw = oracle.grad(cat.pos.astype(np.float64), cat.w.astype(np.float64), G, cat.box, nbins, 0.0, 30.0, lmax,
+                           los_mode=1)
+    for got, ref in ((dpos.cpu().numpy(), rpos), (dw.cpu().numpy()[:, None], rw[:, None])):
+        size = np.abs(ref[pick]).max(axis=1)
+        assert (np.abs(got - ref)[pick].max(axis=1) <= 1e-4 * size + 1e-6 * np.median(size)).all()
