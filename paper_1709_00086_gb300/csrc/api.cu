@@ -1360,7 +1360,9 @@ int forward_entry(g3pcf_plan_t P, CallSpec& c) {
                                   (long long)c.n, (long long)c.n_primary, (long long)c.ncat,
                                   (long long)c.pos_f64,
                                   (long long)(c.flags & ~(G3PCF_F_NO_SYNC | G3PCF_F_GRAPH)),
-                                  (long long)P->opt_chunk, (long long)P->opt_cells, (long long)P->kflush};
+                                  (long long)P->opt_chunk, (long long)P->opt_cells, (long long)P->kflush,
+                                  (long long)P->opt_xref, (long long)P->opt_pair, (long long)P->opt_basis,
+                                  (long long)P->opt_grad, (long long)P->opt_list_bytes};
     key.insert(key.end(), c.offs.begin(), c.offs.end());
     if (!P->gstream) {
         CK(cudaStreamCreateWithFlags(&P->gstream, cudaStreamNonBlocking));

@@ -40,3 +40,21 @@ def test_graph_after_a_plain_forward(keep_alm, options):
         out.append((zr.cpu().numpy(), cr.cpu().numpy(), plan.alm(np.arange(0, cat.w.size, 37))))
     for ref, got in zip(*out):
         np.testing.assert_array_equal(got, ref)
+
+
+@pytest.mark.parametrize("keep_alm,opt", [(False, g3.OPT_BASIS), (True, g3.OPT_GRAD_PRECISION)])
+def test_graph_follows_a_changed_option(keep_alm, opt):
+    # the same call after the option has changed is a new capture, not a replay of the old one
+    cat = catalogs.small_case("clustered", 2000, seed=4, box=300.0, nbins=5, rmin=0.0, rmax=60.0, lmax=5)
+    pos, w = to_dev(cat, torch)
+    prims = np.arange(0, cat.w.size, 37)
+    ref = g3.Plan(**cat.params())
+    ref.set_option(opt, 1)
+    ref.compute(pos, w, keep_alm=keep_alm)
+    plan = g3.Plan(**cat.params())
+    zr = torch.empty((plan.zsize, 2), dtype=torch.float64, device="cuda")
+    cr = torch.empty(cat.nbins, dtype=torch.int64, device="cuda")
+    for value in (0, 0, 1, 1):
+        plan.set_option(opt, value)
+        plan.compute(pos, w, keep_alm=keep_alm, graph=True, out=zr, counts_out=cr)
+    np.testing.assert_array_equal(plan.alm(prims), ref.alm(prims))
