@@ -294,15 +294,20 @@ int g3pcf_fp32_peak(double* tflops, void* stream);
  *   G3PCF_OPT_PAIR_KERNELS    forward pair stage: 1 = the fused kernel (bucket and
  *                             accumulate in one pass), 0 or 2 = pair lists (count,
  *                             scan into per-bin lists of 32 pairs, accumulate; one
- *                             host synchronisation per chunk of primaries; inside a
- *                             captured graph (G3PCF_F_GRAPH) the list passes are
- *                             planned on the device instead)
+ *                             host synchronisation per chunk of primaries; a captured
+ *                             graph (G3PCF_F_GRAPH) has none: one list pass that takes
+ *                             its chunks from a device counter where the pool of the
+ *                             first call holds the lists, else passes planned on the
+ *                             device)
  *   G3PCF_OPT_LIST_BYTES      device bytes for the pair lists (0: up to 40% of free
  *                             memory, at most 32 GB); more pairs than fit are
- *                             processed in several passes.  A plain forward's lists
- *                             take 16 bytes per pair, or 4 where the budget would
- *                             otherwise leave too few primaries per pass; the other
- *                             calls' take 4
+ *                             processed in several passes.  The pool is reserved in
+ *                             chunks of 32 per candidate, not per pair: for every
+ *                             primary its candidates / 32 rounded up, plus nbins (a
+ *                             third to two thirds of the candidates are pairs).  A plain
+ *                             forward's chunk takes 520 bytes, or 136 where the budget
+ *                             would otherwise leave too few primaries per pass; the
+ *                             other calls' take 136
  *   G3PCF_OPT_GRAD_PRECISION  arithmetic of the pair stage for multipoles that are
  *                             differentiated (forwards with G3PCF_F_KEEP_ALM, the
  *                             backward and its recomputation): 0 = double-float

@@ -20,9 +20,10 @@ namespace {
 // CTA; a lane holds 8 x 4 entries of the tile.  Bound by issue: per primary and
 // warp 16 packed FMAs (two issue cycles each) and about 20 other instructions.
 // 32-wide tiles leave 1.5 entries computed per entry of the triangle (64-wide
-// ones 2.1 at B = lmax = 10).  Runs of kFlushRows primaries are summed in FP32, the
-// runs in double-float (head + tail, 2^-48): FP64 additions, at 1/58 of the FP32
-// rate, would take a third of the kernel's time.  20,000 primaries, B = lmax = 10:
+// ones 2.1 at B = lmax = 10).  Runs of kFlushRows primaries are summed in FP32 (2^-24 per
+// addition, which sets the error), the runs in double-float (head + tail, 2^-48 per
+// addition; the warps' sums and the partials' reduction in FP64): FP64 additions, at 1/58
+// of the FP32 rate, would take a third of the kernel's time.  20,000 primaries, B = lmax = 10:
 // 0.20 ms (10 row parts, 1,220 CTAs) against 1.29 ms for 64-wide tiles with 4 x 4 scalar
 // FMAs per thread, whose 129 CTAs left most SMs one block of 8,192 rows.
 constexpr int kT = 32;           // tile edge

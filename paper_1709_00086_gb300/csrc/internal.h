@@ -376,8 +376,8 @@ int launch_adjoint_m(const double* dzeta, int nbins, int lmax, int ncat, int64_t
 int launch_vgemm_rows(const float* A, int RLP, int RL, int64_t row_lo, int64_t row_hi, const float* Mr,
                       int nbins, int lmax, float* V, double* dw, const int* plist, const int* orig,
                       int64_t q0, cudaStream_t st);
-// Double-float forms of the three (M and V as head + tail FP32 pairs, ~48 bits;
-// for the double-float adjoint pass)
+// Double-float forms of the three (M and V as head + tail FP32 pairs; M to 2^-48, V to
+// about 2^-44 of the bound of its sums, see k_vgemm_df; for the double-float adjoint pass)
 // norm: per catalog, order and two bins the largest row sum of |M| (filled with M;
 // adjoint_norm_floats per catalog)
 size_t adjoint_norm_floats(int nbins, int lmax);

@@ -400,38 +400,6 @@ __device__ __forceinline__ int cell_of(float x, const Grid& g) {
     return c < 0 ? 0 : (c >= g.nc ? g.nc - 1 : c);
 }
 
-// The bin of a candidate at squared FP32 distance r2 (-1: not a pair), using the
-// r^2 table, the guard-widened FP32 edges and, inside a guard band, the exact
-// FP64 rule.  tab/dec/e2 are shared-memory copies.
-__device__ __forceinline__ int decide_bin(float r2, float hi_rej, float lo_rej, float tscale,
-                                          const unsigned char* tab, float guard0,
-                                          const float2* dec, float rminf, float invw, int B,
-                                          bool exact_inputs, int code, const float4* __restrict__ pts,
-                                          const double* pts64, int j, const double* pd, double boxd,
-                                          int periodic, const double* e2) {
-    if (!(r2 < hi_rej)) return -1;
-    int ti = (int)(r2 * tscale);
-    ti = ti > kBinTable + 1 ? kBinTable + 1 : ti;
-    const int tv = tab[ti];
-    if (tv < kTabReject) return tv;
-    if (tv == kTabReject) return -1;
-    if (r2 < lo_rej) return -1;
-    int bin;
-    if (!(r2 > guard0)) {
-        bin = (exact_inputs && code == 13 && r2 == 0.f) ? -1 : -2;
-    } else {
-        const float rr = r2 * rsqrtf(r2);
-        int bb = (int)((rr - rminf) * invw);
-        bb = bb < 0 ? 0 : (bb >= B ? B - 1 : bb);
-        const float2 iv = dec[bb];
-        bin = (r2 > iv.x && r2 < iv.y) ? bb : -2;
-    }
-    if (bin == -2)
-        bin = exact_bin(pts, pts64, j, pd[0], pd[1], pd[2], code % 3 - 1, (code / 3) % 3 - 1,
-                        code / 9 - 1, boxd, periodic, e2, B);
-    return bin;
-}
-
 // The bin of a candidate that k_scan's rounding leaves open (see Bins::bin_lim):
 // guard-widened FP32 edges, then the exact FP64 rule.
 __device__ __noinline__ int bin_slow(float r2, float lo_rej, float hi_rej, float guard0, const float2* dec,

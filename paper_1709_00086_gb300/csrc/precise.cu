@@ -1,7 +1,8 @@
 // Pair-stage kernels for multipoles that are differentiated: the forward
 // multipoles a_lm of Sec. 3.1 and the adjoint pair pass, both in double-float
-// arithmetic (an FP32 head plus an FP32 tail, about 44 significant bits) over
-// the same per-bin pair lists as the FP32 kernels of pairlist.cu.
+// arithmetic (an FP32 head plus an FP32 tail: about 44 significant bits per operation; the
+// biased sums below are good to 2^-38 - 2^-45 of their largest terms) over the same
+// per-bin pair lists as the FP32 kernels of pairlist.cu.
 //
 // Why: in the Chebyshev form Y_lm = K_lm sum_k c_k T_k(z) (x + iy)^m the
 // connection coefficients c_k are non-negative and large where D_lm(1) is much
@@ -25,13 +26,13 @@
 //                 (bias_fma).  At the end of a bin the Chebyshev ->
 //                 Legendre-form connection (times K_lm, head + tail
 //                 coefficients) is applied in double-float; the row of A is
-//                 stored at the primary's end.  No FP64 arithmetic: the FP64
-//                 pipe runs at 1/58 of the FP32 rate.  Bound by issue, with
-//                 shared memory (records in and out) close behind: 1,250 cycles
-//                 per chunk and SM quarter at lmax = 6.  100,000 clustered
-//                 points, lmax = 6 (7.1e8 pairs): 23.5 ms, against 40 ms with
+//                 stored at the primary's end.  No FP64 arithmetic (but for the rare
+//                 close pair): the FP64 pipe runs at 1/58 of the FP32 rate.  Bound by
+//                 issue, with shared memory (records in and out) close behind.  100,000
+//                 clustered points, lmax = 6 (7.1e8 pairs): 24.9 ms, against 40 ms with
 //                 12 instead of 6 operations per term and one sum pair per lane
-//                 (twice the shared-memory bytes per term).  Sums in the
+//                 (twice the shared-memory bytes per term); 23.5 ms with a fixed bias,
+//                 biased m = 0 sums and inexact chunk sums.  Sums in the
 //                 registers of the pair's lane alone (no records, a
 //                 reduction of every sum per bin) took 23 ms there, but three
 //                 times this kernel's time at 55 pairs per bin and lmax = 10.
@@ -44,17 +45,19 @@
 //                 double-float: per m the sums against T_k and T_k' on (Re, Im)
 //                 pairs with biased heads, then their products with
 //                 (x + iy)^(m-1), whose partial sums as m descends are the x
-//                 and y derivatives.  Rounded once to FP32 per pair; FP64
+//                 and y derivatives.  Their tails gather residues of half an ulp of
+//                 a head near three times the bin's coefficient norm: a few 2^-44 of the
+//                 norm, where the coefficients themselves carry 2^-25 of theirs from the
+//                 FP32 rows of A.  Rounded once to FP32 per pair; FP64
 //                 atomics for the secondary, a double-float sum for the
-//                 primary.  Bound by issue: about 1,450 cycles of arithmetic
-//                 per chunk and SM quarter at lmax = 6, of 1,880.  100,000
-//                 clustered points, lmax = 6: 36 ms against 57 with error-free
-//                 additions and an FP32 pair per derivative.  Resident CTAs (registers):
-//                 at lmax = 10 four take 2.08 ms on 1.1e7 pairs, three 2.14, two,
-//                 without any limit on the registers, 2.44; at lmax = 4 five
-//                 take 0.83 and four 0.86; at lmax = 6 three and five are 3% slower
-//                 than four.  k_accum_df likewise: at lmax = 6 six CTAs 23.5 ms, five
-//                 24.2, four 25.0; at lmax = 8 four are the best.
+//                 primary; its weight term in FP64.  Bound by issue.  100,000
+//                 clustered points, lmax = 6: 36.4 ms against 57 with error-free
+//                 additions and an FP32 pair per derivative.
+// Resident CTAs (registers), 20,000 uniform points, ms at 3 / 4 / 5 / 6 CTAs per SM:
+// k_accum_df 0.77 / 0.71 / 0.69 / 0.65 at lmax = 6 and six the best below, 0.80 / 0.74 /
+// 0.73 / 0.72 at 7, 1.08 / 0.99 / 1.00 / 0.99 at 8, 1.20 / 1.16 / 1.19 / 1.23 at 10; k_adj_df
+// 0.67 / 0.67 / 0.64 / 0.65 at lmax = 4, 0.89 / 0.82 / 0.77 / 0.80 at 5, 1.04 / 0.96 / 0.98 /
+// 1.00 at 6, 1.46 / 1.43 / 1.53 / 1.57 at 8, 2.14 / 2.13 / 2.14 / 2.23 at 10.
 #include "pair_common.cuh"
 
 namespace g3 {
