@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count(ListArgs a, int lpp) {
 // the candidates near an edge take the exact rule.  32 warps per SM at 64
 // registers: 40 and 48 are 6% and 24% slower.  Staged, two or three loads per trip
 // instead of four are 10% and 3% slower; direct (no stage), three and two are the same,
-// four spill (3%).  200,000 clustered points (L = 696, 4.0e9 pairs): 16.0 ms writing
+// four spill (3%).  200,000 clustered points (L = 696, 4.0e9 pairs): 16.1 ms writing
 // 16 bytes per pair (staged 19.7, which is what the form took that wrote 4 bytes
 // and left the direction to the accumulate kernel).
 //
