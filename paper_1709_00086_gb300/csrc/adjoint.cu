@@ -192,7 +192,7 @@ __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 // |A| there (bins that dL/dzeta leaves out count nothing).  Bound by issue; M (from L2) is read once per 8 rows,
 // coalesced by its symmetry (16 rows per CTA: the same time).  20,000 rows at B =
 // lmax = 10: 0.68 ms against 1.73 with error-free additions (0.65 with one bias per CTA
-// and order); 85 registers and three CTAs per SM, as 64 and four take 0.82.
+// and order); 80 registers and three CTAs per SM, as 64 and four take 0.82.
 // The primary-weight term Re(A^H V) is the pair pass's (k_adj_df).
 __global__ void __launch_bounds__(kVThreads, 3) k_vgemm_df(
     const float* __restrict__ A, int RLP, int RL, const int4* __restrict__ blks, int64_t row_lo, int64_t row_hi,

@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(kDThreads, L <= 5 ? 5 : 4) k_adj_df(ListArgs a
             if (lane == 0) bias[b] = make_float2(3.f * s1, 3.f * s2);
         }
         // the primary's own weight term of dL/dw: Re(A^H V), the heads of V in FP64 and their
-        // tails (2^-25 of them, themselves good to half their bits) in FP32
+        // tails (at most 2^-24 of them, and known to about 2^-20 of themselves) in FP32
         {
             const float* Arow = a.A + (int64_t)(a.chunked ? q - a.q0 : row) * a.RLP;
             double t = 0.0;
